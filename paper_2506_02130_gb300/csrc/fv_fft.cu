@@ -20,175 +20,11 @@
 // complex of padding per 16, which breaks the bank conflicts of the
 // stride-R stores of the first stage); index arithmetic uses
 // multiply-high division by the per-stage constants prepared on the host.
-#include "fv_internal.cuh"
+#include "fv_dft.cuh"
 
 namespace fv {
 
 static constexpr int kThreads = 256;
-
-// ---------------------------------------------------------------- compile-time twiddles
-// e^{2 pi i m / R} for 2 <= R <= 16, from Taylor series on [0, pi/4] after an
-// exact reduction of the rational angle m/R to an octant (constexpr, host compiler).
-namespace cx {
-constexpr double kPi = 3.14159265358979323846264338327950288;
-constexpr double sin_t(double a)
-{
-    double t = a, s = a;
-    for (int n = 1; n < 12; ++n) {
-        t *= -a * a / ((2.0 * n) * (2.0 * n + 1.0));
-        s += t;
-    }
-    return s;
-}
-constexpr double cos_t(double a)
-{
-    double t = 1.0, s = 1.0;
-    for (int n = 1; n < 12; ++n) {
-        t *= -a * a / ((2.0 * n - 1.0) * (2.0 * n));
-        s += t;
-    }
-    return s;
-}
-struct SC { double s, c; };
-constexpr SC sincos2pi(int m, int R)
-{
-    m %= R;
-    if (m < 0) m += R;
-    const long t = 4L * m;
-    const int k = (int)(t / R);            // quarter turns
-    const long rem = t - (long)k * R;      // remaining angle (pi/2) rem / R
-    double s0 = 0, c0 = 0;
-    if (2 * rem <= R) {
-        const double a = (kPi / 2) * (double)rem / R;
-        s0 = sin_t(a);
-        c0 = cos_t(a);
-    } else {
-        const double a = (kPi / 2) * (double)(R - rem) / R;
-        s0 = cos_t(a);
-        c0 = sin_t(a);
-    }
-    if (k == 0) return {s0, c0};
-    if (k == 1) return {c0, -s0};
-    if (k == 2) return {-s0, -c0};
-    return {-c0, s0};
-}
-}  // namespace cx
-
-// v * e^{2 pi i m / R} with compile-time m, R: exact for the quarter turns, otherwise a product by
-// constants folded at compile time (no table load, no FP64 conversion in the FP32 instances)
-template <class G, int M_, int R>
-__device__ __forceinline__ cpx<G> twm(cpx<G> v)
-{
-    constexpr int m = M_ % R;
-    if constexpr (m == 0) return v;
-    else if constexpr (4 * m == R) return cmuli(v);
-    else if constexpr (2 * m == R) return cmk<G>(-v.x, -v.y);
-    else if constexpr (4 * m == 3 * R) return cmk<G>(v.y, -v.x);
-    else {
-        constexpr cx::SC w = cx::sincos2pi(m, R);
-        return cmul(v, cmk<G>((G)w.c, (G)w.s));
-    }
-}
-
-// ---------------------------------------------------------------- register DFTs (+ sign)
-template <int R> struct Fac {
-    static constexpr int A = (R % 4 == 0 && R != 4) ? 4 : (R % 2 == 0 && R != 2) ? 2 : (R % 3 == 0 && R != 3) ? 3 : 5;
-    static constexpr int B = R / A;
-};
-
-template <class G, int R> struct Dft;
-
-template <class G> struct Dft<G, 2> {
-    static __device__ __forceinline__ void run(cpx<G> *v)
-    {
-        cpx<G> a = v[0], b = v[1];
-        v[0] = cadd(a, b);
-        v[1] = csub(a, b);
-    }
-};
-template <class G> struct Dft<G, 3> {
-    static __device__ __forceinline__ void run(cpx<G> *v)
-    {
-        const G h = (G)0.86602540378443864676;   // sin(2 pi / 3)
-        cpx<G> t = cadd(v[1], v[2]), u = cmuli(cscale(csub(v[1], v[2]), h));
-        cpx<G> m = csub(v[0], cscale(t, (G)0.5));
-        v[0] = cadd(v[0], t);
-        v[1] = cadd(m, u);
-        v[2] = csub(m, u);
-    }
-};
-template <class G> struct Dft<G, 4> {
-    static __device__ __forceinline__ void run(cpx<G> *v)
-    {
-        cpx<G> s02 = cadd(v[0], v[2]), d02 = csub(v[0], v[2]);
-        cpx<G> s13 = cadd(v[1], v[3]), d13 = cmuli(csub(v[1], v[3]));
-        v[0] = cadd(s02, s13);
-        v[2] = csub(s02, s13);
-        v[1] = cadd(d02, d13);
-        v[3] = csub(d02, d13);
-    }
-};
-template <class G> struct Dft<G, 5> {
-    static __device__ __forceinline__ void run(cpx<G> *v)
-    {
-        const G c1 = (G)0.30901699437494742410, c2 = (G)-0.80901699437494742410;   // cos(2pi/5), cos(4pi/5)
-        const G s1 = (G)0.95105651629515357212, s2 = (G)0.58778525229247312917;    // sin(2pi/5), sin(4pi/5)
-        cpx<G> t1 = cadd(v[1], v[4]), t2 = cadd(v[2], v[3]);
-        cpx<G> u1 = csub(v[1], v[4]), u2 = csub(v[2], v[3]);
-        cpx<G> a1 = cadd(v[0], cadd(cscale(t1, c1), cscale(t2, c2)));
-        cpx<G> a2 = cadd(v[0], cadd(cscale(t1, c2), cscale(t2, c1)));
-        cpx<G> b1 = cmuli(cadd(cscale(u1, s1), cscale(u2, s2)));
-        cpx<G> b2 = cmuli(csub(cscale(u1, s2), cscale(u2, s1)));
-        v[0] = cadd(v[0], cadd(t1, t2));
-        v[1] = cadd(a1, b1);
-        v[4] = csub(a1, b1);
-        v[2] = cadd(a2, b2);
-        v[3] = csub(a2, b2);
-    }
-};
-
-// Composite R = A B: with r = B r1 + r2 and q = q1 + A q2,
-// w_R^{rq} = w_A^{r1 q1} w_R^{r2 q1} w_B^{r2 q2}:
-// A-point DFTs over r1 for every r2, twiddles w_R^{r2 q1}, B-point DFTs over r2.
-template <class G, int R, int A, int R2, int Q1>
-__device__ __forceinline__ void col_twiddle(const cpx<G> *t, cpx<G> *u)
-{
-    if constexpr (Q1 < A) {
-        u[Q1] = twm<G, R2 * Q1, R>(t[Q1]);
-        col_twiddle<G, R, A, R2, Q1 + 1>(t, u);
-    }
-}
-
-template <class G, int R, int A, int B, int R2>
-__device__ __forceinline__ void col_pass(const cpx<G> *v, cpx<G> (*U)[A])
-{
-    if constexpr (R2 < B) {
-        cpx<G> t[A];
-#pragma unroll
-        for (int r1 = 0; r1 < A; ++r1) t[r1] = v[B * r1 + R2];
-        Dft<G, A>::run(t);
-        col_twiddle<G, R, A, R2, 0>(t, U[R2]);
-        col_pass<G, R, A, B, R2 + 1>(v, U);
-    }
-}
-
-template <class G, int R> struct Dft {
-    static __device__ __forceinline__ void run(cpx<G> *v)
-    {
-        constexpr int A = Fac<R>::A, B = Fac<R>::B;
-        cpx<G> U[B][A];
-        col_pass<G, R, A, B, 0>(v, U);
-#pragma unroll
-        for (int q1 = 0; q1 < A; ++q1) {
-            cpx<G> t[B];
-#pragma unroll
-            for (int r2 = 0; r2 < B; ++r2) t[r2] = U[r2][q1];
-            Dft<G, B>::run(t);
-#pragma unroll
-            for (int q2 = 0; q2 < B; ++q2) v[q1 + A * q2] = t[q2];
-        }
-    }
-};
 
 // ---------------------------------------------------------------- stages
 __device__ __forceinline__ unsigned fdiv(unsigned n, unsigned mul, unsigned sh)
@@ -462,6 +298,75 @@ template cudaError_t launch_fft_pass<double>(const cpx<double> *, cpx<double> *,
                                              const double *, const cpx<double> *, cudaStream_t);
 template cudaError_t launch_fft_pass<float>(const cpx<float> *, cpx<float> *, long, const DimGeom &, const float *,
                                             const cpx<float> *, cudaStream_t);
+
+// ---------------------------------------------------------------- compile-time lengths (fv_fft_fixed.cuh)
+#define FV_FIXED_ARGS const cpx<float> *in, cpx<float> *out, int rows, const DimGeom &dg, int P, int sP, int nz, int nzp, \
+                      const cpx<float> *twB, cudaStream_t st
+cudaError_t fft_fixed_a(FV_FIXED_ARGS);      // lengths up to 864
+cudaError_t fft_fixed_b(FV_FIXED_ARGS);      // up to 1728
+cudaError_t fft_fixed_c(FV_FIXED_ARGS);      // up to 2560
+cudaError_t fft_fixed_d(FV_FIXED_ARGS);      // up to 4096
+
+struct FixedLength { short M, R2, R3; };
+// every product 16 R2 R3 up to 4096 of the radices 4, 5, 6, 8, 9, 10, 12, 15, 16, at most 17 % apart above 480
+static const FixedLength kFixed[] = {
+    {256, 4, 4}, {320, 5, 4}, {384, 6, 4}, {400, 5, 5}, {480, 6, 5}, {512, 8, 4},
+    {576, 6, 6}, {640, 8, 5}, {720, 9, 5}, {768, 8, 6}, {800, 10, 5}, {864, 9, 6},
+    {960, 10, 6}, {1024, 8, 8}, {1152, 9, 8}, {1200, 15, 5}, {1280, 10, 8}, {1296, 9, 9},
+    {1440, 10, 9}, {1536, 12, 8}, {1600, 10, 10}, {1728, 12, 9}, {1920, 12, 10}, {2048, 16, 8},
+    {2160, 15, 9}, {2304, 12, 12}, {2400, 15, 10}, {2560, 16, 10}, {2880, 15, 12}, {3072, 16, 12},
+    {3600, 15, 15}, {3840, 16, 15}, {4096, 16, 16}};
+
+bool fft_choose_fixed(int target, int *radix, int &nstages, int &M)
+{
+    for (const FixedLength &l : kFixed)
+        if (l.M >= target) {
+            M = l.M;
+            radix[0] = 16;
+            radix[1] = l.R2;
+            radix[2] = l.R3;
+            nstages = 3;
+            return true;
+        }
+    return false;
+}
+
+size_t fft_fixed_table(const DimGeom &dg) { return (size_t)16 * dg.radix[1] + dg.M; }
+
+// tb[q 16 + m1] = e^{2 pi i q m1 / (16 R2)}, then tc[q 16 R2 + c] = e^{2 pi i q c / M}
+__global__ void k_fixed_twiddles(cpx<float> *tw, int M, int R2)
+{
+    const int k = blockIdx.x * blockDim.x + threadIdx.x;
+    const int nB = 16 * R2;
+    if (k >= nB + M) return;
+    double s, c;
+    if (k < nB) {
+        sincospi(2.0 * (double)((k / 16) * (k % 16)) / (double)nB, &s, &c);
+    } else {
+        const int j = k - nB;
+        sincospi(2.0 * (double)((j / nB) * (j % nB)) / (double)M, &s, &c);
+    }
+    tw[k] = cmk<float>((float)c, (float)s);
+}
+
+cudaError_t launch_fixed_twiddles(cpx<float> *tw, const DimGeom &dg, cudaStream_t st)
+{
+    const int n = (int)fft_fixed_table(dg);
+    k_fixed_twiddles<<<(n + 255) / 256, 256, 0, st>>>(tw, dg.M, dg.radix[1]);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_fft_fixed(const cpx<float> *in, cpx<float> *out, long rows, const DimGeom &dg, int P, int sP, int nz,
+                             int nzp, const cpx<float> *tw, cudaStream_t st)
+{
+    if (rows <= 0) return cudaSuccess;
+    if (rows > (1L << 30) || P < 1 || nz < 1) return cudaErrorInvalidValue;
+    const int r = (int)rows;
+    if (dg.M <= 864) return fft_fixed_a(in, out, r, dg, P, sP, nz, nzp, tw, st);
+    if (dg.M <= 1728) return fft_fixed_b(in, out, r, dg, P, sP, nz, nzp, tw, st);
+    if (dg.M <= 2560) return fft_fixed_c(in, out, r, dg, P, sP, nz, nzp, tw, st);
+    return fft_fixed_d(in, out, r, dg, P, sP, nz, nzp, tw, st);
+}
 
 // ---------------------------------------------------------------- host planning
 static const int kRadices[] = {16, 15, 12, 10, 9, 8, 6, 5, 4, 3, 2};

@@ -47,6 +47,7 @@ struct DimGeom {
     double pscale;  // M / (2 sigma X) : (x - D) -> target coordinate (FFT cells)
     double D;       // target centre (rad)
     double C;       // source centre
+    int fixed;      // 1: M is a compile-time length (launch_fft_fixed), radix = {16, R2, R3}
     int nstages;
     int radix[FV_MAX_STAGES];
     unsigned mr_mul[FV_MAX_STAGES], mr_sh[FV_MAX_STAGES];   // division by M / radix[s]
@@ -83,6 +84,7 @@ struct TimeBin {
     int nf1_top[3];
     int T[2];               // tile (= bin) size in cells
     int nbx, nby;           // bins per axis
+    int strips;             // bin order: 0 row by row (x fastest), 1 strip by strip (y fastest)
 };
 
 #define FV_SPREAD_SMEM_MAX (96 * 1024)
@@ -422,6 +424,11 @@ template <class G>
 cudaError_t launch_spread_direct(const double *e, long n_src, const void *flux, int flux_fp64, int n_freq,
                                  int f, const SliceGeom &g, cpx<G> *grid, cudaStream_t st);
 
+// Bins that one CTA of the bin scan takes.
+constexpr int kScanBlock = 4096;
+// ints launch_time_binning needs at counts: the bins' counts and the sums of the scan's blocks
+inline size_t bin_count_ints(int nb) { return (size_t)nb + (nb + kScanBlock - 1) / kScanBlock; }
+
 // Per time: rotate, horizon cut and counting sort of the visible sources by
 // top-channel tile.  sdir[3][n_src] and sidx[n_src] hold the sorted visible
 // directions and source indices; offsets[nb] is the visible count.
@@ -456,12 +463,38 @@ cudaError_t launch_spread_scatter(const int *offsets, const int *cell, const G *
                                   cudaStream_t st);
 size_t spread_scatter_smem(int elem_bytes, int n_pol, int nz);
 
+// Preparation and spreading in one launch for FP32 grids (w <= 8, n_pol 1 or 4, at most 16 up planes or height
+// terms): the sources sorted by strips (TimeBin::strips) with their per-time records tc, added to grid
+// [ny][nx][n_pol][strip_planes(nz)], which the caller has cleared; the x and y prescales of g are applied.  Any order of the
+// sources gives the same sums.
+constexpr int kEsTerms = 5;
+struct EsPoly {                       // kernel values of a w <= 8 point kernel as polynomials (es_polynomials)
+    float2 e[4][kEsTerms], o[4][kEsTerms];   // even and odd coefficients, each twice (packed arithmetic)
+};
+EsPoly es_polynomials(int w, double beta);
+// planes per product as the grid holds them: an even number where there is more than one (16-byte additions)
+__host__ __device__ inline int strip_planes(int nz) { return nz == 1 ? 1 : (nz + 1) & ~1; }
+bool spread_strip_fits(int w, int n_pol, int nz);
+cudaError_t launch_spread_strip(const float4 *tc, const int *sidx, const int *nv_ptr, long n_src, const void *flux,
+                                int flux_fp64, int n_freq, int f, const SliceGeom &g, const EsPoly &es,
+                                cpx<float> *grid, cudaStream_t st);
+
 // One FFT pass: rows of length N (input rows contiguous), prescale by pre[l],
 // zero-pad to M, FFT with e^{+2 pi i l m / M}, write band outputs transposed:
 // out[b][row] = P[(b - H) mod M].
 template <class G>
 cudaError_t launch_fft_pass(const cpx<G> *in, cpx<G> *out, long rows, const DimGeom &dg, const G *pre,
                             const cpx<G> *tw, cudaStream_t st);
+
+// The same pass for FP32 rows of a compile-time length (dg.fixed; M >= 2 N, no prescale): row r = (y, p) with
+// P = rows per y, its value l at in[(y N + l) sP + (p / nz) nzp + p % nz] (P = sP = nz = nzp = 1: contiguous rows).
+// tw: the tables of launch_fixed_twiddles (fft_fixed_table complex values).
+cudaError_t launch_fft_fixed(const cpx<float> *in, cpx<float> *out, long rows, const DimGeom &dg, int P, int sP, int nz,
+                             int nzp, const cpx<float> *tw, cudaStream_t st);
+// The smallest compile-time length M >= target, or false (target above 4096).
+bool fft_choose_fixed(int target, int *radix, int &nstages, int &M);
+size_t fft_fixed_table(const DimGeom &dg);
+cudaError_t launch_fixed_twiddles(cpx<float> *tw, const DimGeom &dg, cudaStream_t st);
 
 // Interpolation at the unique targets, deconvolution and postphase: Vu[u][pol] (FP64).
 template <class G>

@@ -139,6 +139,9 @@ struct fv_plan_s {
     int fft_max_radix = 16;
     int spread_method = 0;      // resolved method
     bool ring = false;          // FP32 2-D gather through the shared-memory ring (fv_spread_ring.cu)
+    bool xy_fixed = false;      // every channel's x and y FFT lengths are compile-time lengths (launch_fft_fixed)
+    bool strip = false;         // FP32 gather plans, w <= 7: preparation and spreading in one pass (fv_spread_strip.cu)
+    fv::EsPoly es_poly{};       //   its kernel values as polynomials
     int bin_req[2] = {0, 0};    // fv_opts.bin_size
     int T[2] = {32, 32}, nbx = 1, nby = 1, f_top = 0;
     double qscale_top[3] = {0, 0, 0};

@@ -165,7 +165,7 @@ size_t workspace_layout(const fv_plan_s::WsNeed &need, char *base, fv_plan_s::Wo
     if (need.tiled) {
         const size_t ns = (size_t)need.n_src, nb = (size_t)need.nb;
         o.bin_of = (int *)take(ns * sizeof(int));
-        o.counts = (int *)take(nb * sizeof(int));
+        o.counts = (int *)take(bin_count_ints((int)nb) * sizeof(int));
         o.offsets = (int *)take((nb + 1) * sizeof(int));
         o.cursor = (int *)take(nb * sizeof(int));
         o.sidx = (int *)take(ns * sizeof(int));
@@ -270,11 +270,19 @@ static void resolve_spread(fv_plan_s *p, int gs, int w)
     if (m == FV_SPREAD_GATHER && !gather_ok) m = FV_SPREAD_ATOMIC;
     if (m == FV_SPREAD_SCATTER && !scatter_ok) m = FV_SPREAD_ATOMIC;
     p->spread_method = m;
-    p->ring = ring_ok && (m == FV_SPREAD_GATHER || m == FV_SPREAD_TENSOR);
+    // FP32 gather plans with a kernel of at most 7 points: sources prepared and added in one pass, sorted by
+    // strips (fv_spread_strip.cu); an 8-point kernel fills the window's eight rows, so that every change of row
+    // would empty it, and keeps the ring (or the register gather)
+    p->strip = m == FV_SPREAD_GATHER && gs == 4 && p->precision == FV_MIXED && w <= 7 &&
+               p->xy_fixed && !p->use_basis && spread_strip_fits(w, p->n_pol, nzm);
+    p->ring = !p->strip && ring_ok && (m == FV_SPREAD_GATHER || m == FV_SPREAD_TENSOR);
     p->tiled = m != FV_SPREAD_ATOMIC;
-    // bins of the per-time sort: the plan's size, else 8 x 4 cells of the top channel's grid
-    p->T[0] = p->bin_req[0] > 0 ? p->bin_req[0] : 8;
-    p->T[1] = p->bin_req[1] > 0 ? p->bin_req[1] : 4;
+    // bins of the per-time sort: the plan's size, else 8 x 4 cells of the top channel's grid ((16 - w) x 1
+    // where the bins are ordered by strips: their columns and a footprint fill the 16 columns of the spreading's
+    // window)
+    p->T[0] = p->bin_req[0] > 0 ? p->bin_req[0] : (p->strip ? 16 - w : 8);
+    p->T[1] = p->bin_req[1] > 0 ? p->bin_req[1] : (p->strip ? 1 : 4);
+    if (p->strip) p->es_poly = es_polynomials(w, p->beta);
     p->nbx = (p->nf1_top[0] + p->T[0] - 1) / p->T[0];
     p->nby = (p->nf1_top[1] + p->T[1] - 1) / p->T[1];
 }
@@ -413,7 +421,11 @@ static fv_status dim_geometry(fv_plan_s *p, double X, double S, DimGeom &dg)
     if (nf1 < w + 1) nf1 = w + 1;     // Eq. 5 is the requirement; no 2w floor is needed
     if (nf1 > (1L << 20)) return p->fail(FV_ERR_UNSUPPORTED, "spreading grid too large");
     dg.nf1 = next235even(nf1);
-    dg.M = fft_choose_length((int)std::ceil(p->sigma * dg.nf1 - 1e-9), dg.radix, dg.nstages, p->fft_max_radix);
+    // FP32 grids at sigma >= 2: a compile-time length where there is one (up to 4,096 points)
+    const int target = (int)std::ceil(p->sigma * dg.nf1 - 1e-9);
+    dg.fixed = p->precision == FV_MIXED && p->sigma >= 2.0 && p->fft_max_radix == 16 &&
+               fft_choose_fixed(target, dg.radix, dg.nstages, dg.M);
+    if (!dg.fixed) dg.M = fft_choose_length(target, dg.radix, dg.nstages, p->fft_max_radix);
     if (dg.M < 0 || dg.M > maxM)
         return p->fail(FV_ERR_UNSUPPORTED, "FFT length " + std::to_string(dg.M) + " exceeds " +
                                                std::to_string(maxM) + " for one-CTA FFT passes");
@@ -507,6 +519,8 @@ static fv_status prepare(fv_plan_s *p)
     size_t pre_total = 0, tw_total = 0;
     for (int i = 0; i < 3; ++i) { p->nf1_max[i] = 1; p->M_max[i] = 1; }
     size_t grid_e = 0, bufA_e = 0, bufB_e = 0;
+    std::map<int, size_t> tw_of;
+    p->xy_fixed = true;
     for (int f = 0; f < nf; ++f) {
         SliceGeom &g = p->gf[f];
         g.nu = p->freq[f];
@@ -530,7 +544,7 @@ static fv_status prepare(fv_plan_s *p)
             if (i >= p->d) {
                 // no grid dimension: one plane, or the K planes of the height terms
                 dg.nf1 = i == 2 && p->hK > 0 ? p->hK : 1;
-                dg.M = 1; dg.B = 1; dg.H = 0; dg.qscale = 0; dg.pscale = 0; dg.D = 0; dg.C = 0;
+                dg.M = 1; dg.fixed = 0; dg.B = 1; dg.H = 0; dg.qscale = 0; dg.pscale = 0; dg.D = 0; dg.C = 0;
                 dg.nstages = 0;
                 continue;
             }
@@ -542,8 +556,11 @@ static fv_status prepare(fv_plan_s *p)
             p->M_max[i] = std::max(p->M_max[i], dg.M);
             p->pre_off[(size_t)f * 3 + i] = pre_total;
             pre_total += dg.nf1;
-            p->tw_off[(size_t)f * 3 + i] = tw_total;
-            tw_total += dg.M;
+            // twiddle tables by length: channels of one length share them (a compile-time length has its own
+            // tables behind the plain one)
+            const auto at = tw_of.emplace(dg.M, tw_total);
+            p->tw_off[(size_t)f * 3 + i] = at.first->second;
+            if (at.second) tw_total += dg.M + (dg.fixed ? fft_fixed_table(dg) : 0);
         }
         for (int i = 0; i < 2; ++i) {
             const double a = g.kappa * g.dim[i].pscale;
@@ -554,7 +571,8 @@ static fv_status prepare(fv_plan_s *p)
         g.kap_lo = (float)(g.kappa - (double)g.kap_hi);
         // buffer sizes (complex elements) for this channel
         const DimGeom *D = g.dim;
-        size_t grid_c = (size_t)p->n_pol * D[0].nf1 * D[1].nf1 * D[2].nf1;
+        p->xy_fixed = p->xy_fixed && D[0].fixed && D[1].fixed;
+        size_t grid_c = (size_t)p->n_pol * D[0].nf1 * D[1].nf1 * strip_planes(D[2].nf1);
         size_t pass1 = (size_t)D[0].B * p->n_pol * D[2].nf1 * D[1].nf1;
         size_t pass2 = (size_t)D[1].B * D[0].B * p->n_pol * D[2].nf1;
         size_t pass3 = p->d == 3 ? (size_t)D[2].B * D[1].B * D[0].B * p->n_pol : 0;
@@ -626,14 +644,18 @@ static fv_status prepare(fv_plan_s *p)
     for (int f = 0; f < nf; ++f) {
         for (int i = 0; i < p->d; ++i) {
             const DimGeom &dg = p->gf[f].dim[i];
+            const size_t to = p->tw_off[(size_t)f * 3 + i];
+            const bool first = tw_of.erase(dg.M) != 0;          // the first dimension of this length makes its tables
             if (p->precision == FV_FP64) {
                 CK(launch_prescale_table<double>((double *)p->d_pre + p->pre_off[(size_t)f * 3 + i], dg.nf1, dg.M, w,
                                                  p->beta, p->d_glx, p->d_glw, p->nq, p->stream));
-                CK(launch_twiddles<double>((cpx<double> *)p->d_tw + p->tw_off[(size_t)f * 3 + i], dg.M, p->stream));
+                if (first) CK(launch_twiddles<double>((cpx<double> *)p->d_tw + to, dg.M, p->stream));
             } else {
                 CK(launch_prescale_table<float>((float *)p->d_pre + p->pre_off[(size_t)f * 3 + i], dg.nf1, dg.M, w,
                                                 p->beta, p->d_glx, p->d_glw, p->nq, p->stream));
-                CK(launch_twiddles<float>((cpx<float> *)p->d_tw + p->tw_off[(size_t)f * 3 + i], dg.M, p->stream));
+                if (first) CK(launch_twiddles<float>((cpx<float> *)p->d_tw + to, dg.M, p->stream));
+                if (first && dg.fixed)
+                    CK(launch_fixed_twiddles((cpx<float> *)p->d_tw + to + dg.M, dg, p->stream));
             }
         }
     }
@@ -644,14 +666,15 @@ static fv_status prepare(fv_plan_s *p)
     // the gather spreading reads staged records: 16 (FP32) or 32 (FP64) bytes per source where the split
     // coordinates take 12 or 24, and strengths padded to 16 bytes
     const bool staged = p->spread_method == FV_SPREAD_GATHER || p->spread_method == FV_SPREAD_TENSOR;
-    p->need.frac_per_src = p->ring ? sizeof(RingRec) : (staged ? 4 * gs : 3 * gs);
+    p->need.frac_per_src = p->strip ? 0 : (p->ring ? sizeof(RingRec) : (staged ? 4 * gs : 3 * gs));
     // ring gather: a work list over the tiles of the largest grid, and slots for the parts of split tiles
     // (a tile's candidates come to at most 4 n_src, split tiles have more than kRingPart candidates each,
     // so there are at most 8 n_src / kRingPart parts; beyond kRingSlotsMax tiles run whole)
     p->need.ring_tiles = p->ring ? ring_tiles(p->nf1_max[0], p->nf1_max[1]) : 0;
     p->need.ring_slots = p->ring ? (int)std::min<long>(kRingSlotsMax, 8 * std::max<long>(p->n_src, 1) / kRingPart + 1) : 0;
     p->need.ring_np = p->ring ? p->n_pol : 0;
-    p->need.cs_per_src = staged ? (size_t)staged_cs_stride((int)gs, p->n_pol) * es : (size_t)p->n_pol * es;
+    p->need.cs_per_src =
+        p->strip ? 0 : (staged ? (size_t)staged_cs_stride((int)gs, p->n_pol) * es : (size_t)p->n_pol * es);
     // FP32 grids take each slice's coordinates and prephase from per-time records (no FP64 per slice)
     p->need.tc = p->precision == FV_MIXED && p->tiled;
     const size_t bin_bytes = p->tiled ? workspace_layout(p->need, nullptr, nullptr) -
@@ -688,6 +711,19 @@ static SliceGeom slice_geom_for(const fv_plan_s *p, int f, int t, const fv_plan_
     beam_float_constant(g.beam);
     beam_float_constant(g.beam2);
     return g;
+}
+
+// One FFT pass: the compile-time length where the dimension has one and no prescale is left to apply (tw: the plain
+// table, the fixed ones behind it; rows as launch_fft_fixed), else the general kernel on contiguous rows.
+template <class G>
+static cudaError_t fft_pass(const cpx<G> *in, cpx<G> *out, long rows, const DimGeom &dg, const G *pre, const cpx<G> *tw,
+                            cudaStream_t st, int P = 1, int sP = 1, int nz = 1, int nzp = 1)
+{
+    if constexpr (sizeof(G) == 4) {
+        if (dg.fixed && !pre) return launch_fft_fixed(in, out, rows, dg, P, sP, nz, nzp, tw + dg.M, st);
+    }
+    if (sP != 1) return cudaErrorInvalidValue;
+    return launch_fft_pass<G>(in, out, rows, dg, pre, tw, st);
 }
 
 // Slices of a lattice array (Section 2.2.1): one-bin time binning (rotation and horizon cut), then per
@@ -808,6 +844,7 @@ fv_status run_slices(fv_plan_s *p, fv_plan_s::Workspace &wk, cudaStream_t st, ch
             tb.T[1] = p->T[1];
             tb.nbx = p->nbx;
             tb.nby = p->nby;
+            tb.strips = p->strip ? 1 : 0;
             tb.d = p->d;
             for (int i = 0; i < 3; ++i) tb.D_top[i] = p->gf[p->f_top].dim[i].D;
             CK(prof_begin(p, PC_BIN, st));
@@ -831,7 +868,19 @@ fv_status run_slices(fv_plan_s *p, fv_plan_s::Workspace &wk, cudaStream_t st, ch
             cpx<double> *Vug = wk.Vu + (size_t)gr.u0 * p->n_pol;
             const DimGeom *D = g.dim;
             const size_t gel = (size_t)p->n_pol * D[0].nf1 * D[1].nf1 * D[2].nf1;
-            if (p->tiled) {
+            if (p->strip) {
+                CK(prof_begin(p, PC_MEMSET, st));
+                const size_t held = gel / D[2].nf1 * strip_planes(D[2].nf1);
+                CK(cudaMemsetAsync(grid, 0, held * sizeof(cpx<G>), st));
+                CK(prof_end(p, held * es));
+                g.pre_x = pre + p->pre_off[(size_t)f * 3];         // applied as rows are added to the grid
+                g.pre_y = pre + p->pre_off[(size_t)f * 3 + 1];
+                CK(prof_begin(p, PC_SPREAD, st));
+                CK(launch_spread_strip(wk.tc, wk.sidx, wk.offsets + nb, p->n_src, p->flux, p->flux_fp64, nf, f, g,
+                                       p->es_poly, (cpx<float> *)grid, st));
+                // the visible sources' records, indexes and fluxes read once, the grid written once
+                CK(prof_end(p, nvis * (48.0 + 4.0 + p->n_stokes * (p->flux_fp64 ? 8.0 : 4.0)) + gel * es));
+            } else if (p->tiled) {
                 G *frac = (G *)wk.frac;
                 cpx<G> *cs = (cpx<G> *)wk.cs;
                 // the gather spreading reads staged records (bulk-copied per chunk)
@@ -881,15 +930,18 @@ fv_status run_slices(fv_plan_s *p, fv_plan_s::Workspace &wk, cudaStream_t st, ch
             // the tiled spreading kernels stored the grid with its x and y prescale already applied
             const G *pre_x = p->tiled ? nullptr : pre + p->pre_off[o0];
             const G *pre_y = p->tiled ? nullptr : pre + p->pre_off[o0 + 1];
-            // pass 1 along x: rows (pol, z, y)
-            const long r1 = (long)p->n_pol * D[2].nf1 * D[1].nf1;
+            // pass 1 along x: rows (pol, z, y), or (y, pol, z) where the planes of a cell are adjacent (strips)
+            const int np = p->n_pol, nz = D[2].nf1, nzp = strip_planes(nz);
+            const long r1 = (long)np * nz * D[1].nf1;
             CK(prof_begin(p, PC_FFT_X, st));
-            CK(launch_fft_pass<G>(grid, A, r1, D[0], pre_x, tw + p->tw_off[o0], st));
+            if (p->strip) CK(fft_pass<G>(grid, A, r1, D[0], nullptr, tw + p->tw_off[o0], st, np * nz, np * nzp, nz, nzp));
+            else CK(fft_pass<G>(grid, A, r1, D[0], pre_x, tw + p->tw_off[o0], st));
             CK(prof_end(p, (double)r1 * (D[0].nf1 + D[0].B) * es));
             // pass 2 along y: rows (bx, pol, z)
-            const long r2 = (long)D[0].B * p->n_pol * D[2].nf1;
+            const long r2 = (long)D[0].B * np * nz;
             CK(prof_begin(p, PC_FFT_Y, st));
-            CK(launch_fft_pass<G>(A, Bb, r2, D[1], pre_y, tw + p->tw_off[o0 + 1], st));
+            if (p->strip) CK(fft_pass<G>(A, Bb, r2, D[1], nullptr, tw + p->tw_off[o0 + 1], st, np * nz, np * nz, np * nz, np * nz));
+            else CK(fft_pass<G>(A, Bb, r2, D[1], pre_y, tw + p->tw_off[o0 + 1], st));
             CK(prof_end(p, (double)r2 * (D[1].nf1 + D[1].B) * es));
             if (p->d == 2 || D[2].nf1 <= FV_ZDIRECT_MAX) {
                 // z (if any) summed directly inside the interpolation: no z pass
@@ -1044,7 +1096,7 @@ static fv_status prepare_basis(fv_plan_s *p)
     for (int i = 0; i < 3; ++i) {
         DimGeom &dg = g.dim[i];
         if (i >= p->d) {
-            dg.nf1 = 1; dg.M = 1; dg.B = 1; dg.H = 0; dg.qscale = 0; dg.pscale = 0; dg.D = 0; dg.C = 0;
+            dg.nf1 = 1; dg.fixed = 0; dg.M = 1; dg.B = 1; dg.H = 0; dg.qscale = 0; dg.pscale = 0; dg.D = 0; dg.C = 0;
             dg.nstages = 0;
             continue;
         }
@@ -1092,7 +1144,7 @@ static fv_status prepare_basis(fv_plan_s *p)
         p->pre_off[i] = pre_total;
         pre_total += g.dim[i].nf1;
         p->tw_off[i] = tw_total;
-        tw_total += g.dim[i].M;
+        tw_total += g.dim[i].M + (g.dim[i].fixed ? fft_fixed_table(g.dim[i]) : 0);
     }
     CK(cudaMalloc(&p->d_pre, std::max<size_t>(pre_total, 1) * gs));
     CK(cudaMalloc(&p->d_tw, std::max<size_t>(tw_total, 1) * es));
@@ -1106,6 +1158,7 @@ static fv_status prepare_basis(fv_plan_s *p)
             CK(launch_prescale_table<float>((float *)p->d_pre + p->pre_off[i], dg.nf1, dg.M, w, p->beta, p->d_glx,
                                             p->d_glw, p->nq, p->stream));
             CK(launch_twiddles<float>((cpx<float> *)p->d_tw + p->tw_off[i], dg.M, p->stream));
+            if (dg.fixed) CK(launch_fixed_twiddles((cpx<float> *)p->d_tw + p->tw_off[i] + dg.M, dg, p->stream));
         }
     }
     CK(cudaMalloc(&p->d_bas_M, M.size() * sizeof(double)));
@@ -1232,11 +1285,11 @@ fv_status run_basis(fv_plan_s *p, fv_plan_s::Workspace &wk, cudaStream_t st, cha
             }
             const long r1 = (long)K * D[2].nf1 * D[1].nf1;
             CK(prof_begin(p, PC_FFT_X, st));
-            CK(launch_fft_pass<G>(grid, A, r1, D[0], nullptr, tw + p->tw_off[0], st));
+            CK(fft_pass<G>(grid, A, r1, D[0], nullptr, tw + p->tw_off[0], st));
             CK(prof_end(p, (double)r1 * (D[0].nf1 + D[0].B) * es));
             const long r2 = (long)D[0].B * K * D[2].nf1;
             CK(prof_begin(p, PC_FFT_Y, st));
-            CK(launch_fft_pass<G>(A, Bb, r2, D[1], nullptr, tw + p->tw_off[1], st));
+            CK(fft_pass<G>(A, Bb, r2, D[1], nullptr, tw + p->tw_off[1], st));
             CK(prof_end(p, (double)r2 * (D[1].nf1 + D[1].B) * es));
             const int nug = gr.u1 - gr.u0;
             CK(prof_begin(p, PC_INTERP, st));

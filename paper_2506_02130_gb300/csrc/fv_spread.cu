@@ -23,6 +23,7 @@
 // bins, i.e. one contiguous range of sorted sources per bin row.
 #include "fv_staged.cuh"
 #include "fv_internal.cuh"
+#include "fv_prep.cuh"
 
 #include <math.h>
 
@@ -44,7 +45,7 @@ __global__ void k_bin_count(const double *__restrict__ e, long n_src, TimeBin tb
     const double s1 = tb.R[3] * ex + tb.R[4] * ey + tb.R[5] * ez;
     int cx = top_cell((s0 - tb.C[0]) * tb.qscale_top[0], tb.nf1_top[0]);
     int cy = top_cell((s1 - tb.C[1]) * tb.qscale_top[1], tb.nf1_top[1]);
-    int b = (cy / tb.T[1]) * tb.nbx + cx / tb.T[0];
+    const int b = tb.strips ? (cx / tb.T[0]) * tb.nby + cy / tb.T[1] : (cy / tb.T[1]) * tb.nbx + cx / tb.T[0];
     bin_of[n] = b;
     // warp-aggregated count: one atomic per distinct bin among the active lanes
     const unsigned act = __activemask();
@@ -52,30 +53,78 @@ __global__ void k_bin_count(const double *__restrict__ e, long n_src, TimeBin tb
     if ((int)(threadIdx.x & 31) == __ffs(grp) - 1) atomicAdd(&counts[b], __popc(grp));
 }
 
-// exclusive scan of counts[0..nb) into offsets[0..nb], cursor = offsets (one CTA of 1024 threads)
-__global__ void k_bin_scan(const int *__restrict__ counts, int nb, int *__restrict__ offsets, int *__restrict__ cursor)
+// Exclusive scan of counts[0..nb) into offsets[0..nb], cursor = offsets.  A CTA of 1,024 threads scans
+// kScanBlock values, four a thread, by warp shuffles.  Up to kScanBlock bins one CTA does it all; more bins
+// take one CTA per kScanBlock values, with the sums of the blocks before it added up from blk (k_bin_sums).
+// (One CTA walking all the bins took 49 us for the 35,000 bins of the 350-antenna workload: a serial chain on
+// one SM; the strips of the FP32 spreading have four times as many.)
+__device__ __forceinline__ int block_scan_1024(int v, int *s_warp, int &total)
 {
-    __shared__ int part[1024];
-    const int t = threadIdx.x;
-    const int per = (nb + 1023) / 1024;
-    const int lo = t * per, hi = min(nb, lo + per);
-    int s = 0;
-    for (int i = lo; i < hi; ++i) s += counts[i];
-    part[t] = s;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    int incl = v;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int t = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += t;
+    }
+    if (lane == 31) s_warp[warp] = incl;
     __syncthreads();
-    for (int o = 1; o < 1024; o <<= 1) {
-        int v = t >= o ? part[t - o] : 0;
-        __syncthreads();
-        part[t] += v;
-        __syncthreads();
+    if (warp == 0) {
+        int w = s_warp[lane];
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int t = __shfl_up_sync(0xffffffffu, w, o);
+            if (lane >= o) w += t;
+        }
+        s_warp[lane] = w;
     }
-    int run = part[t] - s;   // exclusive prefix of this thread's chunk
-    for (int i = lo; i < hi; ++i) {
-        offsets[i] = run;
-        cursor[i] = run;
-        run += counts[i];
+    __syncthreads();
+    total = s_warp[31];
+    return incl - v + (warp > 0 ? s_warp[warp - 1] : 0);
+}
+
+__global__ void __launch_bounds__(1024) k_bin_sums(const int *__restrict__ counts, int nb, int *__restrict__ blk)
+{
+    __shared__ int s_warp[32];
+    const int i0 = blockIdx.x * kScanBlock + threadIdx.x;
+    int v = 0;
+#pragma unroll
+    for (int k = 0; k < kScanBlock / 1024; ++k) {
+        const int i = i0 + k * 1024;
+        if (i < nb) v += counts[i];
     }
-    if (t == 1023) offsets[nb] = part[1023];
+    int total;
+    block_scan_1024(v, s_warp, total);
+    if (threadIdx.x == 0) blk[blockIdx.x] = total;
+}
+
+__global__ void __launch_bounds__(1024) k_bin_scan(const int *__restrict__ counts, int nb, int *__restrict__ offsets,
+                                                   int *__restrict__ cursor, const int *__restrict__ blk)
+{
+    __shared__ int s_warp[32], s_warp2[32];
+    constexpr int kPer = kScanBlock / 1024;
+    int before = 0, total;
+    if (blockIdx.x > 0) {
+        int v = 0;
+        for (int i = threadIdx.x; i < (int)blockIdx.x; i += 1024) v += blk[i];
+        block_scan_1024(v, s_warp2, before);
+    }
+    const int i0 = blockIdx.x * kScanBlock + threadIdx.x * kPer;
+    int c[kPer], s = 0;
+#pragma unroll
+    for (int k = 0; k < kPer; ++k) {
+        c[k] = i0 + k < nb ? counts[i0 + k] : 0;
+        s += c[k];
+    }
+    int run = before + block_scan_1024(s, s_warp, total);
+#pragma unroll
+    for (int k = 0; k < kPer; ++k)
+        if (i0 + k < nb) {
+            offsets[i0 + k] = run;
+            cursor[i0 + k] = run;
+            run += c[k];
+            if (i0 + k == nb - 1) offsets[nb] = run;
+        }
 }
 
 // Two floats hi + lo holding an FP64 value to about 2^-48 of its magnitude.
@@ -132,7 +181,10 @@ cudaError_t launch_time_binning(const double *e, long n_src, const TimeBin &tb, 
     cudaError_t err = cudaMemsetAsync(counts, 0, (size_t)nb * sizeof(int), st);
     if (err != cudaSuccess) return err;
     if (n_src > 0) k_bin_count<<<(unsigned)((n_src + 255) / 256), 256, 0, st>>>(e, n_src, tb, bin_of, counts);
-    k_bin_scan<<<1, 1024, 0, st>>>(counts, nb, offsets, cursor);
+    const int blocks = (nb + kScanBlock - 1) / kScanBlock;
+    int *blk = counts + nb;                    // the blocks' sums lie behind the counts (bin_count_ints)
+    if (blocks > 1) k_bin_sums<<<blocks, 1024, 0, st>>>(counts, nb, blk);
+    k_bin_scan<<<blocks, 1024, 0, st>>>(counts, nb, offsets, cursor, blk);
     if (n_src > 0)
         k_bin_scatter<<<(unsigned)((n_src + 255) / 256), 256, 0, st>>>(e, n_src, tb, bin_of, cursor, sdir, sidx,
                                                                        tc);
@@ -214,64 +266,6 @@ __global__ void __launch_bounds__(256) k_prep(const double *__restrict__ sdir, c
             frac[(size_t)k * n_src + i] = fr[k];
         }
     }
-}
-
-// FP32 grids: the same strengths, prephase and grid coordinates from the per-time records tc (see
-// launch_time_binning) without FP64 arithmetic.  Every channel's coordinate and prephase are the top
-// channel's times r = kappa / kappa_top, formed in double-float arithmetic (an exact product by FMA plus
-// the cross terms, about 2^-44 relative); the prephase is reduced by 2 pi split in two floats; the first
-// footprint cell follows from the accurate offset l0 - q, which is brought into [-w/2, 1 - w/2).
-__device__ __forceinline__ float2 mul_df(float ah, float al, float bh, float bl)
-{
-    const float p = ah * bh;
-    const float e = fmaf(ah, bh, -p) + (ah * bl + al * bh);
-    return make_float2(p, e);
-}
-
-// One source of one slice from its per-time record (a, b, sd) and source index n: strengths with prephase
-// c[0..np), first footprint cells ci and offsets fr.
-struct PrepOne {
-    cpx<float> c[4];
-    int np;
-    int ci[3];
-    float fr[3];
-};
-
-__device__ __forceinline__ void prep_tc_one(const float4 a, const float4 b, const float4 sd, long n, const void *flux,
-                                            int flux_fp64, long n_src, int n_freq, int f, const SliceGeom &g,
-                                            PrepOne &o)
-{
-    o.np = source_strengths<float, float>(g, sd.x, sd.y, sd.z, n, flux, flux_fp64, n_src, n_freq, f, o.c);
-    // prephase r ph_top, reduced to about [-pi, pi]: 2 pi = 6.2831855 - 1.7484555e-7
-    const float2 ph = mul_df(g.rsc_hi, g.rsc_lo, b.z, b.w);
-    const float k = rintf(ph.x * 0.15915494f);
-    const float phr = fmaf(-k, -1.7484555e-7f, fmaf(-k, 6.2831855f, ph.x)) + ph.y;
-    float sp, cp;
-    sincosf(phr, &sp, &cp);
-#pragma unroll
-    for (int p = 0; p < 4; ++p)
-        if (p < o.np) o.c[p] = cmul(o.c[p], cmk<float>(cp, sp));
-    const float hw = 0.5f * (float)g.w;
-#pragma unroll
-    for (int k3 = 0; k3 < 3; ++k3) {
-        o.ci[k3] = 0;
-        o.fr[k3] = 0.0f;
-        if (k3 < g.d) {
-            const float qh = k3 == 0 ? a.x : (k3 == 1 ? a.z : b.x), ql = k3 == 0 ? a.y : (k3 == 1 ? a.w : b.y);
-            const float2 q = mul_df(g.rsc_hi, g.rsc_lo, qh, ql);
-            float l0 = ceilf(q.x - hw);
-            float off = (l0 - q.x) - q.y;                 // l0 - q
-            if (off >= 1.0f - hw) { l0 -= 1.0f; off -= 1.0f; }
-            else if (off < -hw) { l0 += 1.0f; off += 1.0f; }
-            int c = (int)l0 + g.dim[k3].nf1 / 2;
-            const int hi = g.dim[k3].nf1 - g.w;
-            if (c < 0) { off -= (float)c; c = 0; }
-            else if (c > hi) { off -= (float)(c - hi); c = hi; }
-            o.ci[k3] = c;
-            o.fr[k3] = off;
-        }
-    }
-    if (g.K) o.fr[2] = (sd.z - g.hc_f) * g.hs_inv_f;    // height terms: the argument u of T_q
 }
 
 // MODE 0: cell / frac / cs arrays; 1: staged records
