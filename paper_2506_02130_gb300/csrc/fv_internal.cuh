@@ -118,17 +118,18 @@ struct SliceGeom {
     // follow from k b_up (height_weight)
     int K;
     double hc, hs;
-    float hc_f, hs_inv_f;
+    float hc_f, hs_f, hs_inv_f;
     // nu and beta rounded to FP32 once on the host (a per-thread FP64 -> FP32 conversion runs on the
     // narrow FP64 pipe)
     float nu_f, beta_f;
     // FP32 two-dimensional interpolation without FP64: the target's grid coordinate is
     // p_i = -(kappa pscale_i) (b_i - bcen_i) and its postphase argument -kappa (b . C), formed as
     // double-float products of the per-channel factors (a_i = kappa pscale_i and kappa as float pairs)
-    // and the per-target tables tgt_db[u] = (b_x - bcen_x, b_y - bcen_y) and tgt_bc[u] = b . C (float
+    // and the per-target tables tgt_db[u] = (b_x - bcen_x, b_y - bcen_y) and tgt_bc[u] = b . C (over the
+    // grid's dimensions, and b_up hc with height terms; a float pair) and b_up (float
     // pairs, channel independent; nullptr: the FP64 set-up)
     const float4 *tgt_db;
-    const float2 *tgt_bc;
+    const float4 *tgt_bc;
     float a_hi[2], a_lo[2], kap_hi, kap_lo;
 };
 
@@ -200,6 +201,31 @@ __device__ __forceinline__ cpx<G> height_weight(const SliceGeom &g, double b_up,
         im = -t;
     }
     return cmk<G>((G)re, (G)im);
+}
+
+// The same weight without its phase exp(-i k b_up hc), which the FP32 targets' postphase holds (tgt_bc), in FP32
+// for the argument's series |k b_up hs| <= 2 (every term is below the first), else from the FP64 series.
+__device__ __forceinline__ cpx<float> height_bessel(const SliceGeom &g, float b_up, int q)
+{
+    const float x = g.kap_hi * b_up * g.hs_f, h = 0.5f * x;
+    float j;
+    if (fabsf(x) <= 2.0f) {
+        float term = 1.0f;
+        for (int k = 1; k <= q; ++k) term *= h * (1.0f / (float)k);
+        float sum = term;
+        const float h2 = h * h;
+        for (int m = 1; m < 24; ++m) {
+            term *= -h2 / ((float)m * (float)(m + q));
+            sum += term;
+            if (fabsf(term) <= 1e-8f * fabsf(sum)) break;
+        }
+        j = sum;
+    } else {
+        j = (float)bessel_jq(q, g.kappa * (double)b_up * g.hs, 1e-10);
+    }
+    if (q > 0) j *= 2.0f;
+    // (-i)^q
+    return (q & 1) ? cmk<float>(0.0f, (q & 2) ? j : -j) : cmk<float>((q & 2) ? -j : j, 0.0f);
 }
 
 // Position of Stokes parameter k of source n at channel f in the fluxes a slice reads (flux_index) and
@@ -510,9 +536,9 @@ struct SliceOut {
     int u_base;
 };
 
-// Whether launch_interp_zdirect can write a slice's output itself for this geometry (two-dimensional
-// grids without height terms, n_pol 1 or 4).
-bool interp_fuses_scatter(const SliceGeom &g);
+// Whether launch_interp_zdirect can write a slice's output itself for this geometry and grid precision
+// (two-dimensional grids without height terms; FP32 grids with an even number of planes per cell).
+bool interp_fuses_scatter(const SliceGeom &g, int elem_bytes);
 
 // Same, reading the band after the x and y passes only ([b_y][b_x][pol][l_z]),
 // with the z axis summed directly (nf1_z <= 16).  so (or nullptr): write the output of the targets'

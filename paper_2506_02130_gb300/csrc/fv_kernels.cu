@@ -507,273 +507,69 @@ __global__ void __launch_bounds__(256) k_interp_zdirect(const cpx<G> *__restrict
     }
 }
 
-// The same sum for one polarisation and a short, even z axis in FP32, read
-// row by row: one warp per target, lane = c * (Nz/2) + h holds z values
-// (2h, 2h+1) of footprint cell c of the current footprint row, so a warp
-// reads one row of the footprint (w cells x Nz values, contiguous in the
-// band) with a single 16-byte load per lane.  The lane applies K(2h),
-// K(2h+1) and the row's y weight, scales by its cell's x weight at the end,
-// and the warp reduces.  Needs w * Nz / 2 <= 32.
-__global__ void __launch_bounds__(256) k_interp_zrow(const cpx<float> *__restrict__ band,
-                                                     const double *__restrict__ bu, int n_u,
-                                                     const double *__restrict__ dec, SliceGeom g,
-                                                     const float *__restrict__ prez,
-                                                     const cpx<float> *__restrict__ twz, cpx<double> *__restrict__ Vu)
+constexpr int kIbMaxW = 16;                  // largest kernel width of the warp-per-target forms
+
+// FP32 set-up of a target without FP64: double-float products of the per-channel factors and the target's float
+// pairs, then the first footprint cell m = ceil(p - w/2) and f = p - m brought into (w/2 - 1, w/2] (as the FP64
+// form), and the postphase reduced by 2 pi = 6.2831855 - 1.7484555e-7.
+__device__ __forceinline__ void target_setup(const SliceGeom &g, long u, int &m0, int &m1, float &f0, float &f1,
+                                             float &phr, float &b_up)
 {
-    const int lane = threadIdx.x & 31;
-    const int u = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    if (u >= n_u) return;
-    const int w = g.w;
-    const float two_over_w = 2.0f / (float)w;
-    const float beta = g.beta_f;
-    double x[3] = {0.0, 0.0, 0.0};
-    float fr[3];
-    int m0[3] = {0, 0, 0};
+    const float4 db = g.tgt_db[u];
+    const float4 bc = g.tgt_bc[u];
+    b_up = bc.z;
+    const float hw = 0.5f * (float)g.w;
+    float mm[2], ff[2];
 #pragma unroll
-    for (int i = 0; i < 3; ++i) {
-        fr[i] = 0.0f;
-        if (i < g.d) {
-            x[i] = -g.kappa * bu[3 * u + i];
-            double p = (x[i] - g.dim[i].D) * g.dim[i].pscale;
-            double m = ceil(p - 0.5 * w);
-            m0[i] = (int)m;
-            fr[i] = (float)(p - m);
-        }
+    for (int i = 0; i < 2; ++i) {
+        const float dh = i == 0 ? db.x : db.z, dl = i == 0 ? db.y : db.w;
+        float ph = g.a_hi[i] * dh;
+        float pl = fmaf(g.a_hi[i], dh, -ph) + (g.a_hi[i] * dl + g.a_lo[i] * dh);
+        ph = -ph;
+        pl = -pl;                                   // p = ph + pl
+        float m = ceilf(ph - hw);
+        float f = (ph - m) + pl;
+        if (f > hw) { m += 1.0f; f -= 1.0f; }
+        else if (f <= hw - 1.0f) { m -= 1.0f; f += 1.0f; }
+        mm[i] = m;
+        ff[i] = f;
     }
-    const int Nz = g.d == 3 || g.K ? g.dim[2].nf1 : 1;     // up planes or height terms
-    const int L = Nz / 2;                    // lanes per footprint cell
-    // K(l_z) for l_z = lane < Nz, as in k_interp_zdirect
-    cpx<float> Kmine = cmk<float>(1.0f, 0.0f);
-    if (lane < Nz && g.K) {
-        Kmine = height_weight<float>(g, bu[3 * u + 2], lane);
-    } else if (lane < Nz) {
-        const int Mz = g.dim[2].M;
-        const int lc = lane - Nz / 2;
-        cpx<float> acc = cmk<float>(0.0f, 0.0f);
-        int e = (lc * m0[2]) % Mz;
-        if (e < 0) e += Mz;
-        int step = lc % Mz;
-        if (step < 0) step += Mz;
-        for (int jz = 0; jz < w; ++jz) {
-            const float wt = es_kernel(two_over_w * (fr[2] - (float)jz), beta);
-            acc = cadd(acc, cscale(twz[e], wt));
-            e += step;
-            if (e >= Mz) e -= Mz;
-        }
-        Kmine = cscale(acc, prez[lane]);
-    }
-    const int c = lane / L, h = lane - c * L;
-    const bool active = c < w;
-    const int src = active ? 2 * h : 0;
-    const cpx<float> K0 = cmk<float>(__shfl_sync(0xffffffffu, Kmine.x, src), __shfl_sync(0xffffffffu, Kmine.y, src));
-    const cpx<float> K1 =
-        cmk<float>(__shfl_sync(0xffffffffu, Kmine.x, src + 1), __shfl_sync(0xffffffffu, Kmine.y, src + 1));
-    const float wxm = lane < w ? es_kernel(two_over_w * (fr[0] - (float)lane), beta) : 0.0f;
-    const float wym = lane < w ? es_kernel(two_over_w * (fr[1] - (float)lane), beta) : 0.0f;
-    const float wx = __shfl_sync(0xffffffffu, wxm, active ? c : 0);
-    const int Bx = g.dim[0].B;
-    const int bx0 = m0[0] + g.dim[0].H, by0 = m0[1] + g.dim[1].H;
-    float ax = 0.0f, ay = 0.0f;
-    for (int jy = 0; jy < w; ++jy) {        // same trip count on every lane (shuffle inside)
-        const float wy = __shfl_sync(0xffffffffu, wym, jy);
-        if (active) {
-            const cpx<float> *cell = band + ((size_t)(by0 + jy) * Bx + (bx0 + c)) * Nz + 2 * h;
-            cpx<float> v0, v1;
-            load_pair(cell, v0, v1);
-            const cpx<float> s = cadd(cmul(v0, K0), cmul(v1, K1));
-            ax += wy * s.x;
-            ay += wy * s.y;
-        }
-    }
-    ax *= wx;
-    ay *= wx;
-    for (int o = 16; o > 0; o >>= 1) {
-        ax += __shfl_xor_sync(0xffffffffu, ax, o);
-        ay += __shfl_xor_sync(0xffffffffu, ay, o);
-    }
-    if (lane == 0) {
-        double ph = 0.0;
-#pragma unroll
-        for (int i = 0; i < 3; ++i)
-            if (i < g.d) ph += x[i] * g.dim[i].C;
-        double sp, cp;
-        sincos(ph, &sp, &cp);
-        const double dk = dec[u];
-        const cpx<double> v = cmk<double>((double)ax * dk, (double)ay * dk);
-        Vu[u] = cmul(v, cmk<double>(cp, sp));
-    }
+    m0 = (int)mm[0];
+    m1 = (int)mm[1];
+    f0 = ff[0];
+    f1 = ff[1];
+    float qh = g.kap_hi * bc.x;
+    const float ql = fmaf(g.kap_hi, bc.x, -qh) + (g.kap_hi * bc.y + g.kap_lo * bc.x);
+    qh = -qh;                                        // argument -kappa (b . C) = qh - ql
+    const float k = rintf(qh * 0.15915494f);
+    phr = fmaf(-k, -1.7484555e-7f, fmaf(-k, 6.2831855f, qh)) - ql;
 }
 
-// Interpolation with the per-target set-up spread over the threads.  A CTA
-// takes 32 targets: first threads 0-31 compute, one target each, the FP64
-// coordinates, the first footprint cell, the kernel values of x and y (and
-// for a short z axis the vector K(l_z) of the direct z sum), and the postphase
-// and deconvolution factor, into shared memory.  Then each of the 4 warps
-// walks 8 of the targets, all lanes reading footprint values from the band
-// (ZROW: one footprint row of w cells x Nz z values per load round, one
-// 16-byte load per lane; 2-D: lanes over the w x w cells, n_pol values each),
-// and reduces; lane 0 writes the target's value.
-constexpr int kIbThreads = 128;
-constexpr int kIbTargets = 32;
-constexpr int kIbPerWarp = kIbTargets / (kIbThreads / 32);
-constexpr int kIbMaxW = 16;
-
-template <class G, bool ZROW>
-__global__ void __launch_bounds__(kIbThreads) k_interp_batch(const cpx<G> *__restrict__ band,
-                                                             const double *__restrict__ bu, int n_u,
-                                                             const double *__restrict__ dec, SliceGeom g,
-                                                             const G *__restrict__ prez,
-                                                             const cpx<G> *__restrict__ twz,
-                                                             cpx<double> *__restrict__ Vu)
+// The NP values of a target to its nb baselines u_bl[b0 ..): out[b][p].  Four indexes are read ahead of their
+// stores: the shortest baseline of a regular array has hundreds of copies, and its warp sets the launch's length.
+template <class G, int NP>
+__device__ __forceinline__ void write_target(const SliceOut &so, int b0, int nb, const G *rx, const G *ry, int lane)
 {
-    __shared__ G s_wx[kIbTargets][kIbMaxW + 1], s_wy[kIbTargets][kIbMaxW + 1];
-    __shared__ cpx<G> s_K[ZROW ? kIbTargets : 1][ZROW ? 8 : 1];
-    __shared__ int s_bx[kIbTargets], s_by[kIbTargets];
-    __shared__ cpx<double> s_post[kIbTargets];
-    const long u0 = (long)blockIdx.x * kIbTargets;
-    const int w = g.w;
-    const G two_over_w = (G)2 / (G)w, beta = geom_beta<G>(g);
-    // --- per-target set-up, one target per thread
-    if (threadIdx.x < kIbTargets) {
-        const int tl = threadIdx.x;
-        const long u = u0 + tl;
-        const bool valid = u < n_u;
-        double x[3] = {0.0, 0.0, 0.0};
-        int m0[3] = {0, 0, 0};
-        G fr[3] = {(G)0, (G)0, (G)0};
+    cpx<G> *o = reinterpret_cast<cpx<G> *>(so.out);
+    const int p = NP == 1 ? 0 : lane & 3;            // the same for every value of a lane
+    G vx = rx[0], vy = ry[0];
 #pragma unroll
-        for (int i = 0; i < 3; ++i) {
-            if (i < g.d && valid) {
-                x[i] = -g.kappa * bu[3 * u + i];
-                const double pp = (x[i] - g.dim[i].D) * g.dim[i].pscale;
-                const double m = ceil(pp - 0.5 * w);
-                m0[i] = (int)m;
-                fr[i] = (G)(pp - m);
-            }
+    for (int q = 1; q < NP; ++q)
+        if (p == q) {
+            vx = rx[q];
+            vy = ry[q];
         }
-        for (int j = 0; j < w; ++j) {
-            s_wx[tl][j] = es_kernel(two_over_w * (fr[0] - (G)j), beta);
-            s_wy[tl][j] = es_kernel(two_over_w * (fr[1] - (G)j), beta);
+    const int n = nb * NP;
+    for (int k = lane; k < n; k += 128) {
+        int b[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const int kk = k + 32 * j;
+            b[j] = kk < n ? so.u_bl[b0 + (NP == 1 ? kk : kk >> 2)] : -1;
         }
-        s_bx[tl] = m0[0] + g.dim[0].H;
-        s_by[tl] = m0[1] + g.dim[1].H;
-        if (ZROW && g.K) {
-            // height terms: the weights are computed by all threads below
-        } else if (ZROW) {
-            const int Nz = g.dim[2].nf1, Mz = g.dim[2].M;
-            G phz[kIbMaxW];
 #pragma unroll
-            for (int jz = 0; jz < kIbMaxW; ++jz)
-                phz[jz] = jz < w ? es_kernel(two_over_w * (fr[2] - (G)jz), beta) : (G)0;
-            for (int lz = 0; lz < Nz; ++lz) {
-                const int lc = lz - Nz / 2;
-                int e = (lc * m0[2]) % Mz;
-                if (e < 0) e += Mz;
-                int step = lc % Mz;
-                if (step < 0) step += Mz;
-                cpx<G> acc = cmk<G>((G)0, (G)0);
-#pragma unroll
-                for (int jz = 0; jz < kIbMaxW; ++jz) {
-                    if (jz < w) {
-                        acc = cadd(acc, cscale(twz[e], phz[jz]));
-                        e += step;
-                        if (e >= Mz) e -= Mz;
-                    }
-                }
-                s_K[ZROW ? tl : 0][ZROW ? lz : 0] = cscale(acc, prez[lz]);
-            }
-        }
-        cpx<double> post = cmk<double>(0.0, 0.0);
-        if (valid) {
-            double ph = 0.0;
-#pragma unroll
-            for (int i = 0; i < 3; ++i)
-                if (i < g.d) ph += x[i] * g.dim[i].C;
-            double sp, cp;
-            sincos(ph, &sp, &cp);
-            post = cmk<double>(cp * dec[u], sp * dec[u]);
-        }
-        s_post[tl] = post;
-    }
-    if (ZROW && g.K) {
-        // height weights of the CTA's targets, one (target, term) pair per thread and round
-        const int Nz = g.dim[2].nf1;
-        for (int idx = threadIdx.x; idx < kIbTargets * Nz; idx += kIbThreads) {
-            const int tl = idx / Nz, lz = idx - tl * Nz;
-            const long u = u0 + tl;
-            s_K[ZROW ? tl : 0][ZROW ? lz : 0] = u < n_u ? height_weight<G>(g, bu[3 * u + 2], lz) : cmk<G>((G)0, (G)0);
-        }
-    }
-    __syncthreads();
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int np = g.n_pol;
-    const int Bx = g.dim[0].B;
-    const int t0 = warp * kIbPerWarp;
-    const int nt = (int)max(0L, min((long)kIbPerWarp, (long)n_u - u0 - t0));
-    if (ZROW) {
-        const int Nz = g.dim[2].nf1, L = Nz / 2;
-        const int c = lane / L, h = lane - c * L;
-        const bool active = c < w;
-        const size_t rstride = (size_t)Bx * Nz;
-        for (int tt = 0; tt < nt; ++tt) {
-            const int t = t0 + tt;
-            G ax = (G)0, ay = (G)0;
-            if (active) {
-                const cpx<G> K0 = s_K[ZROW ? t : 0][ZROW ? 2 * h : 0];
-                const cpx<G> K1 = s_K[ZROW ? t : 0][ZROW ? 2 * h + 1 : 0];
-                const cpx<G> *rowp = band + ((size_t)s_by[t] * Bx + (s_bx[t] + c)) * Nz + 2 * h;
-#pragma unroll 4
-                for (int jy = 0; jy < w; ++jy) {
-                    cpx<G> v0, v1;
-                    load_pair(rowp + jy * rstride, v0, v1);
-                    const cpx<G> sm = cadd(cmul(v0, K0), cmul(v1, K1));
-                    const G wy = s_wy[t][jy];
-                    ax += wy * sm.x;
-                    ay += wy * sm.y;
-                }
-                const G wx = s_wx[t][c];
-                ax *= wx;
-                ay *= wx;
-            }
-            for (int o = 16; o > 0; o >>= 1) {
-                ax += __shfl_xor_sync(0xffffffffu, ax, o);
-                ay += __shfl_xor_sync(0xffffffffu, ay, o);
-            }
-            if (lane == 0) Vu[u0 + t] = cmul(cmk<double>((double)ax, (double)ay), s_post[t]);
-        }
-    } else {
-        const int ww = w * w;
-        for (int tt = 0; tt < nt; ++tt) {
-            const int t = t0 + tt;
-            G acc[8];
-#pragma unroll
-            for (int k = 0; k < 8; ++k) acc[k] = (G)0;
-            const int bx0 = s_bx[t], by0 = s_by[t];
-            for (int idx = lane; idx < ww; idx += 32) {
-                const int jy = idx / w, jx = idx - jy * w;
-                const G wt = s_wx[t][jx] * s_wy[t][jy];
-                const cpx<G> *cell = band + ((size_t)(by0 + jy) * Bx + (bx0 + jx)) * np;
-#pragma unroll
-                for (int p = 0; p < 4; ++p) {
-                    if (p < np) {
-                        const cpx<G> v = cell[p];
-                        acc[2 * p] += wt * v.x;
-                        acc[2 * p + 1] += wt * v.y;
-                    }
-                }
-            }
-#pragma unroll
-            for (int k = 0; k < 8; ++k)
-                if (k < 2 * np)   // np is the same on every lane
-                    for (int o = 16; o > 0; o >>= 1) acc[k] += __shfl_xor_sync(0xffffffffu, acc[k], o);
-            if (lane == 0) {
-#pragma unroll
-                for (int p = 0; p < 4; ++p)
-                    if (p < np)
-                        Vu[(size_t)(u0 + t) * np + p] =
-                            cmul(cmk<double>((double)acc[2 * p], (double)acc[2 * p + 1]), s_post[t]);
-            }
-        }
+        for (int j = 0; j < 4; ++j)
+            if (b[j] >= 0) o[(size_t)b[j] * NP + p] = cmk<G>(vx, vy);
     }
 }
 
@@ -792,41 +588,18 @@ __global__ void __launch_bounds__(256) k_interp_warp(const cpx<G> *__restrict__ 
     const int lane = threadIdx.x & 31;
     const long u = (long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
     if (u >= n_u) return;   // whole warps
+    // read early: the list of the target's baselines is needed last
+    const int b0 = so.out ? so.u_off[so.u_base + u] : 0, nb = so.out ? so.u_off[so.u_base + u + 1] - b0 : 0;
     const int w = g.w;
     const G two_over_w = (G)2 / (G)w, beta = geom_beta<G>(g);
     int m0 = 0, m1 = 0;
     G f0 = (G)0, f1 = (G)0, phr = (G)0;
     if (sizeof(G) == 4 && g.tgt_db) {
-        // FP32 set-up on every lane, no FP64: double-float products of the per-channel factors and the
-        // target's float pairs, then the first footprint cell m = ceil(p - w/2) and f = p - m brought into
-        // (w/2 - 1, w/2] (as the FP64 form), and the postphase reduced by 2 pi = 6.2831855 - 1.7484555e-7
-        const float4 db = g.tgt_db[u];
-        const float2 bc = g.tgt_bc[u];
-        const float hw = 0.5f * (float)w;
-        float mm[2], ff[2];
-#pragma unroll
-        for (int i = 0; i < 2; ++i) {
-            const float dh = i == 0 ? db.x : db.z, dl = i == 0 ? db.y : db.w;
-            float ph = g.a_hi[i] * dh;
-            float pl = fmaf(g.a_hi[i], dh, -ph) + (g.a_hi[i] * dl + g.a_lo[i] * dh);
-            ph = -ph;
-            pl = -pl;                                   // p = ph + pl
-            float m = ceilf(ph - hw);
-            float f = (ph - m) + pl;
-            if (f > hw) { m += 1.0f; f -= 1.0f; }
-            else if (f <= hw - 1.0f) { m -= 1.0f; f += 1.0f; }
-            mm[i] = m;
-            ff[i] = f;
-        }
-        m0 = (int)mm[0];
-        m1 = (int)mm[1];
-        f0 = (G)ff[0];
-        f1 = (G)ff[1];
-        float qh = g.kap_hi * bc.x;
-        const float ql = fmaf(g.kap_hi, bc.x, -qh) + (g.kap_hi * bc.y + g.kap_lo * bc.x);
-        qh = -qh;                                        // argument -kappa (b . C) = qh - ql
-        const float k = rintf(qh * 0.15915494f);
-        phr = (G)(fmaf(-k, -1.7484555e-7f, fmaf(-k, 6.2831855f, qh)) - ql);
+        float a0, a1, ap, bup;
+        target_setup(g, u, m0, m1, a0, a1, ap, bup);
+        f0 = (G)a0;
+        f1 = (G)a1;
+        phr = (G)ap;
     } else if (lane == 0) {
         // FP64 set-up on lane 0
         double ph = 0.0;
@@ -940,20 +713,7 @@ __global__ void __launch_bounds__(256) k_interp_warp(const cpx<G> *__restrict__ 
                 }
             }
         }
-        const int gu = so.u_base + (int)u;
-        const int b0 = so.u_off[gu], nb = so.u_off[gu + 1] - b0;
-        cpx<G> *o = reinterpret_cast<cpx<G> *>(so.out);
-        for (int k = lane; k < nb * NP; k += 32) {
-            const int kb = NP == 1 ? k : k >> 2, p = NP == 1 ? 0 : k & 3;
-            G vx = rx[0], vy = ry[0];
-#pragma unroll
-            for (int q = 1; q < NP; ++q)
-                if (p == q) {
-                    vx = rx[q];
-                    vy = ry[q];
-                }
-            o[(size_t)so.u_bl[b0 + kb] * NP + p] = cmk<G>(vx, vy);
-        }
+        write_target<G, NP>(so, b0, nb, rx, ry, lane);
         return;
     }
     if (NP == 1) {
@@ -985,15 +745,131 @@ __global__ void __launch_bounds__(256) k_interp_warp(const cpx<G> *__restrict__ 
     }
 }
 
-static bool zrow_fits(const SliceGeom &g, int elem_bytes)
+// Interpolation of FP32 bands that hold several planes per cell (height terms, or a short up axis summed directly):
+// one warp per target, the band [b_y][b_x][P], P = n_pol nz even.  A footprint row is w P consecutive complex
+// values; lane L holds pairs L, L + 32, ... (R of them) of that run for every row, so a row costs R 16-byte loads
+// and 2 R packed FMAs a lane with the row's y weight alone, and the x weight, the target's weight of the value's
+// plane (height_weight, or the direct sum K(l_z)) and the sum over the lanes come once per target.  The set-up needs
+// no FP64 (tgt_db, tgt_bc); the result is written to the target's baselines (no scatter).  Measured on the
+// 127-antenna workload (8,001 targets, 8 terms): 28.7 us and 6.3 us of scatter before.
+// R: pairs a lane; NP: products; W: largest kernel width.
+template <int NP, int R, int W>
+__global__ void __launch_bounds__(128) k_interp_planes(const cpx<float> *__restrict__ band,
+                                                       const double *__restrict__ bu, int n_u,
+                                                       const double *__restrict__ dec, SliceGeom g,
+                                                       const float *__restrict__ prez,
+                                                       const cpx<float> *__restrict__ twz, SliceOut so)
 {
-    if (elem_bytes != 4 || (g.d != 3 && g.K == 0) || g.n_pol != 1) return false;
-    const int Nz = g.dim[2].nf1;
-    return Nz >= 2 && Nz % 2 == 0 && g.w * (Nz / 2) <= 32;
+    const int lane = threadIdx.x & 31;
+    const int u = (int)(blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5));
+    if (u >= n_u) return;                       // whole warps
+    const int gu = so.u_base + u;
+    const int b0 = so.u_off[gu], nb = so.u_off[gu + 1] - b0;
+    const float dd = (float)dec[u];
+    const int w = g.w, nz = g.dim[2].nf1, P = NP * nz;
+    int m0, m1;
+    float f0, f1, phr, b_up;
+    target_setup(g, u, m0, m1, f0, f1, phr, b_up);
+    const float two_over_w = 2.0f / (float)w, beta = g.beta_f;
+    // this lane's pairs: their cell's column and planes
+    const int pairs = w * P / 2;
+    const cpx<float> *col = band + ((size_t)(m1 + g.dim[1].H) * g.dim[0].B + (m0 + g.dim[0].H)) * P;
+    const size_t rstride = (size_t)g.dim[0].B * P;
+    float2 acc[R][2];
+#pragma unroll
+    for (int r = 0; r < R; ++r) acc[r][0] = acc[r][1] = make_float2(0.0f, 0.0f);
+    const float wyl = lane < w ? es_kernel(two_over_w * (f1 - (float)lane), beta) : 0.0f;
+#pragma unroll
+    for (int y = 0; y < W; ++y) {
+        if (y < w) {
+            const float wy = __shfl_sync(0xffffffffu, wyl, y);
+            const float2 wy2 = make_float2(wy, wy);
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                const int v = lane + 32 * r;
+                if (v < pairs) {
+                    const float4 t = __ldg(reinterpret_cast<const float4 *>(col + y * rstride) + v);
+                    acc[r][0] = __ffma2_rn(wy2, make_float2(t.x, t.y), acc[r][0]);
+                    acc[r][1] = __ffma2_rn(wy2, make_float2(t.z, t.w), acc[r][1]);
+                }
+            }
+        }
+    }
+    // the target's weight of plane lane (< nz)
+    cpx<float> Kmine = cmk<float>(0.0f, 0.0f);
+    if (g.K) {
+        if (lane < nz) Kmine = height_bessel(g, b_up, lane);
+    } else {
+        // up planes: K(l_z) = sum_m phi((2/w)(p_z - m)) e^{2 pi i l_z m / M_z}, the z prescale folded in
+        const double x2 = -g.kappa * bu[3 * (size_t)u + 2];
+        const double pp = (x2 - g.dim[2].D) * g.dim[2].pscale;
+        const double md = ceil(pp - 0.5 * w);
+        const float fz = (float)(pp - md);
+        if (lane < nz) {
+            const int Mz = g.dim[2].M, lc = lane - nz / 2;
+            int e = (lc * (int)md) % Mz;
+            if (e < 0) e += Mz;
+            int step = lc % Mz;
+            if (step < 0) step += Mz;
+            for (int j = 0; j < w; ++j) {
+                Kmine = cadd(Kmine, cscale(twz[e], es_kernel(two_over_w * (fz - (float)j), beta)));
+                e += step;
+                if (e >= Mz) e -= Mz;
+            }
+            Kmine = cscale(Kmine, prez[lane]);
+        }
+    }
+    const float wxl = lane < w ? es_kernel(two_over_w * (f0 - (float)lane), beta) : 0.0f;
+    float sx[NP], sy[NP];
+#pragma unroll
+    for (int p = 0; p < NP; ++p) sx[p] = sy[p] = 0.0f;
+    const unsigned inv_P = 65536u / (unsigned)P + 1u, inv_nz = 65536u / (unsigned)nz + 1u;   // exact below 512
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int v = 2 * (lane + 32 * r) + h;          // value of the row: cell v / P, plane v % P
+            const int c = (int)(((unsigned)v * inv_P) >> 16), pl = v - c * P;
+            const int pol = NP == 1 ? 0 : (int)(((unsigned)pl * inv_nz) >> 16), z = pl - pol * nz;
+            const float kx = __shfl_sync(0xffffffffu, Kmine.x, z), ky = __shfl_sync(0xffffffffu, Kmine.y, z);
+            const float wx = __shfl_sync(0xffffffffu, wxl, c);           // zero past the row (c >= w)
+            const float ax = acc[r][h].x * wx, ay = acc[r][h].y * wx;
+            const float rx = ax * kx - ay * ky, ry = ax * ky + ay * kx;
+#pragma unroll
+            for (int p = 0; p < NP; ++p)
+                if (NP == 1 || pol == p) {
+                    sx[p] += rx;
+                    sy[p] += ry;
+                }
+        }
+    }
+    float sp, cp;
+    sincosf(phr, &sp, &cp);
+    float vx[NP], vy[NP];
+#pragma unroll
+    for (int p = 0; p < NP; ++p) {
+        for (int o = 16; o > 0; o >>= 1) {
+            sx[p] += __shfl_xor_sync(0xffffffffu, sx[p], o);
+            sy[p] += __shfl_xor_sync(0xffffffffu, sy[p], o);
+        }
+        vx[p] = (sx[p] * cp - sy[p] * sp) * dd;
+        vy[p] = (sx[p] * sp + sy[p] * cp) * dd;
+    }
+    write_target<float, NP>(so, b0, nb, vx, vy, lane);
 }
 
-bool interp_fuses_scatter(const SliceGeom &g)
+// k_interp_planes: pairs of planes, at most four (one product) or five (four products, w <= 8) pairs a lane
+static bool planes_fit(const SliceGeom &g, int elem_bytes)
 {
+    if (elem_bytes != 4 || (g.d != 3 && g.K == 0) || (g.n_pol != 1 && g.n_pol != 4)) return false;
+    if (g.w > (g.n_pol == 1 ? 16 : 8)) return false;
+    const int P = g.n_pol * g.dim[2].nf1;
+    return g.dim[2].nf1 <= 16 && P % 2 == 0 && g.w * P / 2 <= 160;
+}
+
+bool interp_fuses_scatter(const SliceGeom &g, int elem_bytes)
+{
+    if (planes_fit(g, elem_bytes)) return true;
     return g.w <= kIbMaxW && g.d == 2 && g.K == 0 && (g.n_pol == 1 || g.n_pol == 4);
 }
 
@@ -1002,12 +878,11 @@ cudaError_t launch_interp_zdirect(const cpx<G> *band, const double *bu, int n_u,
                                   const SliceGeom &g, const G *prez, const cpx<G> *twz, cpx<double> *Vu,
                                   cudaStream_t st, const SliceOut *so)
 {
-    if (so && so->out && !interp_fuses_scatter(g)) return cudaErrorInvalidValue;
+    if (so && so->out && !interp_fuses_scatter(g, (int)sizeof(G))) return cudaErrorInvalidValue;
     const SliceOut sov = so ? *so : SliceOut{nullptr, nullptr, nullptr, 0};
     if (n_u <= 0) return cudaSuccess;
     if ((g.d == 3 || g.K) && g.dim[2].nf1 > 16) return cudaErrorInvalidValue;
     long threads = (long)n_u * 32;
-    const unsigned ib_blocks = (unsigned)((n_u + kIbTargets - 1) / kIbTargets);
     if (g.w <= kIbMaxW) {
         if (g.d == 2 && g.K == 0) {
             // one warp per target, 8 per CTA
@@ -1019,13 +894,26 @@ cudaError_t launch_interp_zdirect(const cpx<G> *band, const double *bu, int n_u,
             return cudaGetLastError();
         }
         if constexpr (sizeof(G) == 4) {
-            if (zrow_fits(g, 4) && g.dim[2].nf1 <= 8) {
-                k_interp_batch<G, true><<<ib_blocks, kIbThreads, 0, st>>>(band, bu, n_u, dec, g, prez, twz, Vu);
-                return cudaGetLastError();
-            }
-            if (zrow_fits(g, 4)) {
-                k_interp_zrow<<<(unsigned)((threads + 255) / 256), 256, 0, st>>>(band, bu, n_u, dec, g, prez, twz,
-                                                                                Vu);
+            if (sov.out && g.tgt_db && planes_fit(g, 4)) {
+                const unsigned pb = (unsigned)((n_u + 3) / 4);
+                const int R = (g.w * g.n_pol * g.dim[2].nf1 / 2 + 31) / 32;
+#define FV_PLANES(NP, R, W) k_interp_planes<NP, R, W><<<pb, 128, 0, st>>>(band, bu, n_u, dec, g, prez, twz, sov)
+                if (g.n_pol == 1 && g.w <= 8) {
+                    if (R == 1) FV_PLANES(1, 1, 8);
+                    else FV_PLANES(1, 2, 8);            // nz <= 16: at most 64 pairs
+                } else if (g.n_pol == 1) {
+                    if (R <= 2) FV_PLANES(1, 2, 16);
+                    else FV_PLANES(1, 4, 16);           // at most 128 pairs
+                } else {
+                    switch (R) {
+                    case 1: FV_PLANES(4, 1, 8); break;
+                    case 2: FV_PLANES(4, 2, 8); break;
+                    case 3: FV_PLANES(4, 3, 8); break;
+                    case 4: FV_PLANES(4, 4, 8); break;
+                    default: FV_PLANES(4, 5, 8); break;
+                    }
+                }
+#undef FV_PLANES
                 return cudaGetLastError();
             }
         }

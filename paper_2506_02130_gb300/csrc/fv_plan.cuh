@@ -64,10 +64,10 @@ struct fv_plan_s {
     double *d_bu = nullptr, *d_dec = nullptr;
     // per unique target, float pairs for the FP32 interpolation set-up (SliceGeom::tgt_db, tgt_bc)
     float4 *d_tgt_db = nullptr;
-    float2 *d_tgt_bc = nullptr;
+    float4 *d_tgt_bc = nullptr;
     int tgt_n = 0;
     std::vector<float4> h_tgt_db;
-    std::vector<float2> h_tgt_bc;
+    std::vector<float4> h_tgt_bc;
     int *d_bl2u = nullptr;
     // unique target -> its baselines (CSR: d_u_off[n_u + 1] into d_u_bl[n_bl]), for the interpolation
     // that writes a slice's output itself

@@ -538,6 +538,7 @@ static fv_status prepare(fv_plan_s *p)
         g.hc = p->C[2];
         g.hs = p->S[2] > 0.0 ? p->S[2] : 1.0;
         g.hc_f = (float)g.hc;
+        g.hs_f = (float)g.hs;
         g.hs_inv_f = (float)(1.0 / g.hs);
         for (int i = 0; i < 3; ++i) {
             DimGeom &dg = g.dim[i];
@@ -604,7 +605,7 @@ static fv_status prepare(fv_plan_s *p)
             dfree_t(p->d_tgt_db);
             dfree_t(p->d_tgt_bc);
             CK(cudaMalloc(&p->d_tgt_db, (size_t)p->n_u * sizeof(float4)));
-            CK(cudaMalloc(&p->d_tgt_bc, (size_t)p->n_u * sizeof(float2)));
+            CK(cudaMalloc(&p->d_tgt_bc, (size_t)p->n_u * sizeof(float4)));
             p->tgt_n = p->n_u;
         }
         p->h_tgt_db.resize(p->n_u);
@@ -620,11 +621,14 @@ static fv_status prepare(fv_plan_s *p)
             pair(b[1] - p->bcen[1], t.z, t.w);
             double bc = 0.0;
             for (int i = 0; i < p->d; ++i) bc += b[i] * p->C[i];
+            if (p->hK > 0) bc += b[2] * p->C[2];            // hc: the height terms' phase
             pair(bc, p->h_tgt_bc[u].x, p->h_tgt_bc[u].y);
+            p->h_tgt_bc[u].z = (float)b[2];
+            p->h_tgt_bc[u].w = 0.0f;
         }
         CK(cudaMemcpyAsync(p->d_tgt_db, p->h_tgt_db.data(), (size_t)p->n_u * sizeof(float4), cudaMemcpyHostToDevice,
                            p->stream));
-        CK(cudaMemcpyAsync(p->d_tgt_bc, p->h_tgt_bc.data(), (size_t)p->n_u * sizeof(float2), cudaMemcpyHostToDevice,
+        CK(cudaMemcpyAsync(p->d_tgt_bc, p->h_tgt_bc.data(), (size_t)p->n_u * sizeof(float4), cudaMemcpyHostToDevice,
                            p->stream));
     }
     const bool reuse = p->d_pre != nullptr && sig == p->geo_sig;
@@ -855,8 +859,9 @@ fv_status run_slices(fv_plan_s *p, fv_plan_s::Workspace &wk, cudaStream_t st, ch
         }
         const int ntm = om.nt > 0 ? om.nt : nt;
         char *out = vis + ((size_t)(f - om.f0) * ntm + (t - om.t0)) * slice_bytes;
-        // two-dimensional grids: the interpolation writes the baselines' output itself (no scatter)
-        const bool fused = p->d == 2 && p->hK == 0 && p->d_u_off && interp_fuses_scatter(p->gf[f]);
+        // the interpolation writes the baselines' output itself (no scatter) where its kernel can
+        const bool fused = p->d_u_off && p->tgt_n == p->n_u && (p->d == 2 || p->gf[f].dim[2].nf1 <= FV_ZDIRECT_MAX) &&
+                           interp_fuses_scatter(p->gf[f], (int)sizeof(G));
         // one transform per beam group: strengths with the group's two beams, targets [u0, u1)
         for (const auto &gr : p->groups) {
             if (gr.u1 <= gr.u0) continue;

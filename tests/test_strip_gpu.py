@@ -86,3 +86,19 @@ def test_fft_lengths_against_the_general_passes(scale):
     out, info = _run(prob, 1e-6)
     ref, _ = _run(prob, 1e-6, fft_max_radix=8)
     assert rel_l2(out, ref) <= 1e-5, info["nf2_max"]
+
+
+@pytest.mark.parametrize("z_sigma,polarised,kw", [(0.05, False, dict(heights="terms")), (0.02, True, dict(heights="terms")),
+                                                 (0.1, False, dict(heights="grid")), (0.02, True, dict(heights="grid")),
+                                                 (0.02, False, dict(heights="terms", kernel_width=11)),
+                                                 (0.05, False, dict(heights="grid", kernel_width=14))])
+def test_plane_interpolation_writes_every_copy_of_a_baseline(z_sigma, polarised, kw):
+    """Antennas in pairs of equal offset, so that targets have several baselines, with planes to sum."""
+    prob = _prob(900, polarised, radius=2, z_sigma=z_sigma)
+    n = len(prob.ant_enu)
+    prob.ant_enu = np.concatenate([prob.ant_enu, prob.ant_enu + [512.0, 256.0, 0.0]]) * [0.25, 0.25, 1.0]
+    prob.ant_enu = np.round(prob.ant_enu * 1024) / 1024          # exact differences
+    prob.pairs = W.cross_pairs(2 * n)
+    out, info = _run(prob, 1e-6, **kw)
+    assert info["n_unique"] < info["n_bl"]
+    assert rel_l2(out, oracle_vis(OracleProblem.from_workload(prob), "factored")) <= 2e-5
