@@ -66,7 +66,8 @@ static bool covers(const fv_plan_s::WsNeed &have, const fv_plan_s::WsNeed &need)
     return have.grid >= need.grid && have.bufA >= need.bufA && have.bufB >= need.bufB && have.vu >= need.vu &&
            (!need.tiled || (have.tiled && have.n_src >= need.n_src && have.nb >= need.nb &&
                             have.frac_per_src >= need.frac_per_src && have.cs_per_src >= need.cs_per_src &&
-                            (have.tc || !need.tc) && have.ring_tiles >= need.ring_tiles &&
+                            (have.tc || !need.tc) && (have.rec || !need.rec) && (have.dirs || !need.dirs) &&
+                            have.ring_tiles >= need.ring_tiles &&
                             have.ring_slots >= need.ring_slots && have.ring_np >= need.ring_np));
 }
 
@@ -184,7 +185,14 @@ static fv_status add_items(fv_batch_t b, fv_plan_t p, void *vis, int t_lo, int t
                                     slice_bytes, b->stream));
         return FV_OK;
     }
-    const double per_slice = (double)(p->need.grid + p->need.bufA + p->need.bufB) + 64.0 * p->n_src;
+    // bytes of grid and bands as the measure of a slice's work; direct mode sums by their multiply-adds (a tenth of a
+    // byte each by the slices' times, pairs of floats in FP64 eight times that)
+    const double per_slice =
+        64.0 * p->n_src +
+        (p->use_lattice && p->lat_dense
+             ? 0.1 * p->n_src * (double)(2 * p->dense.H1 + 1) * (p->dense.H2 + 1) * (p->dense.J + 2) *
+                   (p->precision == FV_FP64 ? 8.0 : 1.0)
+             : (double)(p->need.grid + p->need.bufA + p->need.bufB));
     for (int t = t_lo; t < t_hi; ++t) {
         fv_batch_s::Item it{p, (char *)vis, (long)t * nf + f_lo, (long)t * nf + f_hi, per_slice * (f_hi - f_lo), om,
                             p->gen};
@@ -231,6 +239,7 @@ fv_status fv_batch_execute(fv_batch_t b, int use_graph)
         }
     }
     fv_plan_s::WsNeed need;
+    need.dirs = false;
     for (const auto &it : b->items) {
         const auto &n = it.p->need;
         need.grid = std::max(need.grid, n.grid);
@@ -244,6 +253,8 @@ fv_status fv_batch_execute(fv_batch_t b, int use_graph)
             need.frac_per_src = std::max(need.frac_per_src, n.frac_per_src);
             need.cs_per_src = std::max(need.cs_per_src, n.cs_per_src);
             need.tc = need.tc || n.tc;
+            need.rec = need.rec || n.rec;
+            need.dirs = need.dirs || n.dirs;
             need.ring_tiles = std::max(need.ring_tiles, n.ring_tiles);
             need.ring_slots = std::max(need.ring_slots, n.ring_slots);
             need.ring_np = std::max(need.ring_np, n.ring_np);

@@ -84,6 +84,7 @@ struct TimeBin {
     int nf1_top[3];
     int T[2];               // tile (= bin) size in cells
     int nbx, nby;           // bins per axis
+    double a[2][2];         // lattice vectors (launch_time_compact's records)
     int strips;             // bin order: 0 row by row (x fastest), 1 strip by strip (y fastest)
 };
 
@@ -463,6 +464,13 @@ inline size_t bin_count_ints(int nb) { return (size_t)nb + (nb + kScanBlock - 1)
 // tc[3i] = {qx_hi, qx_lo, qy_hi, qy_lo}, tc[3i+1] = {qz_hi, qz_lo, ph_hi, ph_lo}, tc[3i+2] = {s0, s1, s2, 0}.
 cudaError_t launch_time_binning(const double *e, long n_src, const TimeBin &tb, int *bin_of, int *counts,
                                 int *offsets, int *cursor, double *sdir, int *sidx, float4 *tc, cudaStream_t st);
+
+// Per time, without bins: the sources above the horizon in their own order (sdir, sidx); offsets[time_compact_blocks]
+// is their number.  counts, offsets and cursor as for that many bins.
+// tc (nullable): in sdir's place {a_1 . s (hi, lo), a_2 . s (hi, lo)} and {s, 2 s_up - 1} per source (TimeBin::a).
+int time_compact_blocks(long n_src);
+cudaError_t launch_time_compact(const double *e, long n_src, const TimeBin &tb, int *counts, int *offsets, int *cursor,
+                                double *sdir, int *sidx, float4 *tc, cudaStream_t st);
 
 // Per slice: strengths with prephase and split grid coordinates of the sorted sources.
 template <class G>

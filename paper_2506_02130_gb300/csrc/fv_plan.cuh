@@ -3,6 +3,7 @@
 #pragma once
 #include "../../include/fv.h"
 #include "fv_internal.cuh"
+#include "fv_lattice_dense.cuh"
 
 #include <string>
 #include <utility>
@@ -109,6 +110,7 @@ struct fv_plan_s {
         int *cell = nullptr;
         double *sdir = nullptr;
         void *frac = nullptr, *cs = nullptr;
+        float4 *rec = nullptr;    // per-time records of the direct mode sums (launch_time_compact)
         float4 *tc = nullptr;     // per-time coordinate records of the sorted sources (FP32 grids)
         int *tiles = nullptr;     // ring gather: ticket and work-list counts (reset by the prep kernel)
         // ring gather work list (fv_spread_ring.cu): tiles' bin rectangles, unsplit tiles, parts of split
@@ -127,6 +129,8 @@ struct fv_plan_s {
         size_t frac_per_src = 0, cs_per_src = 0;       // bytes per source
         bool tiled = false;
         bool tc = false;                               // per-time coordinate records (48 bytes per source)
+        bool rec = false;                              // direct mode sums in FP32: their records (32 bytes per source)
+        bool dirs = true;                              //   in place of directions and cells
         int ring_tiles = 0, ring_slots = 0, ring_np = 0; // ring gather: tiles of the largest grid, part slots, n_pol
     } need;
     int n_streams = 1;
@@ -155,6 +159,12 @@ struct fv_plan_s {
     double lat_basis[4] = {0, 0, 0, 0};
     int lat_H[2] = {0, 0};
     int *d_bln = nullptr;             // [n_bl][2] lattice offsets n of the baselines
+    std::vector<int> lat_bln;         //   the same on the host
+    bool lat_dense = false;           // direct mode sums instead of the type-1 transform (fv_lattice_dense.cu)
+    fv::DenseGeom dense{};
+    int dense_ch = 1;                 //   channels one launch takes
+    int *d_lat_tiles = nullptr;       //   mode tiles in use
+    double *d_lat_freq = nullptr;     //   [n_freq] Hz
     fv::LatGeom lg{};
     fv::DimGeom lat_dim[2]{};         // FFT geometry of the two passes
     void *d_lat_pre = nullptr, *d_lat_tw = nullptr;   // ones (prescale) and twiddles per axis

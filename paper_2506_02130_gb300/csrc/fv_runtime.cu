@@ -169,8 +169,9 @@ size_t workspace_layout(const fv_plan_s::WsNeed &need, char *base, fv_plan_s::Wo
         o.offsets = (int *)take((nb + 1) * sizeof(int));
         o.cursor = (int *)take(nb * sizeof(int));
         o.sidx = (int *)take(ns * sizeof(int));
-        o.cell = (int *)take(3 * ns * sizeof(int));
-        o.sdir = (double *)take(3 * ns * sizeof(double));
+        o.cell = need.dirs ? (int *)take(3 * ns * sizeof(int)) : nullptr;
+        o.sdir = need.dirs ? (double *)take(3 * ns * sizeof(double)) : nullptr;
+        o.rec = need.rec ? (float4 *)take(ns * 2 * sizeof(float4)) : nullptr;
         // 64 bytes of slack: the band spreader's bulk copies round their ends up to 16 bytes
         o.frac = take(ns * need.frac_per_src + 64);
         o.cs = take(ns * need.cs_per_src + 64);
@@ -227,6 +228,8 @@ static void free_geometry(fv_plan_s *p)
     dfree_t(p->d_lat_dec);
     dfree_t(p->d_lat_bup);
     dfree_t(p->d_lat_wq);
+    dfree_t(p->d_lat_tiles);
+    dfree_t(p->d_lat_freq);
     dfree_t(p->d_bas_M);
     dfree_t(p->d_bas_d);
     dfree_t(p->d_bas_freq);
@@ -359,24 +362,40 @@ static fv_status prepare_lattice(fv_plan_s *p)
     dfree(p->d_lat_pre);
     dfree(p->d_lat_tw);
     dfree_t(p->d_lat_dec);
-    const size_t npre = (size_t)lg.nf[0] + lg.nf[1];
-    CK(cudaMalloc(&p->d_lat_pre, npre * gs));
-    CK(cudaMalloc(&p->d_lat_tw, npre * es));
-    CK(cudaMalloc(&p->d_lat_dec, (size_t)(2 * lg.H[0] + 1 + 2 * lg.H[1] + 1) * sizeof(double)));
-    if (p->precision == FV_FP64) {
-        std::vector<double> ones(npre, 1.0);
-        CK(cudaMemcpyAsync(p->d_lat_pre, ones.data(), npre * gs, cudaMemcpyHostToDevice, p->stream));
-        CK(launch_twiddles<double>((cpx<double> *)p->d_lat_tw, lg.nf[0], p->stream));
-        CK(launch_twiddles<double>((cpx<double> *)p->d_lat_tw + lg.nf[0], lg.nf[1], p->stream));
-    } else {
-        std::vector<float> ones(npre, 1.0f);
-        CK(cudaMemcpyAsync(p->d_lat_pre, ones.data(), npre * gs, cudaMemcpyHostToDevice, p->stream));
-        CK(launch_twiddles<float>((cpx<float> *)p->d_lat_tw, lg.nf[0], p->stream));
-        CK(launch_twiddles<float>((cpx<float> *)p->d_lat_tw + lg.nf[0], lg.nf[1], p->stream));
+    // the mode sums directly where the lattice is small enough (fv_lattice_dense.cu), else the type-1 transform
+    std::vector<int> tiles;
+    p->lat_dense = dense_plan((int)gs, p->eps, K, p->n_pol, lg.H[0], lg.H[1], p->n_bl, p->lat_bln.data(), p->dense, tiles);
+    dfree_t(p->d_lat_tiles);
+    dfree_t(p->d_lat_freq);
+    if (p->lat_dense) {
+        std::memcpy(p->dense.a, lg.a, sizeof(lg.a));
+        CK(cudaMalloc(&p->d_lat_tiles, tiles.size() * sizeof(int)));
+        CK(cudaMalloc(&p->d_lat_freq, p->freq.size() * sizeof(double)));
+        CK(cudaMemcpy(p->d_lat_tiles, tiles.data(), tiles.size() * sizeof(int), cudaMemcpyHostToDevice));
+        CK(cudaMemcpyAsync(p->d_lat_freq, p->freq.data(), p->freq.size() * sizeof(double), cudaMemcpyHostToDevice,
+                           p->stream));
+        p->dense.tiles = p->d_lat_tiles;
     }
-    CK(launch_lattice_deconv(p->d_lat_dec, lg.H[0], lg.nf[0], w, p->beta, p->d_glx, p->d_glw, p->nq, p->stream));
-    CK(launch_lattice_deconv(p->d_lat_dec + 2 * lg.H[0] + 1, lg.H[1], lg.nf[1], w, p->beta, p->d_glx, p->d_glw,
-                             p->nq, p->stream));
+    const size_t npre = (size_t)lg.nf[0] + lg.nf[1];
+    if (!p->lat_dense) {
+        CK(cudaMalloc(&p->d_lat_pre, npre * gs));
+        CK(cudaMalloc(&p->d_lat_tw, npre * es));
+        CK(cudaMalloc(&p->d_lat_dec, (size_t)(2 * lg.H[0] + 1 + 2 * lg.H[1] + 1) * sizeof(double)));
+        if (p->precision == FV_FP64) {
+            std::vector<double> ones(npre, 1.0);
+            CK(cudaMemcpyAsync(p->d_lat_pre, ones.data(), npre * gs, cudaMemcpyHostToDevice, p->stream));
+            CK(launch_twiddles<double>((cpx<double> *)p->d_lat_tw, lg.nf[0], p->stream));
+            CK(launch_twiddles<double>((cpx<double> *)p->d_lat_tw + lg.nf[0], lg.nf[1], p->stream));
+        } else {
+            std::vector<float> ones(npre, 1.0f);
+            CK(cudaMemcpyAsync(p->d_lat_pre, ones.data(), npre * gs, cudaMemcpyHostToDevice, p->stream));
+            CK(launch_twiddles<float>((cpx<float> *)p->d_lat_tw, lg.nf[0], p->stream));
+            CK(launch_twiddles<float>((cpx<float> *)p->d_lat_tw + lg.nf[0], lg.nf[1], p->stream));
+        }
+        CK(launch_lattice_deconv(p->d_lat_dec, lg.H[0], lg.nf[0], w, p->beta, p->d_glx, p->d_glw, p->nq, p->stream));
+        CK(launch_lattice_deconv(p->d_lat_dec + 2 * lg.H[0] + 1, lg.H[1], lg.nf[1], w, p->beta, p->d_glx, p->d_glw,
+                                 p->nq, p->stream));
+    }
     dfree_t(p->d_lat_bup);
     dfree_t(p->d_lat_wq);
     if (K > 1 && p->n_bl > 0) {
@@ -389,21 +408,32 @@ static fv_status prepare_lattice(fv_plan_s *p)
             CK(launch_lattice_wterms(p->d_lat_bup, p->n_bl, K, 2.0 * M_PI * p->freq[f] / FV_C_LIGHT,
                                      p->d_lat_wq + (size_t)f * p->n_bl * K, p->stream));
     }
-    // workspace of one lattice slice: grid, the two bands, one-bin time binning, prepared sources
+    // workspace of one lattice slice: grid, the two bands, one-bin time binning, prepared sources; or the mode sums
+    // of the channels that one launch takes
     fv_plan_s::WsNeed nd;
     const int np = p->n_pol;
-    nd.grid = (size_t)K * np * lg.nf[0] * lg.nf[1] * es;
-    nd.bufA = (size_t)(2 * lg.H[0] + 1) * K * np * lg.nf[1] * es;
-    nd.bufB = (size_t)(2 * lg.H[1] + 1) * (2 * lg.H[0] + 1) * K * np * es;
     nd.vu = sizeof(cpx<double>);
     nd.tiled = true;
     nd.n_src = std::max<long>(p->n_src, 1);
-    nd.nb = 1;
-    nd.frac_per_src = (3 + 2 * (size_t)w) * gs;     // fx, fy, u and the 2w kernel values
+    nd.nb = time_compact_blocks(p->n_src);
+    nd.grid = (size_t)K * np * lg.nf[0] * lg.nf[1] * es;
+    nd.bufA = (size_t)(2 * lg.H[0] + 1) * K * np * lg.nf[1] * es;
+    nd.bufB = (size_t)(2 * lg.H[1] + 1) * (2 * lg.H[0] + 1) * K * np * es;
+    nd.frac_per_src = (3 + 2 * (size_t)w) * gs;         // fx, fy, u and the 2w kernel values
     nd.cs_per_src = (size_t)np * es;
+    if (p->lat_dense) {
+        // at most what the type-1 transform would hold, so that the static scratch takes every plan it took with it
+        const size_t one = dense_modes(p->dense) * sizeof(cpx<double>);
+        const size_t most = nd.grid + nd.bufA + nd.bufB + (size_t)nd.n_src * (nd.frac_per_src + nd.cs_per_src);
+        p->dense_ch = (int)std::max<size_t>(1, std::min<size_t>({p->freq.size(), (size_t)64, most / one}));
+        nd.grid = one * p->dense_ch;
+        nd.bufA = nd.bufB = nd.frac_per_src = nd.cs_per_src = 0;
+        nd.rec = p->precision == FV_MIXED;
+        nd.dirs = !nd.rec;
+    }
     free_workspaces(p->ws);
     p->need = nd;
-    p->ws_bytes = (long long)(npre * (gs + es) + p->n_streams * workspace_layout(nd, nullptr, nullptr) +
+    p->ws_bytes = (long long)((p->lat_dense ? 0 : npre * (gs + es)) + p->n_streams * workspace_layout(nd, nullptr, nullptr) +
                               (K > 1 ? p->freq.size() * (size_t)p->n_bl * K * sizeof(cpx<double>) : 0));
     return FV_OK;
 }
@@ -747,23 +777,49 @@ static fv_status run_slices_lattice(fv_plan_s *p, fv_plan_s::Workspace &wk, cuda
     const size_t gel = (size_t)lg.K * np * lg.nf[0] * lg.nf[1];
     const int Bx = 2 * lg.H[0] + 1, By = 2 * lg.H[1] + 1;
     const double nvis = 0.5 * p->n_src;
+    const int *n_up = wk.offsets + time_compact_blocks(p->n_src);
+    float4 *tc = p->lat_dense && sizeof(G) == 4 ? wk.rec : nullptr;     // direct sums in FP32 read the time's records
     int t_binned = -1;
-    for (long k = k_begin; k < k_end; ++k) {
+    for (long k = k_begin, kn; k < k_end; k = kn) {
         const int t = (int)(k / nf), f = (int)(k % nf);
+        kn = k + 1;
         if (t != t_binned) {
             TimeBin tb{};
             std::memcpy(tb.R, &p->Rt[(size_t)t * 9], 9 * sizeof(double));
-            for (int i = 0; i < 3; ++i) tb.nf1_top[i] = 1;
-            tb.T[0] = tb.T[1] = 1;
-            tb.nbx = tb.nby = 1;
             CK(prof_begin(p, PC_BIN, st));
-            CK(launch_time_binning(p->d_e, p->n_src, tb, wk.bin_of, wk.counts, wk.offsets, wk.cursor, wk.sdir,
-                                   wk.sidx, nullptr, st));
+            std::memcpy(tb.a, lg.a, sizeof(tb.a));
+            CK(launch_time_compact(p->d_e, p->n_src, tb, wk.counts, wk.offsets, wk.cursor, wk.sdir, wk.sidx, tc, st));
             CK(prof_end(p, (double)p->n_src * 80.0));
             t_binned = t;
         }
         // one set of transforms per beam group (Section 2.2.3), evaluated at the group's baselines
         const bool single = p->groups.size() == 1;
+        if (p->lat_dense) {
+            // direct mode sums: as many channels of this time as one launch takes
+            const int ch = (int)std::min<long>({k_end - k, (long)(nf - f), (long)p->dense_ch});
+            kn = k + ch;
+            const int ntm = om.nt > 0 ? om.nt : nt;
+            char *out = vis + ((size_t)(f - om.f0) * ntm + (t - om.t0)) * slice_bytes;
+            for (const auto &gr : p->groups) {
+                const int nbl = gr.bl1 - gr.bl0;
+                if (nbl <= 0) continue;
+                const SliceGeom g = slice_geom_for(p, f, t, gr);
+                CK(prof_begin(p, PC_SPREAD, st));
+                CK(launch_lattice_dense<G>(wk.sdir, tc, wk.sidx, n_up, p->n_src, p->flux, p->flux_fp64, nf, f, ch,
+                                           p->d_lat_freq, g, p->dense, (cpx<double> *)wk.grid, st));
+                CK(prof_end(p, ch * (nvis * (28.0 + p->n_stokes * (p->flux_fp64 ? 8.0 : 4.0)) + dense_modes(p->dense) * 16.0)));
+                CK(prof_begin(p, PC_INTERP, st));
+                CK(launch_dense_gather<G>((const cpx<double> *)wk.grid, p->d_bln, single ? nullptr : p->d_grp_bl + gr.bl0, nbl, p->n_bl, np,
+                                          p->dense, f, ch, p->d_lat_wq, out, (long)(ntm * slice_bytes), st));
+                CK(prof_end(p, ch * ((double)nbl * (8.0 + (p->d_lat_wq ? 16.0 * lg.K : 0.0)) + dense_modes(p->dense) * 16.0 +
+                                     (double)slice_bytes * nbl / std::max(p->n_bl, 1))));
+            }
+            for (int c = 0; om.host && c < ch; ++c) {
+                const size_t off = (out - vis) + (size_t)c * ntm * slice_bytes;
+                CK(cudaMemcpyAsync(om.host + off, vis + off, slice_bytes, cudaMemcpyDeviceToHost, st));
+            }
+            continue;
+        }
         for (const auto &gr : p->groups) {
             const int nbl = gr.bl1 - gr.bl0;
             if (nbl <= 0) continue;
@@ -771,7 +827,7 @@ static fv_status run_slices_lattice(fv_plan_s *p, fv_plan_s::Workspace &wk, cuda
             G *frac = (G *)wk.frac;
             cpx<G> *cs = (cpx<G> *)wk.cs;
             CK(prof_begin(p, PC_PREP, st));
-            CK(launch_prep_lattice<G>(wk.sdir, wk.sidx, wk.offsets + 1, p->n_src, p->flux, p->flux_fp64, nf, f, g, lg,
+            CK(launch_prep_lattice<G>(wk.sdir, wk.sidx, n_up, p->n_src, p->flux, p->flux_fp64, nf, f, g, lg,
                                       wk.cell, frac, cs, st));
             CK(prof_end(p, nvis * (24.0 + 4.0 + p->n_stokes * (p->flux_fp64 ? 8.0 : 4.0) + 8.0 + 2.0 * sizeof(G) +
                                    np * es)));
@@ -779,7 +835,7 @@ static fv_status run_slices_lattice(fv_plan_s *p, fv_plan_s::Workspace &wk, cuda
             CK(cudaMemsetAsync(grid, 0, gel * sizeof(cpx<G>), st));
             CK(prof_end(p, gel * es));
             CK(prof_begin(p, PC_SPREAD, st));
-            CK(launch_spread_lattice<G>(wk.offsets + 1, wk.cell, frac, cs, p->n_src, g, lg, grid, st));
+            CK(launch_spread_lattice<G>(n_up, wk.cell, frac, cs, p->n_src, g, lg, grid, st));
             CK(prof_end(p, nvis * (8.0 + 3.0 * sizeof(G) + np * es) + gel * es));
             const long r1 = (long)lg.K * np * lg.nf[1];
             CK(prof_begin(p, PC_FFT_X, st));
@@ -1677,6 +1733,7 @@ static fv_status setup_array(fv_plan_s *p)
         return p->fail(FV_ERR_UNSUPPORTED, "transform = FV_TRANSFORM_LATTICE, but the antennas' horizontal "
                                            "positions are not a lattice within lattice_tol_m");
     if (!lat_ok) p->lat_bup.clear();
+    p->lat_bln = bln;
     p->lat_ok = lat_ok;        // reported whatever the route; the lattice route also needs transform != TYPE3
                                // and dims != 3
     std::memcpy(p->lat_basis, lat_basis, sizeof(lat_basis));

@@ -25,6 +25,7 @@
 #include "fv_internal.cuh"
 #include "fv_prep.cuh"
 
+#include <algorithm>
 #include <math.h>
 
 namespace fv {
@@ -172,6 +173,68 @@ __global__ void k_bin_scatter(const double *__restrict__ e, long n_src, TimeBin 
         tc[3 * (size_t)pos + 1] = make_float4(qz.x, qz.y, pp.x, pp.y);
         tc[3 * (size_t)pos + 2] = make_float4((float)s[0], (float)s[1], (float)s[2], 0.0f);
     }
+}
+
+// The sources above the horizon in their own order (no bins): counts per block of 256 sources, the scan of the
+// blocks and a ranked copy.  The order, and with it the sums over the sources, is the same every time.
+constexpr int kCompact = 256;
+__global__ void __launch_bounds__(kCompact) k_compact_count(const double *__restrict__ e, long n_src, TimeBin tb,
+                                                            int *__restrict__ counts)
+{
+    const long n = blockIdx.x * (long)kCompact + threadIdx.x;
+    bool up = false;
+    if (n < n_src) up = tb.R[6] * e[n] + tb.R[7] * e[n_src + n] + tb.R[8] * e[2 * n_src + n] > 0.0;
+    const int c = __syncthreads_count(up);
+    if (threadIdx.x == 0) counts[blockIdx.x] = c;
+}
+
+__global__ void __launch_bounds__(kCompact) k_compact_copy(const double *__restrict__ e, long n_src, TimeBin tb,
+                                                           const int *__restrict__ offsets, double *__restrict__ sdir,
+                                                           int *__restrict__ sidx, float4 *__restrict__ tc)
+{
+    __shared__ int s_n[kCompact / 32];
+    const long n = blockIdx.x * (long)kCompact + threadIdx.x;
+    double ex = 0.0, ey = 0.0, ez = 0.0, s2 = 0.0;
+    if (n < n_src) {
+        ex = e[n];
+        ey = e[n_src + n];
+        ez = e[2 * n_src + n];
+        s2 = tb.R[6] * ex + tb.R[7] * ey + tb.R[8] * ez;
+    }
+    const bool up = s2 > 0.0;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const unsigned m = __ballot_sync(0xffffffffu, up);
+    if (lane == 0) s_n[warp] = __popc(m);
+    __syncthreads();
+    if (!up) return;
+    int pos = offsets[blockIdx.x] + __popc(m & ((1u << lane) - 1u));
+    for (int w = 0; w < warp; ++w) pos += s_n[w];
+    const double s0 = tb.R[0] * ex + tb.R[1] * ey + tb.R[2] * ez, s1 = tb.R[3] * ex + tb.R[4] * ey + tb.R[5] * ez;
+    sidx[pos] = (int)n;
+    if (tc) {
+        const float2 a = split_f2(tb.a[0][0] * s0 + tb.a[0][1] * s1), b = split_f2(tb.a[1][0] * s0 + tb.a[1][1] * s1);
+        tc[2 * (size_t)pos] = make_float4(a.x, a.y, b.x, b.y);
+        tc[2 * (size_t)pos + 1] = make_float4((float)s0, (float)s1, (float)s2, (float)(2.0 * s2 - 1.0));
+    } else {
+        sdir[pos] = s0;
+        sdir[n_src + pos] = s1;
+        sdir[2 * n_src + pos] = s2;
+    }
+}
+
+int time_compact_blocks(long n_src) { return (int)std::max<long>(1, (n_src + kCompact - 1) / kCompact); }
+
+cudaError_t launch_time_compact(const double *e, long n_src, const TimeBin &tb, int *counts, int *offsets, int *cursor,
+                                double *sdir, int *sidx, float4 *tc, cudaStream_t st)
+{
+    const int nb = time_compact_blocks(n_src);
+    k_compact_count<<<nb, kCompact, 0, st>>>(e, n_src, tb, counts);
+    const int blocks = (nb + kScanBlock - 1) / kScanBlock;
+    int *blk = counts + nb;
+    if (blocks > 1) k_bin_sums<<<blocks, 1024, 0, st>>>(counts, nb, blk);
+    k_bin_scan<<<blocks, 1024, 0, st>>>(counts, nb, offsets, cursor, blk);
+    if (n_src > 0) k_compact_copy<<<nb, kCompact, 0, st>>>(e, n_src, tb, offsets, sdir, sidx, tc);
+    return cudaGetLastError();
 }
 
 cudaError_t launch_time_binning(const double *e, long n_src, const TimeBin &tb, int *bin_of, int *counts,
