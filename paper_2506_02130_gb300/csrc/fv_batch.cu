@@ -85,13 +85,21 @@ static fv_status enqueue(fv_batch_s *b)
         per[l].push_back(i);
         load[l] += b->items[i].cost;
     }
-    // each member plan's channel-major flux copy from its borrowed buffer, once per execution, before the fork
-    std::vector<fv_plan_s *> seen;
-    for (const auto &it : b->items)
-        if (std::find(seen.begin(), seen.end(), it.p) == seen.end()) {
-            seen.push_back(it.p);
-            CKB(refresh_flux_t(it.p, b->stream));
+    // the channels that the batch's items take of each member plan's channel-major flux copy, from its borrowed buffer,
+    // once per execution, before the fork
+    std::vector<std::pair<fv_plan_s *, std::pair<int, int>>> seen;
+    for (const auto &it : b->items) {
+        const long nf = (long)it.p->freq.size();
+        const int f0 = (int)(it.k0 % nf), f1 = f0 + (int)(it.k1 - it.k0);      // an item is channels of one time
+        auto s = std::find_if(seen.begin(), seen.end(), [&](const auto &v) { return v.first == it.p; });
+        if (s == seen.end()) {
+            seen.push_back({it.p, {f0, f1}});
+        } else {
+            s->second.first = std::min(s->second.first, f0);
+            s->second.second = std::max(s->second.second, f1);
         }
+    }
+    for (const auto &v : seen) CKB(refresh_flux_t(v.first, v.second.first, v.second.second, b->stream));
     CKB(cudaEventRecord(b->ev_fork, b->stream));
     for (int l = 0; l < L; ++l) CKB(cudaStreamWaitEvent(b->lanes[l], b->ev_fork, 0));
     for (int l = 0; l < L; ++l) {

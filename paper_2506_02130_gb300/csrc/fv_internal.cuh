@@ -85,7 +85,6 @@ struct TimeBin {
     int T[2];               // tile (= bin) size in cells
     int nbx, nby;           // bins per axis
     double a[2][2];         // lattice vectors (launch_time_compact's records)
-    int strips;             // bin order: 0 row by row (x fastest), 1 strip by strip (y fastest)
 };
 
 #define FV_SPREAD_SMEM_MAX (96 * 1024)
@@ -418,13 +417,14 @@ __device__ __forceinline__ int source_strengths(const SliceGeom &g, S s0, S s1, 
 // ---------------------------------------------------------------- launchers
 // All launchers enqueue on `st` and return the launch error (cudaSuccess if fine).
 
-// Channel-major copy of the fluxes: out[f][n][k] = flux[k][n][f] (n_stokes k, n_src n, n_freq f), in the
+// Channel-major copy of channels [f0, f1) of the fluxes: out[f][n][k] = flux[k][n][f] (n_stokes k, n_src n, n_freq f), in the
 // fluxes' precision.
-cudaError_t launch_flux_transpose(const void *flux, int fp64, long n_src, int n_stokes, int n_freq, void *out,
-                                  cudaStream_t st);
+cudaError_t launch_flux_transpose(const void *flux, int fp64, long n_src, int n_stokes, int n_freq, int f0, int f1,
+                                  void *out, cudaStream_t st);
 
 // e[3][n]: equatorial unit vectors from (ra, dec).
-cudaError_t launch_radec_to_unit(const double *ra, const double *dec, long n, double *e, cudaStream_t st);
+// ep (nullable): the same as float pairs, [3][n].
+cudaError_t launch_radec_to_unit(const double *ra, const double *dec, long n, double *e, float2 *ep, cudaStream_t st);
 
 // Per-block min/max of visible ENU directions over all times: out[nblocks][6].
 cudaError_t launch_source_extents(const double *e, long n, const double *R_all, int n_time,
@@ -465,6 +465,11 @@ inline size_t bin_count_ints(int nb) { return (size_t)nb + (nb + kScanBlock - 1)
 cudaError_t launch_time_binning(const double *e, long n_src, const TimeBin &tb, int *bin_of, int *counts,
                                 int *offsets, int *cursor, double *sdir, int *sidx, float4 *tc, cudaStream_t st);
 
+// The same for FP32 plans whose sources are sorted by strips, in pair arithmetic from the directions' float pairs ep
+// (e decides where the horizon is within their rounding): only tc and sidx are written.  slot: n_src ints.
+cudaError_t launch_time_strips(const double *e, const float2 *ep, long n_src, const TimeBin &tb, int *bin_of, int *slot,
+                               int *counts, int *offsets, int *cursor, int *sidx, float4 *tc, cudaStream_t st);
+
 // Per time, without bins: the sources above the horizon in their own order (sdir, sidx); offsets[time_compact_blocks]
 // is their number.  counts, offsets and cursor as for that many bins.
 // tc (nullable): in sdir's place {a_1 . s (hi, lo), a_2 . s (hi, lo)} and {s, 2 s_up - 1} per source (TimeBin::a).
@@ -498,7 +503,7 @@ cudaError_t launch_spread_scatter(const int *offsets, const int *cell, const G *
 size_t spread_scatter_smem(int elem_bytes, int n_pol, int nz);
 
 // Preparation and spreading in one launch for FP32 grids (w <= 8, n_pol 1 or 4, at most 16 up planes or height
-// terms): the sources sorted by strips (TimeBin::strips) with their per-time records tc, added to grid
+// terms): the sources sorted by strips (launch_time_strips) with their per-time records tc, added to grid
 // [ny][nx][n_pol][strip_planes(nz)], which the caller has cleared; the x and y prescales of g are applied.  Any order of the
 // sources gives the same sums.
 constexpr int kEsTerms = 5;

@@ -22,10 +22,9 @@
 // CTAs are FP64.  A 37-antenna slice of 1,000 sources takes 29 us (172 us of FP64 spreading, 63 of preparation and
 // 28 of FFT passes before) with an error against the direct sum of 1.3e-14 where the transform gave 5.8e-11.
 #include "fv_lattice_dense.cuh"
-#include "fv_plan.cuh"
+#include "fv_pair.cuh"
 
 #include <algorithm>
-#include <cstdlib>
 
 namespace fv {
 
@@ -107,28 +106,6 @@ template <> struct Dense<double> {
         return cmk<double>((double)a.h.x + (double)a.l.x, (double)a.h.y + (double)a.l.y);
     }
 };
-
-// a pair product and a pair sum of scalars (the powers of a source's phase factors)
-struct Pf { float h, l; };
-__device__ __forceinline__ Pf pf(double v)
-{
-    const float h = (float)v;
-    return Pf{h, (float)(v - (double)h)};
-}
-__device__ __forceinline__ Pf pmul(Pf a, Pf b)
-{
-    const float p = a.h * b.h;
-    const float e = fmaf(a.l, b.h, fmaf(a.h, b.l, fmaf(a.h, b.h, -p)));
-    const float h = __fadd_rn(p, e);
-    return Pf{h, __fadd_rn(e, -__fadd_rn(h, -p))};
-}
-__device__ __forceinline__ Pf padd(Pf a, Pf b)
-{
-    const float s = __fadd_rn(a.h, b.h), t = __fadd_rn(s, -a.h);
-    const float e = __fadd_rn(__fadd_rn(__fadd_rn(a.h, -__fadd_rn(s, -t)), __fadd_rn(b.h, -t)), __fadd_rn(a.l, b.l));
-    const float h = __fadd_rn(s, e);
-    return Pf{h, __fadd_rn(e, -__fadd_rn(h, -s))};
-}
 
 }  // namespace
 

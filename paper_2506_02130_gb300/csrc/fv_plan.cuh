@@ -79,10 +79,11 @@ struct fv_plan_s {
     long n_src = 0;
     int n_stokes = 1;
     double *d_e = nullptr;
+    float2 *d_ep = nullptr;          // FP32 plans: d_e as float pairs
     void *d_flux_owned = nullptr;
     // sky buffers are kept across fv_set_sky calls of the same size (allocating and freeing gigabytes of
     // fluxes each time cost more than the copies): capacities in bytes, and the small scratch of set_sky
-    size_t e_bytes = 0, flux_owned_bytes = 0, flux_t_bytes = 0, radec_bytes = 0;
+    size_t e_bytes = 0, ep_bytes = 0, flux_owned_bytes = 0, flux_t_bytes = 0, radec_bytes = 0;
     double *d_radec = nullptr, *d_Rt = nullptr, *d_ext = nullptr;
     const void *flux = nullptr;
     int flux_fp64 = 0;
@@ -248,8 +249,8 @@ fv_status run_slices(fv_plan_s *p, fv_plan_s::Workspace &wk, cudaStream_t st, ch
 template <class G>
 fv_status run_basis(fv_plan_s *p, fv_plan_s::Workspace &wk, cudaStream_t st, char *vis, size_t slice_bytes,
                     int t_begin, int t_end);
-// Refresh the channel-major flux copy from a borrowed device flux, on stream st (no-op otherwise).
-cudaError_t refresh_flux_t(fv_plan_s *p, cudaStream_t st);
+// Refresh channels [f0, f1) of the channel-major flux copy from a borrowed device flux, on stream st (no-op otherwise).
+cudaError_t refresh_flux_t(fv_plan_s *p, int f0, int f1, cudaStream_t st);
 // Device status word of a plan: copy it behind an execution's work, and report (once) a bounded wait
 // that ran out in an earlier execution as FV_ERR_TIMEOUT.
 cudaError_t plan_post_status(fv_plan_s *p);

@@ -904,12 +904,15 @@ fv_status run_slices(fv_plan_s *p, fv_plan_s::Workspace &wk, cudaStream_t st, ch
             tb.T[1] = p->T[1];
             tb.nbx = p->nbx;
             tb.nby = p->nby;
-            tb.strips = p->strip ? 1 : 0;
             tb.d = p->d;
             for (int i = 0; i < 3; ++i) tb.D_top[i] = p->gf[p->f_top].dim[i].D;
             CK(prof_begin(p, PC_BIN, st));
-            CK(launch_time_binning(p->d_e, p->n_src, tb, wk.bin_of, wk.counts, wk.offsets, wk.cursor, wk.sdir,
-                                   wk.sidx, sizeof(G) == 4 ? wk.tc : nullptr, st));
+            if (p->strip)
+                CK(launch_time_strips(p->d_e, p->d_ep, p->n_src, tb, wk.bin_of, wk.cell, wk.counts, wk.offsets,
+                                      wk.cursor, wk.sidx, wk.tc, st));
+            else
+                CK(launch_time_binning(p->d_e, p->n_src, tb, wk.bin_of, wk.counts, wk.offsets, wk.cursor, wk.sdir,
+                                       wk.sidx, sizeof(G) == 4 ? wk.tc : nullptr, st));
             CK(prof_end(p, (double)p->n_src * 80.0 + nb * 12.0 + (wk.tc ? p->n_src * 0.5 * 48.0 : 0.0)));
             t_binned = t;
         }
@@ -1372,10 +1375,13 @@ fv_status run_basis(fv_plan_s *p, fv_plan_s::Workspace &wk, cudaStream_t st, cha
 template fv_status run_basis<float>(fv_plan_s *, fv_plan_s::Workspace &, cudaStream_t, char *, size_t, int, int);
 template fv_status run_basis<double>(fv_plan_s *, fv_plan_s::Workspace &, cudaStream_t, char *, size_t, int, int);
 
-cudaError_t refresh_flux_t(fv_plan_s *p, cudaStream_t st)
+// One channel of one Stokes parameter is channel-major as it is: the slices read the plan's copy or the caller's buffer.
+static bool flux_in_place(const fv_plan_s *p) { return p->n_stokes == 1 && p->freq.size() == 1; }
+
+cudaError_t refresh_flux_t(fv_plan_s *p, int f0, int f1, cudaStream_t st)
 {
     if (!p->flux_borrowed || !p->d_flux_t || p->n_src == 0) return cudaSuccess;
-    return launch_flux_transpose(p->flux, p->flux_fp64, p->n_src, p->n_stokes, (int)p->freq.size(), p->d_flux_t,
+    return launch_flux_transpose(p->flux, p->flux_fp64, p->n_src, p->n_stokes, (int)p->freq.size(), f0, f1, p->d_flux_t,
                                  st);
 }
 
@@ -1425,7 +1431,7 @@ static fv_status execute_slices(fv_plan_s *p, char *vis, size_t slice_bytes, cha
     else if (p->flux_borrowed && p->d_flux_t) {
         // the channel-major flux copy from the borrowed buffer (read and written once)
         CK(prof_begin(p, PC_FLUX_T, p->stream));
-        CK(refresh_flux_t(p, p->stream));
+        CK(refresh_flux_t(p, 0, (int)p->freq.size(), p->stream));
         CK(prof_end(p, 2.0 * p->n_src * p->n_stokes * p->freq.size() * (p->flux_fp64 ? 8 : 4)));
     }
     const int S = (int)std::min<long>(p->n_streams, std::max<long>(total, 1));
@@ -2023,7 +2029,8 @@ fv_status fv_set_sky(fv_plan_t p, long n_src, const double *ra_rad, const double
         CK(cudaMemcpyAsync(d_tmp, ra_rad, n_src * sizeof(double), cudaMemcpyHostToDevice, p->stream));
         CK(cudaMemcpyAsync(d_tmp + ns, dec_rad, n_src * sizeof(double), cudaMemcpyHostToDevice, p->stream));
     }
-    CK(launch_radec_to_unit(d_tmp, d_tmp + ns, n_src, p->d_e, p->stream));
+    if (p->precision == FV_MIXED) CK(ensure((void **)&p->d_ep, p->ep_bytes, ns * 3 * sizeof(float2)));
+    CK(launch_radec_to_unit(d_tmp, d_tmp + ns, n_src, p->d_e, p->d_ep, p->stream));
     const size_t fbytes = (size_t)n_stokes * n_src * p->freq.size() * (p->flux_fp64 ? 8 : 4);
     if (flux_on_device) {
         p->flux = flux;
@@ -2035,13 +2042,16 @@ fv_status fv_set_sky(fv_plan_t p, long n_src, const double *ra_rad, const double
         CK(cudaMemcpyAsync(p->d_flux_owned, flux, fbytes, cudaMemcpyHostToDevice, p->stream));
         p->flux = p->d_flux_owned;
     }
-    if (n_src && !p->use_basis) {
+    if (flux_in_place(p)) {
+        dfree(p->d_flux_t);
+        p->flux_t_bytes = 0;
+    } else if (n_src && !p->use_basis) {
         // the channel-major copy the slices read: made now from an owned copy, at every execution from a
         // borrowed buffer
         CK(ensure(&p->d_flux_t, p->flux_t_bytes, fbytes));
         if (!p->flux_borrowed)
-            CK(launch_flux_transpose(p->flux, p->flux_fp64, n_src, n_stokes, (int)p->freq.size(), p->d_flux_t,
-                                     p->stream));
+            CK(launch_flux_transpose(p->flux, p->flux_fp64, n_src, n_stokes, (int)p->freq.size(), 0,
+                                     (int)p->freq.size(), p->d_flux_t, p->stream));
     }
     // source extents over all times (visible directions only)
     const int nb = 304;
@@ -2142,6 +2152,7 @@ fv_status fv_destroy(fv_plan_t p)
     dfree_t(p->d_bln);
     dfree_t(p->d_grp_bl);
     dfree_t(p->d_e);
+    dfree_t(p->d_ep);
     dfree(p->d_flux_owned);
     dfree(p->d_flux_t);
     dfree_t(p->d_radec);

@@ -127,7 +127,7 @@ extern "C" fv_status fv_execute_static(fv_plan_t p, void *vis)
     }
     // the channel-major flux copy (a plan-owned buffer made at fv_set_sky), then every slice on the plan's
     // stream, in order, through the one scratch workspace
-    CKS(refresh_flux_t(p, p->stream));
+    CKS(refresh_flux_t(p, 0, (int)p->freq.size(), p->stream));
     fv_status s = p->precision == FV_FP64 ? run_slices<double>(p, wk, p->stream, (char *)vis, slice_bytes, 0, total)
                                           : run_slices<float>(p, wk, p->stream, (char *)vis, slice_bytes, 0, total);
     if (s == FV_OK) CKS(plan_post_status(p));   // a copy of the status word into pinned memory: no allocation

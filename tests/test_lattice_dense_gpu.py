@@ -84,7 +84,7 @@ def test_many_channels_and_windows_of_a_batch():
 @pytest.mark.parametrize("precision,eps,tol", [(fv.FV_FP64, 1e-11, 1e-9), (fv.FV_MIXED, 1e-6, 2e-5)])
 def test_lattices_too_large_for_direct_sums_keep_the_grid(precision, eps, tol):
     prob = W.config_hex127(seed=12, n_chan=2, n_time=1, n_point=200, nside=0, radius=1)
-    prob.ant_enu = np.array([[2.0 * k, 0.0, 0.0] for k in (0, 1, 3, 850)])      # 1,701 modes along the line
+    prob.ant_enu = np.array([[0.5 * k, 0.0, 0.0] for k in (0, 1, 3, 850)])      # 1,701 modes along the line
     prob.pairs = W.cross_pairs(4)
     out, info = _run(prob, precision, eps)
     assert info["lattice_modes"][0] == 1701

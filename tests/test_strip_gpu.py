@@ -102,3 +102,42 @@ def test_plane_interpolation_writes_every_copy_of_a_baseline(z_sigma, polarised,
     out, info = _run(prob, 1e-6, **kw)
     assert info["n_unique"] < info["n_bl"]
     assert rel_l2(out, oracle_vis(OracleProblem.from_workload(prob), "factored")) <= 2e-5
+
+
+@pytest.mark.parametrize("n_chan", [1, 2, 3, 31, 33])
+@pytest.mark.parametrize("dtype", [np.float32, np.float64])
+@pytest.mark.parametrize("polarised", [False, True])
+def test_flux_layouts(n_chan, dtype, polarised):
+    """The channel-major copy of the fluxes: one channel to more than a tile's, both types, host and borrowed."""
+    torch = pytest.importorskip("torch")
+    prob = _prob(1500, polarised, radius=1, n_chan=n_chan)
+    prob.sky.flux = np.ascontiguousarray(prob.sky.flux.astype(dtype))
+    out, _ = _run(prob, 1e-6)
+    assert rel_l2(out, oracle_vis(OracleProblem.from_workload(prob), "factored")) <= 2e-5
+    dev = torch.from_numpy(prob.sky.flux).cuda()
+    p = fv.Plan.from_problem(prob, precision=fv.FV_MIXED, eps=1e-6, transform="type3")
+    p.set_sky(prob.sky.ra, prob.sky.dec, dev)
+    assert rel_l2(p.run(), out) <= 2e-6
+    dev *= 2.0                                   # rewritten in place between executions
+    torch.cuda.synchronize()
+    assert rel_l2(p.run(), 2.0 * out) <= 2e-6
+    p.close()
+
+
+def test_sources_on_the_horizon_are_cut_as_in_fp64():
+    """Sources within a few FP64 roundings of the horizon: the pair arithmetic of the sort must not decide them."""
+    prob = _prob(400, False, radius=2, n_chan=1)
+    lst, lat = prob.lsts_rad[0], prob.latitude_rad
+    az = np.linspace(0.0, 2 * np.pi, 400, endpoint=False)
+    alt = np.repeat([0.0, 1e-17, -1e-17, 1e-16, -1e-16, 1e-15, -1e-15, 1e-13], 50)
+    e, n, u = np.cos(alt) * np.sin(az), np.cos(alt) * np.cos(az), np.sin(alt)
+    z = n * np.cos(lat) + u * np.sin(lat)
+    r = -n * np.sin(lat) + u * np.cos(lat)
+    prob.sky.dec = np.arcsin(np.clip(z, -1, 1))
+    prob.sky.ra = (lst + np.arctan2(e, r)) % (2 * np.pi)
+    prob.beam, prob.beam_param = "uniform", ()          # a beam that reaches the horizon
+    mixed, _ = _run(prob, 1e-6)
+    p = fv.Plan.from_problem(prob, precision=fv.FV_FP64, eps=1e-9, transform="type3")
+    p.set_sky(prob.sky.ra, prob.sky.dec, prob.sky.flux)
+    assert rel_l2(mixed, p.run()) <= 2e-5
+    p.close()
