@@ -203,12 +203,12 @@ cudaError_t launch_basis_targets(const double *bu, int n_u, const double *kappa,
 
 // ------------------------------------------------------------------ interpolation with the expansion
 // One warp per target (u, q).  The band after the x and y passes holds, per (b_y, b_x) cell, the K
-// planes' z values contiguously ([k][l_z], K * Nz values).  Lane L holds the values j = L + 32 r
-// (r < R = ceil(K Nz / 32)) of that run, with the weights c_j = M_qk K(l_z), where
-// K(l_z) = sum_{m_z} phi((2/w)(p_z - m_z)) e^{2 pi i l_z m_z / M_z} (z prescale folded in) is the
-// direct z sum of the short z axis; each footprint tap is then R coalesced loads per warp, scaled by
-// the tap's x and y kernel values, and the warp reduces at the end.  The target's constants come from
-// the per-target table, so the kernel does no FP64 arithmetic.
+// planes' z values contiguously ([k][l_z], K * Nz values).  Lane L sums the values j = L + 32 r
+// (r < R = ceil(K Nz / 32)) of that run over the footprint, weighted by the taps' x and y kernel values
+// alone, and applies the weights c_j = M_qk K(l_z) once at the
+// end, where K(l_z) = sum_{m_z} phi((2/w)(p_z - m_z)) e^{2 pi i l_z m_z / M_z} (z prescale folded in) is
+// the direct z sum of the short z axis.  The target's constants come from the per-target table, so the
+// kernel does no FP64 arithmetic on FP32 grids.
 template <class G, bool HASZ, int R>
 __global__ void __launch_bounds__(256) k_interp_basis(const cpx<G> *__restrict__ band, int u0, int n_ug, int n_u,
                                                       int n_freq, const G *__restrict__ M, int K,
@@ -230,67 +230,62 @@ __global__ void __launch_bounds__(256) k_interp_basis(const cpx<G> *__restrict__
     const int4 mm = tm[tix];
     const G frx = tf[4 * tix], fry = tf[4 * tix + 1], frz = tf[4 * tix + 2];
     const int Nz = HASZ ? g.dim[2].nf1 : 1;
+    const int KN = K * Nz;                      // R = ceil(KN / 32), a template parameter
+    const int Bx = g.dim[0].B;
+    const int bx0 = mm.x + g.dim[0].H, by0 = mm.y + g.dim[1].H;
+    // x and y kernel values: lane j < w holds the j-th
+    const G wxm = lane < w ? es_phi(two_over_w * (frx - (G)lane), beta) : (G)0;
+    const G wym = lane < w ? es_phi(two_over_w * (fry - (G)lane), beta) : (G)0;
+    cpx<G> acc[R];
+#pragma unroll
+    for (int r = 0; r < R; ++r) acc[r] = cmk<G>((G)0, (G)0);
+    for (int jy = 0; jy < w; ++jy) {
+        const G wy = __shfl_sync(0xffffffffu, wym, jy);
+        const cpx<G> *c = band + ((size_t)(by0 + jy) * Bx + bx0) * KN + lane;
+#pragma unroll 4
+        for (int jx = 0; jx < w; ++jx, c += KN) {
+            const G wt = wy * __shfl_sync(0xffffffffu, wxm, jx);
+#pragma unroll
+            for (int r = 0; r < R; ++r)
+                if (r < R - 1 || lane + 32 * r < KN) {
+                    const cpx<G> v = c[32 * r];
+                    acc[r].x += wt * v.x;
+                    acc[r].y += wt * v.y;
+                }
+        }
+    }
     // lane lz < Nz builds K(l_z)
     cpx<G> Kmine = cmk<G>((G)1, (G)0);
     if (HASZ && lane < Nz) {
         const int Mz = g.dim[2].M;
         const int lc = lane - Nz / 2;
-        cpx<G> acc = cmk<G>((G)0, (G)0);
+        cpx<G> s = cmk<G>((G)0, (G)0);
         int e = (lc * mm.z) % Mz;
         if (e < 0) e += Mz;
         int step = lc % Mz;
         if (step < 0) step += Mz;
         for (int jz = 0; jz < w; ++jz) {
             const G wt = es_phi(two_over_w * (frz - (G)jz), beta);
-            acc = cadd(acc, cscale(twz[e], wt));
+            s = cadd(s, cscale(twz[e], wt));
             e += step;
             if (e >= Mz) e -= Mz;
         }
-        Kmine = cscale(acc, prez[lane]);
+        Kmine = cscale(s, prez[lane]);
     }
-    // this lane's weights c_r = M_qk K(l_z) for j = lane + 32 r (shuffles taken by every lane)
-    const int KN = K * Nz;                      // R = ceil(KN / 32), a template parameter
-    cpx<G> cf[R];
+    // this lane's weights M_qk K(l_z) of j = lane + 32 r (shuffles taken by every lane)
+    G ax = (G)0, ay = (G)0;
 #pragma unroll
     for (int r = 0; r < R; ++r) {
-        cf[r] = cmk<G>((G)0, (G)0);
-        {
-            const int j = lane + 32 * r;
-            const bool valid = j < KN;
-            const int k = valid ? j / Nz : 0;
-            const int lz = valid ? j - k * Nz : 0;
-            const G kx = __shfl_sync(0xffffffffu, Kmine.x, lz);
-            const G ky = __shfl_sync(0xffffffffu, Kmine.y, lz);
-            if (valid) {
-                const G mk = M[q * K + k];
-                cf[r] = cmk<G>(kx * mk, ky * mk);
-            }
-        }
-    }
-    const int Bx = g.dim[0].B;
-    const int bx0 = mm.x + g.dim[0].H, by0 = mm.y + g.dim[1].H;
-    // x and y kernel values: lane j < w holds the j-th
-    const G wxm = lane < w ? es_phi(two_over_w * (frx - (G)lane), beta) : (G)0;
-    const G wym = lane < w ? es_phi(two_over_w * (fry - (G)lane), beta) : (G)0;
-    G ax = (G)0, ay = (G)0;
-    for (int jy = 0; jy < w; ++jy) {
-        const G wy = __shfl_sync(0xffffffffu, wym, jy);
-        const cpx<G> *row = band + ((size_t)(by0 + jy) * Bx + bx0) * KN;
-        for (int jx = 0; jx < w; ++jx) {
-            const G wt = wy * __shfl_sync(0xffffffffu, wxm, jx);
-            const cpx<G> *c = row + (size_t)jx * KN;
-            G sx = (G)0, sy = (G)0;
-#pragma unroll
-            for (int r = 0; r < R; ++r) {
-                const int j = lane + 32 * r;
-                if (r < R - 1 || j < KN) {
-                    const cpx<G> v = c[j];
-                    sx += v.x * cf[r].x - v.y * cf[r].y;
-                    sy += v.x * cf[r].y + v.y * cf[r].x;
-                }
-            }
-            ax += wt * sx;
-            ay += wt * sy;
+        const int j = lane + 32 * r;
+        const bool valid = j < KN;
+        const int k = valid ? j / Nz : 0;
+        const int lz = valid ? j - k * Nz : 0;
+        const G kx = __shfl_sync(0xffffffffu, Kmine.x, lz);
+        const G ky = __shfl_sync(0xffffffffu, Kmine.y, lz);
+        if (valid) {
+            const G mk = M[q * K + k];
+            ax += mk * (acc[r].x * kx - acc[r].y * ky);
+            ay += mk * (acc[r].x * ky + acc[r].y * kx);
         }
     }
     for (int o = 16; o > 0; o >>= 1) {
@@ -299,6 +294,106 @@ __global__ void __launch_bounds__(256) k_interp_basis(const cpx<G> *__restrict__
     }
     if (lane == 0) {
         const cpx<G> v = cmul(cmk<G>(ax, ay), ts[tix]);
+        Vq[(size_t)q * n_u + u] = cmk<double>((double)v.x, (double)v.y);
+    }
+}
+
+// The same for FP32 bands and w <= 8, with the work around the taps cut down (it was half of 1,600 instructions a
+// target): the z kernel values are computed one a lane and shared, the divisions go by multiplications, the x weights
+// sit in registers, and no load is predicated (a lane past a cell's values reads the next cell's and drops its sum;
+// the band has room behind it).  Bound by the L1's bytes, 49 taps x 88 values a target (17.7 GB a time on the
+// 127-antenna workload), about 70 % of whose rate it reaches: 0.90 ms a time against 1.27 with the complex weights
+// applied at every tap.  Tried and slower: 16-byte loads across a whole footprint row (1.38 ms, half the warps), two
+// to four neighbouring targets a warp sharing the union of their footprints (1.4 to 2.0: the targets are too sparse).
+struct BasisDiv { unsigned nf_mul, nf_sh, nz_inv; float mz_inv; };
+
+template <bool HASZ, int R>
+__global__ void __launch_bounds__(256, R <= 4 ? 5 : 4)
+    k_interp_basis_taps(const cpx<float> *__restrict__ band, int u0, int n_ug, int n_u, int n_freq,
+                        const float *__restrict__ M, int K, const int *__restrict__ perm, const int4 *__restrict__ tm,
+                        const float *__restrict__ tf, const cpx<float> *__restrict__ ts, float beta, SliceGeom g,
+                        BasisDiv dv, const float *__restrict__ prez, const cpx<float> *__restrict__ twz,
+                        cpx<double> *__restrict__ Vq)
+{
+    constexpr int W = 8;
+    const int lane = threadIdx.x & 31;
+    const long tg = (blockIdx.x * (long)blockDim.x + threadIdx.x) >> 5;
+    if (tg >= (long)n_ug * n_freq) return;     // whole warps
+    const int tix = perm[(long)u0 * n_freq + tg];
+    const int w = g.w;
+    const float two_over_w = 2.0f / (float)w;
+    const int4 mm = tm[tix];
+    const float4 fr = *reinterpret_cast<const float4 *>(tf + 4 * (size_t)tix);
+    const int Nz = HASZ ? g.dim[2].nf1 : 1, KN = K * Nz;
+    const float fl = (float)lane;
+    const float wxm = lane < w ? es_phi(two_over_w * (fr.x - fl), beta) : 0.0f;
+    const float wym = lane < w ? es_phi(two_over_w * (fr.y - fl), beta) : 0.0f;
+    float wx[W];
+#pragma unroll
+    for (int j = 0; j < W; ++j) wx[j] = __shfl_sync(0xffffffffu, wxm, j);
+    float2 acc[R];
+#pragma unroll
+    for (int r = 0; r < R; ++r) acc[r] = make_float2(0.0f, 0.0f);
+    const size_t rstride = (size_t)g.dim[0].B * KN;
+    const float2 *row = reinterpret_cast<const float2 *>(
+        band + ((size_t)(mm.y + g.dim[1].H) * g.dim[0].B + (mm.x + g.dim[0].H)) * KN + lane);
+    for (int jy = 0; jy < w; ++jy, row += rstride) {
+        const float wy = __shfl_sync(0xffffffffu, wym, jy);
+        const float2 *c = row;
+#pragma unroll
+        for (int j = 0; j < W; ++j) {
+            if (j < w) {                        // the same on every lane
+                const float wt = wy * wx[j];
+#pragma unroll
+                for (int r = 0; r < R; ++r) {
+                    const float2 v = __ldg(c + 32 * r);
+                    acc[r].x = fmaf(wt, v.x, acc[r].x);
+                    acc[r].y = fmaf(wt, v.y, acc[r].y);
+                }
+                c += KN;
+            }
+        }
+    }
+    // lane lz < Nz: K(l_z)
+    cpx<float> Kmine = cmk<float>(1.0f, 0.0f);
+    if (HASZ) {
+        const float wzm = lane < w ? es_phi(two_over_w * (fr.z - fl), beta) : 0.0f;
+        const int Mz = g.dim[2].M, lc = min(lane, Nz - 1) - Nz / 2;
+        auto mod = [&](int a) {                 // a mod Mz for |a| far below 2^20
+            int m = a - (int)floorf((float)a * dv.mz_inv) * Mz;
+            m += m < 0 ? Mz : 0;
+            return m >= Mz ? m - Mz : m;
+        };
+        int e = mod(lc * mod(mm.z));
+        const int step = mod(lc);
+        cpx<float> s = cmk<float>(0.0f, 0.0f);
+        for (int jz = 0; jz < w; ++jz) {
+            s = cadd(s, cscale(twz[e], __shfl_sync(0xffffffffu, wzm, jz)));
+            e += step;
+            if (e >= Mz) e -= Mz;
+        }
+        Kmine = cscale(s, prez[min(lane, Nz - 1)]);
+    }
+    const int u = (int)((__umulhi((unsigned)tix, dv.nf_mul) + (unsigned)tix) >> dv.nf_sh), q = tix - u * n_freq;
+    float ax = 0.0f, ay = 0.0f;
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        const int j = min(lane + 32 * r, KN - 1);
+        const int k = Nz > 1 ? (int)__umulhi((unsigned)j, dv.nz_inv) : j;
+        const int lz = j - k * Nz;
+        const float kx = __shfl_sync(0xffffffffu, Kmine.x, lz), ky = __shfl_sync(0xffffffffu, Kmine.y, lz);
+        if (lane + 32 * r < KN) {
+            const float mk = M[q * K + k];
+            ax += mk * (acc[r].x * kx - acc[r].y * ky);
+            ay += mk * (acc[r].x * ky + acc[r].y * kx);
+        }
+    }
+    for (int o = 16; o > 0; o >>= 1) {
+        ax += __shfl_xor_sync(0xffffffffu, ax, o);
+        ay += __shfl_xor_sync(0xffffffffu, ay, o);
+    }
+    if (lane == 0) {
+        const cpx<float> v = cmul(cmk<float>(ax, ay), ts[tix]);
         Vq[(size_t)q * n_u + u] = cmk<double>((double)v.x, (double)v.y);
     }
 }
@@ -324,6 +419,32 @@ cudaError_t launch_interp_basis(const cpx<G> *band, int u0, int n_ug, int n_u, i
     const long threads = (long)n_ug * n_freq * 32;
     const unsigned blocks = (unsigned)((threads + 255) / 256);
     const int R = (K * Nz + 31) / 32;
+    if constexpr (sizeof(G) == 4) {
+        if (g.w <= 8) {
+            BasisDiv dv{};
+            fft_magic((unsigned)n_freq, dv.nf_mul, dv.nf_sh);
+            dv.nz_inv = Nz > 1 ? 0xffffffffu / (unsigned)Nz + 1u : 0u;
+            dv.mz_inv = 1.0f / (float)(g.d == 3 ? g.dim[2].M : 1);
+#define FV_TAPS(Z, R) k_interp_basis_taps<Z, R><<<blocks, 256, 0, st>>>(band, u0, n_ug, n_u, n_freq, M, K, perm, tm, tf, ts, \
+                                                                       (float)g.beta, g, dv, prez, twz, Vq)
+            if (g.d != 3) {
+                FV_TAPS(false, 1);
+            } else {
+                switch (R) {
+                case 1: FV_TAPS(true, 1); break;
+                case 2: FV_TAPS(true, 2); break;
+                case 3: FV_TAPS(true, 3); break;
+                case 4: FV_TAPS(true, 4); break;
+                case 5: FV_TAPS(true, 5); break;
+                case 6: FV_TAPS(true, 6); break;
+                case 7: FV_TAPS(true, 7); break;
+                default: FV_TAPS(true, 8); break;
+                }
+            }
+#undef FV_TAPS
+            return cudaGetLastError();
+        }
+    }
     if (g.d == 3) {
         switch (R) {
         case 1: interp_basis_launch<G, true, 1>(blocks, band, u0, n_ug, n_u, n_freq, M, K, perm, tm, tf, ts, g, prez, twz, Vq, st); break;

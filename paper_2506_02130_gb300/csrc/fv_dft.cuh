@@ -5,26 +5,6 @@
 
 namespace fv {
 
-// complex sums and differences: one packed FP32 x 2 instruction in FP32 (the same rounding as two scalar ones)
-template <class G> __device__ __forceinline__ cpx<G> dadd(cpx<G> a, cpx<G> b)
-{
-    if constexpr (sizeof(G) == 4) {
-        const float2 r = __fadd2_rn(make_float2(a.x, a.y), make_float2(b.x, b.y));
-        return cmk<G>(r.x, r.y);
-    } else {
-        return cadd(a, b);
-    }
-}
-template <class G> __device__ __forceinline__ cpx<G> dsub(cpx<G> a, cpx<G> b)
-{
-    if constexpr (sizeof(G) == 4) {
-        const float2 r = __ffma2_rn(make_float2(b.x, b.y), make_float2(-1.0f, -1.0f), make_float2(a.x, a.y));
-        return cmk<G>(r.x, r.y);
-    } else {
-        return csub(a, b);
-    }
-}
-
 // ---------------------------------------------------------------- compile-time twiddles
 // e^{2 pi i m / R} for 2 <= R <= 16, from Taylor series on [0, pi/4] after an
 // exact reduction of the rational angle m/R to an octant (constexpr, host compiler).
@@ -101,30 +81,30 @@ template <class G> struct Dft<G, 2> {
     static __device__ __forceinline__ void run(cpx<G> *v)
     {
         cpx<G> a = v[0], b = v[1];
-        v[0] = dadd(a, b);
-        v[1] = dsub(a, b);
+        v[0] = cadd(a, b);
+        v[1] = csub(a, b);
     }
 };
 template <class G> struct Dft<G, 3> {
     static __device__ __forceinline__ void run(cpx<G> *v)
     {
         const G h = (G)0.86602540378443864676;   // sin(2 pi / 3)
-        cpx<G> t = dadd(v[1], v[2]), u = cmuli(cscale(dsub(v[1], v[2]), h));
-        cpx<G> m = dsub(v[0], cscale(t, (G)0.5));
-        v[0] = dadd(v[0], t);
-        v[1] = dadd(m, u);
-        v[2] = dsub(m, u);
+        cpx<G> t = cadd(v[1], v[2]), u = cmuli(cscale(csub(v[1], v[2]), h));
+        cpx<G> m = csub(v[0], cscale(t, (G)0.5));
+        v[0] = cadd(v[0], t);
+        v[1] = cadd(m, u);
+        v[2] = csub(m, u);
     }
 };
 template <class G> struct Dft<G, 4> {
     static __device__ __forceinline__ void run(cpx<G> *v)
     {
-        cpx<G> s02 = dadd(v[0], v[2]), d02 = dsub(v[0], v[2]);
-        cpx<G> s13 = dadd(v[1], v[3]), d13 = cmuli(dsub(v[1], v[3]));
-        v[0] = dadd(s02, s13);
-        v[2] = dsub(s02, s13);
-        v[1] = dadd(d02, d13);
-        v[3] = dsub(d02, d13);
+        cpx<G> s02 = cadd(v[0], v[2]), d02 = csub(v[0], v[2]);
+        cpx<G> s13 = cadd(v[1], v[3]), d13 = cmuli(csub(v[1], v[3]));
+        v[0] = cadd(s02, s13);
+        v[2] = csub(s02, s13);
+        v[1] = cadd(d02, d13);
+        v[3] = csub(d02, d13);
     }
 };
 template <class G> struct Dft<G, 5> {
@@ -132,17 +112,17 @@ template <class G> struct Dft<G, 5> {
     {
         const G c1 = (G)0.30901699437494742410, c2 = (G)-0.80901699437494742410;   // cos(2pi/5), cos(4pi/5)
         const G s1 = (G)0.95105651629515357212, s2 = (G)0.58778525229247312917;    // sin(2pi/5), sin(4pi/5)
-        cpx<G> t1 = dadd(v[1], v[4]), t2 = dadd(v[2], v[3]);
-        cpx<G> u1 = dsub(v[1], v[4]), u2 = dsub(v[2], v[3]);
-        cpx<G> a1 = dadd(v[0], dadd(cscale(t1, c1), cscale(t2, c2)));
-        cpx<G> a2 = dadd(v[0], dadd(cscale(t1, c2), cscale(t2, c1)));
-        cpx<G> b1 = cmuli(dadd(cscale(u1, s1), cscale(u2, s2)));
-        cpx<G> b2 = cmuli(dsub(cscale(u1, s2), cscale(u2, s1)));
-        v[0] = dadd(v[0], dadd(t1, t2));
-        v[1] = dadd(a1, b1);
-        v[4] = dsub(a1, b1);
-        v[2] = dadd(a2, b2);
-        v[3] = dsub(a2, b2);
+        cpx<G> t1 = cadd(v[1], v[4]), t2 = cadd(v[2], v[3]);
+        cpx<G> u1 = csub(v[1], v[4]), u2 = csub(v[2], v[3]);
+        cpx<G> a1 = cadd(v[0], cadd(cscale(t1, c1), cscale(t2, c2)));
+        cpx<G> a2 = cadd(v[0], cadd(cscale(t1, c2), cscale(t2, c1)));
+        cpx<G> b1 = cmuli(cadd(cscale(u1, s1), cscale(u2, s2)));
+        cpx<G> b2 = cmuli(csub(cscale(u1, s2), cscale(u2, s1)));
+        v[0] = cadd(v[0], cadd(t1, t2));
+        v[1] = cadd(a1, b1);
+        v[4] = csub(a1, b1);
+        v[2] = cadd(a2, b2);
+        v[3] = csub(a2, b2);
     }
 };
 

@@ -385,7 +385,7 @@ static bool factor_into(int M, int maxStages, int maxRadix, int *rad, int &n)
 }
 
 // multiply-high division by d: q = (umulhi(n, mul) + n) >> sh for n < 2^31
-static void magic_u32(unsigned d, unsigned &mul, unsigned &sh)
+void fft_magic(unsigned d, unsigned &mul, unsigned &sh)
 {
     unsigned s = 0;
     while ((1ull << s) < d) ++s;
@@ -414,8 +414,8 @@ void fft_stage_constants(DimGeom &dg)
 {
     int Ns = 1;
     for (int s = 0; s < dg.nstages; ++s) {
-        magic_u32((unsigned)(dg.M / dg.radix[s]), dg.mr_mul[s], dg.mr_sh[s]);
-        magic_u32((unsigned)Ns, dg.ns_mul[s], dg.ns_sh[s]);
+        fft_magic((unsigned)(dg.M / dg.radix[s]), dg.mr_mul[s], dg.mr_sh[s]);
+        fft_magic((unsigned)Ns, dg.ns_mul[s], dg.ns_sh[s]);
         Ns *= dg.radix[s];
     }
 }

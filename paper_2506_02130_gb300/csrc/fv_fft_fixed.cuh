@@ -14,7 +14,8 @@
 //
 // What bounds it: instruction issue (52-58 % busy), with half of the multi-length kernel's instructions (15.1 M
 // against 29.1 M for 3,000 rows of 3,072: no index divisions by variables, no products for the twiddles, half of
-// the first stage's inputs and of the last one's outputs left out, packed sums), then the waits for the rows.
+// the first stage's inputs and of the last one's outputs left out), then the waits for the rows.  Packed FP32 x 2
+// sums (one instruction for a complex sum) changed nothing: 22.2 against 21.6 us, the operands' moves take the slots.
 // Measured per slice, one stream, against the multi-length kernel: 350-antenna workload 22 + 21 us (x and y) against
 // 55 + 50, 127-antenna workload with 8 height terms 17 + 16 against 38 + 36.
 #pragma once
@@ -44,9 +45,9 @@ __device__ __forceinline__ void dft16_half(const cpx<float> *v, cpx<float> *o)
     C U[4][4];
     auto column = [&](const int r2, C a, C d) {
         // points r2 (r1 = 0) and 12 + r2 (r1 = 3): a + d e^{2 pi i 3 q / 4}
-        U[r2][0] = dadd(a, d);
+        U[r2][0] = cadd(a, d);
         U[r2][1] = cmk<float>(a.x + d.y, a.y - d.x);
-        U[r2][2] = dsub(a, d);
+        U[r2][2] = csub(a, d);
         U[r2][3] = cmk<float>(a.x - d.y, a.y + d.x);
     };
     column(0, v[0], v[4]);

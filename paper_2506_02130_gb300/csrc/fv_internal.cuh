@@ -614,6 +614,8 @@ int fft_rows_per_cta(int M, int elem_bytes);
 // Smallest even M >= target that is a product of at most 3 (4 above 4096)
 // supported radices; fills radix[] and nstages.  -1 if none.
 int fft_choose_length(int target, int *radix, int &nstages, int maxRadix);
+// Constants of a division by d: n / d = (umulhi(n, mul) + n) >> sh for n < 2^31.
+void fft_magic(unsigned d, unsigned &mul, unsigned &sh);
 // Per-stage multiply-high division constants of dg (needs M, nstages, radix).
 void fft_stage_constants(DimGeom &dg);
 

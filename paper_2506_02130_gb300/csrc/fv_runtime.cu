@@ -1277,7 +1277,7 @@ static fv_status prepare_basis(fv_plan_s *p)
     p->need = fv_plan_s::WsNeed{};
     p->need.grid = (size_t)p->basis_Kp * D[0].nf1 * D[1].nf1 * D[2].nf1 * es;
     p->need.bufA = (size_t)D[0].B * K * D[2].nf1 * D[1].nf1 * es;
-    p->need.bufB = (size_t)D[1].B * D[0].B * K * D[2].nf1 * es;
+    p->need.bufB = (size_t)D[1].B * D[0].B * K * D[2].nf1 * es + 64 * es;   // room behind the band (interpolation)
     p->need.vu = std::max<size_t>(nt_all, 1) * sizeof(cpx<double>);
     p->need.tiled = true;
     p->need.n_src = std::max<long>(p->n_src, 1);
