@@ -67,6 +67,7 @@ static bool covers(const fv_plan_s::WsNeed &have, const fv_plan_s::WsNeed &need)
            (!need.tiled || (have.tiled && have.n_src >= need.n_src && have.nb >= need.nb &&
                             have.frac_per_src >= need.frac_per_src && have.cs_per_src >= need.cs_per_src &&
                             (have.tc || !need.tc) && (have.rec || !need.rec) && (have.dirs || !need.dirs) &&
+                            (have.cells || !need.cells) && have.pairs >= need.pairs &&
                             have.ring_tiles >= need.ring_tiles &&
                             have.ring_slots >= need.ring_slots && have.ring_np >= need.ring_np));
 }
@@ -247,7 +248,7 @@ fv_status fv_batch_execute(fv_batch_t b, int use_graph)
         }
     }
     fv_plan_s::WsNeed need;
-    need.dirs = false;
+    need.dirs = need.cells = false;
     for (const auto &it : b->items) {
         const auto &n = it.p->need;
         need.grid = std::max(need.grid, n.grid);
@@ -263,6 +264,8 @@ fv_status fv_batch_execute(fv_batch_t b, int use_graph)
             need.tc = need.tc || n.tc;
             need.rec = need.rec || n.rec;
             need.dirs = need.dirs || n.dirs;
+            need.cells = need.cells || n.cells;
+            need.pairs = std::max(need.pairs, n.pairs);
             need.ring_tiles = std::max(need.ring_tiles, n.ring_tiles);
             need.ring_slots = std::max(need.ring_slots, n.ring_slots);
             need.ring_np = std::max(need.ring_np, n.ring_np);

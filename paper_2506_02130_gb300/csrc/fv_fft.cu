@@ -21,6 +21,7 @@
 // stride-R stores of the first stage); index arithmetic uses
 // multiply-high division by the per-stage constants prepared on the host.
 #include "fv_dft.cuh"
+#include "fv_pair.cuh"
 
 namespace fv {
 
@@ -300,12 +301,16 @@ template cudaError_t launch_fft_pass<float>(const cpx<float> *, cpx<float> *, lo
                                             const cpx<float> *, cudaStream_t);
 
 // ---------------------------------------------------------------- compile-time lengths (fv_fft_fixed.cuh)
-#define FV_FIXED_ARGS const cpx<float> *in, cpx<float> *out, int rows, const DimGeom &dg, int P, int sP, int nz, int nzp, \
-                      const cpx<float> *twB, cudaStream_t st
-cudaError_t fft_fixed_a(FV_FIXED_ARGS);      // lengths up to 864
-cudaError_t fft_fixed_b(FV_FIXED_ARGS);      // up to 1728
-cudaError_t fft_fixed_c(FV_FIXED_ARGS);      // up to 2560
-cudaError_t fft_fixed_d(FV_FIXED_ARGS);      // up to 4096
+#define FV_FIXED_ARGS(G) const cpx<G> *in, cpx<G> *out, int rows, const DimGeom &dg, int P, int sP, int nz, int nzp, \
+                         const cpx<G> *twB, cudaStream_t st
+cudaError_t fft_fixed_a(FV_FIXED_ARGS(float));      // lengths up to 864
+cudaError_t fft_fixed_b(FV_FIXED_ARGS(float));      // up to 1728
+cudaError_t fft_fixed_c(FV_FIXED_ARGS(float));      // up to 2560
+cudaError_t fft_fixed_d(FV_FIXED_ARGS(float));      // up to 4096
+cudaError_t fft_pairs_a(FV_FIXED_ARGS(Pf));
+cudaError_t fft_pairs_b(FV_FIXED_ARGS(Pf));
+cudaError_t fft_pairs_c(FV_FIXED_ARGS(Pf));
+cudaError_t fft_pairs_d(FV_FIXED_ARGS(Pf));
 
 struct FixedLength { short M, R2, R3; };
 // every product 16 R2 R3 up to 4096 of the radices 4, 5, 6, 8, 9, 10, 12, 15, 16, at most 17 % apart above 480
@@ -334,7 +339,7 @@ bool fft_choose_fixed(int target, int *radix, int &nstages, int &M)
 size_t fft_fixed_table(const DimGeom &dg) { return (size_t)16 * dg.radix[1] + dg.M; }
 
 // tb[q 16 + m1] = e^{2 pi i q m1 / (16 R2)}, then tc[q 16 R2 + c] = e^{2 pi i q c / M}
-__global__ void k_fixed_twiddles(cpx<float> *tw, int M, int R2)
+template <class G> __global__ void k_fixed_twiddles(cpx<G> *tw, int M, int R2)
 {
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
     const int nB = 16 * R2;
@@ -346,27 +351,41 @@ __global__ void k_fixed_twiddles(cpx<float> *tw, int M, int R2)
         const int j = k - nB;
         sincospi(2.0 * (double)((j / nB) * (j % nB)) / (double)M, &s, &c);
     }
-    tw[k] = cmk<float>((float)c, (float)s);
+    tw[k] = cmk<G>((G)c, (G)s);
 }
 
-cudaError_t launch_fixed_twiddles(cpx<float> *tw, const DimGeom &dg, cudaStream_t st)
+template <class G> cudaError_t launch_fixed_twiddles(cpx<G> *tw, const DimGeom &dg, cudaStream_t st)
 {
     const int n = (int)fft_fixed_table(dg);
-    k_fixed_twiddles<<<(n + 255) / 256, 256, 0, st>>>(tw, dg.M, dg.radix[1]);
+    k_fixed_twiddles<G><<<(n + 255) / 256, 256, 0, st>>>(tw, dg.M, dg.radix[1]);
     return cudaGetLastError();
 }
+template cudaError_t launch_fixed_twiddles<float>(cpx<float> *, const DimGeom &, cudaStream_t);
+template cudaError_t launch_fixed_twiddles<Pf>(cpx<Pf> *, const DimGeom &, cudaStream_t);
 
-cudaError_t launch_fft_fixed(const cpx<float> *in, cpx<float> *out, long rows, const DimGeom &dg, int P, int sP, int nz,
-                             int nzp, const cpx<float> *tw, cudaStream_t st)
+template <class G>
+cudaError_t launch_fft_fixed(const cpx<G> *in, cpx<G> *out, long rows, const DimGeom &dg, int P, int sP, int nz, int nzp,
+                             const cpx<G> *tw, cudaStream_t st)
 {
     if (rows <= 0) return cudaSuccess;
     if (rows > (1L << 30) || P < 1 || nz < 1) return cudaErrorInvalidValue;
     const int r = (int)rows;
-    if (dg.M <= 864) return fft_fixed_a(in, out, r, dg, P, sP, nz, nzp, tw, st);
-    if (dg.M <= 1728) return fft_fixed_b(in, out, r, dg, P, sP, nz, nzp, tw, st);
-    if (dg.M <= 2560) return fft_fixed_c(in, out, r, dg, P, sP, nz, nzp, tw, st);
-    return fft_fixed_d(in, out, r, dg, P, sP, nz, nzp, tw, st);
+    if constexpr (sizeof(G) == 4) {
+        if (dg.M <= 864) return fft_fixed_a(in, out, r, dg, P, sP, nz, nzp, tw, st);
+        if (dg.M <= 1728) return fft_fixed_b(in, out, r, dg, P, sP, nz, nzp, tw, st);
+        if (dg.M <= 2560) return fft_fixed_c(in, out, r, dg, P, sP, nz, nzp, tw, st);
+        return fft_fixed_d(in, out, r, dg, P, sP, nz, nzp, tw, st);
+    } else {
+        if (dg.M <= 864) return fft_pairs_a(in, out, r, dg, P, sP, nz, nzp, tw, st);
+        if (dg.M <= 1728) return fft_pairs_b(in, out, r, dg, P, sP, nz, nzp, tw, st);
+        if (dg.M <= 2560) return fft_pairs_c(in, out, r, dg, P, sP, nz, nzp, tw, st);
+        return fft_pairs_d(in, out, r, dg, P, sP, nz, nzp, tw, st);
+    }
 }
+template cudaError_t launch_fft_fixed<float>(const cpx<float> *, cpx<float> *, long, const DimGeom &, int, int, int, int,
+                                             const cpx<float> *, cudaStream_t);
+template cudaError_t launch_fft_fixed<Pf>(const cpx<Pf> *, cpx<Pf> *, long, const DimGeom &, int, int, int, int,
+                                          const cpx<Pf> *, cudaStream_t);
 
 // ---------------------------------------------------------------- host planning
 static const int kRadices[] = {16, 15, 12, 10, 9, 8, 6, 5, 4, 3, 2};

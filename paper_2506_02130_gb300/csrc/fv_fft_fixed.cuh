@@ -1,4 +1,4 @@
-// FFT passes of FP32 grids with compile-time lengths M = 16 R2 R3 (M >= 2 N, no prescale): the same transform as
+// FFT passes of FP32 grids, and of grids of float pairs (G = Pf: FP64 plans), with compile-time lengths M = 16 R2 R3 (M >= 2 N, no prescale): the same transform as
 // k_fft_rows (zero-padded rows of N values at l - N/2 mod M, sign +, band of outputs m in [-H, B-1-H], written
 // transposed as out[b][row]).
 //
@@ -20,66 +20,68 @@
 // 55 + 50, 127-antenna workload with 8 height terms 17 + 16 against 38 + 36.
 #pragma once
 #include "fv_dft.cuh"
+#include "fv_pair.cuh"
 
 namespace fv {
 
-template <int R2, int R3> struct FixedFft {
+template <class G, int R2, int R3> struct FixedFft {
+    static constexpr bool P = sizeof(G) == 8;                    // pairs: 16 bytes a value, twice the registers
     static constexpr int M = 16 * R2 * R3;
-    static constexpr int R = M <= 3072 ? 4 : 2;                 // rows a CTA
+    static constexpr int R = P ? (M <= 2304 ? 2 : 1) : (M <= 3072 ? 4 : 2);     // rows a CTA (32 bytes of a transposed store)
     static constexpr int S3 = R3 | 1, S1 = (R2 * S3) | 1;       // strides of n2 and m1
-    static constexpr int kOff = R == 4 ? 4 : 8;
+    static constexpr int kOff = R == 4 || P ? 4 : 8;             // pairs move 8 lanes at a time, others 16
     static constexpr int S0 = (16 * S1 + 15 - kOff) / 16 * 16 + kOff;   // of a row: kOff modulo 16
     static constexpr int items = R * M / 16;
     static constexpr int rounds = items <= 320 ? 1 : (items <= 768 ? 2 : 3);
     static constexpr int T = (items + 32 * rounds - 1) / (32 * rounds) * 32;
-    static constexpr int smem = R * S0 * 8;
-    static constexpr int by_smem = 225000 / (smem + 1024), by_regs = 65536 / (T * 80);
+    static constexpr int smem = R * S0 * 2 * (int)sizeof(G);
+    static constexpr int by_smem = 225000 / (smem + 1024), by_regs = 65536 / (T * (P ? 160 : 80));
     static constexpr int blocks = by_smem < by_regs ? (by_smem > 0 ? by_smem : 1) : (by_regs > 0 ? by_regs : 1);
     static constexpr int keep = R3 / 4;                          // outputs m3 <= keep and m3 >= R3 - 1 - keep
 };
 
 // first-stage DFT of 16 points of which 4..11 are zero: v[0..3] = points 0..3, v[4..7] = points 12..15
-__device__ __forceinline__ void dft16_half(const cpx<float> *v, cpx<float> *o)
+template <class G> __device__ __forceinline__ void dft16_half(const cpx<G> *v, cpx<G> *o)
 {
-    using C = cpx<float>;
+    using C = cpx<G>;
     C U[4][4];
     auto column = [&](const int r2, C a, C d) {
         // points r2 (r1 = 0) and 12 + r2 (r1 = 3): a + d e^{2 pi i 3 q / 4}
         U[r2][0] = cadd(a, d);
-        U[r2][1] = cmk<float>(a.x + d.y, a.y - d.x);
+        U[r2][1] = cmk<G>(a.x + d.y, a.y - d.x);
         U[r2][2] = csub(a, d);
-        U[r2][3] = cmk<float>(a.x - d.y, a.y + d.x);
+        U[r2][3] = cmk<G>(a.x - d.y, a.y + d.x);
     };
     column(0, v[0], v[4]);
     column(1, v[1], v[5]);
     column(2, v[2], v[6]);
     column(3, v[3], v[7]);
-    U[1][1] = twm<float, 1, 16>(U[1][1]);
-    U[1][2] = twm<float, 2, 16>(U[1][2]);
-    U[1][3] = twm<float, 3, 16>(U[1][3]);
-    U[2][1] = twm<float, 2, 16>(U[2][1]);
-    U[2][2] = twm<float, 4, 16>(U[2][2]);
-    U[2][3] = twm<float, 6, 16>(U[2][3]);
-    U[3][1] = twm<float, 3, 16>(U[3][1]);
-    U[3][2] = twm<float, 6, 16>(U[3][2]);
-    U[3][3] = twm<float, 9, 16>(U[3][3]);
+    U[1][1] = twm<G, 1, 16>(U[1][1]);
+    U[1][2] = twm<G, 2, 16>(U[1][2]);
+    U[1][3] = twm<G, 3, 16>(U[1][3]);
+    U[2][1] = twm<G, 2, 16>(U[2][1]);
+    U[2][2] = twm<G, 4, 16>(U[2][2]);
+    U[2][3] = twm<G, 6, 16>(U[2][3]);
+    U[3][1] = twm<G, 3, 16>(U[3][1]);
+    U[3][2] = twm<G, 6, 16>(U[3][2]);
+    U[3][3] = twm<G, 9, 16>(U[3][3]);
 #pragma unroll
     for (int q1 = 0; q1 < 4; ++q1) {
         C t[4] = {U[0][q1], U[1][q1], U[2][q1], U[3][q1]};
-        Dft<float, 4>::run(t);
+        Dft<G, 4>::run(t);
 #pragma unroll
         for (int q2 = 0; q2 < 4; ++q2) o[q1 + 4 * q2] = t[q2];
     }
 }
 
 // rows (y, p), y = row / P, p = row % P: value l at in[(y N + l) sP + (p / nz) nzp + p % nz]
-template <int R2, int R3>
-__global__ void __launch_bounds__((FixedFft<R2, R3>::T), (FixedFft<R2, R3>::blocks))
-    k_fft_fixed(const cpx<float> *__restrict__ in, cpx<float> *__restrict__ out, int rows, int N, int H, int B, int P,
-                int sP, int nz, int nzp, const cpx<float> *__restrict__ twB, const cpx<float> *__restrict__ twC)
+template <class G, int R2, int R3>
+__global__ void __launch_bounds__((FixedFft<G, R2, R3>::T), (FixedFft<G, R2, R3>::blocks))
+    k_fft_fixed(const cpx<G> *__restrict__ in, cpx<G> *__restrict__ out, int rows, int N, int H, int B, int P,
+                int sP, int nz, int nzp, const cpx<G> *__restrict__ twB, const cpx<G> *__restrict__ twC)
 {
-    using F = FixedFft<R2, R3>;
-    using C = cpx<float>;
+    using F = FixedFft<G, R2, R3>;
+    using C = cpx<G>;
     constexpr int M = F::M, R = F::R, T = F::T, S0 = F::S0, S1 = F::S1, S3 = F::S3, MB = R2 * R3;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     C *buf = reinterpret_cast<C *>(smem_raw);
@@ -99,12 +101,12 @@ __global__ void __launch_bounds__((FixedFft<R2, R3>::T), (FixedFft<R2, R3>::bloc
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
                 const int pos = j + q * MB;                                     // l - N/2
-                v[q] = live && pos < N - half ? src[(size_t)(pos + half) * sP] : cmk<float>(0.0f, 0.0f);
+                v[q] = live && pos < N - half ? src[(size_t)(pos + half) * sP] : cmk<G>((G)0.0, (G)0.0);
             }
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
                 const int l = j + (q - 4) * MB + half;
-                v[4 + q] = live && l >= 0 ? src[(size_t)l * sP] : cmk<float>(0.0f, 0.0f);
+                v[4 + q] = live && l >= 0 ? src[(size_t)l * sP] : cmk<G>((G)0.0, (G)0.0);
             }
             dft16_half(v, o);
             C *d = mine + (j / R3) * S3 + j % R3;
@@ -125,7 +127,7 @@ __global__ void __launch_bounds__((FixedFft<R2, R3>::T), (FixedFft<R2, R3>::bloc
             v[0] = d[0];
 #pragma unroll
             for (int q = 1; q < R2; ++q) v[q] = cmul(d[q * S3], twB[q * 16 + m1]);
-            Dft<float, R2>::run(v);
+            Dft<G, R2>::run(v);
 #pragma unroll
             for (int q = 0; q < R2; ++q) d[q * S3] = v[q];
         }
@@ -142,7 +144,7 @@ __global__ void __launch_bounds__((FixedFft<R2, R3>::T), (FixedFft<R2, R3>::bloc
             v[0] = d[0];
 #pragma unroll
             for (int q = 1; q < R3; ++q) v[q] = cmul(d[q], twC[q * items + c]);
-            Dft<float, R3>::run(v);
+            Dft<G, R3>::run(v);
             if (!live) continue;
 #pragma unroll
             for (int q = 0; q <= F::keep; ++q) {
@@ -158,11 +160,11 @@ __global__ void __launch_bounds__((FixedFft<R2, R3>::T), (FixedFft<R2, R3>::bloc
     }
 }
 
-template <int R2, int R3>
-cudaError_t fft_fixed_go(const cpx<float> *in, cpx<float> *out, int rows, const DimGeom &dg, int P, int sP, int nz,
-                         int nzp, const cpx<float> *twB, cudaStream_t st)
+template <class G, int R2, int R3>
+cudaError_t fft_fixed_go(const cpx<G> *in, cpx<G> *out, int rows, const DimGeom &dg, int P, int sP, int nz, int nzp,
+                         const cpx<G> *twB, cudaStream_t st)
 {
-    using F = FixedFft<R2, R3>;
+    using F = FixedFft<G, R2, R3>;
     static_assert(F::T % F::R == 0 && F::T <= 1024, "a thread keeps one row");
     // what the kernel leaves out has to be empty: the row within half of M, the band within the kept outputs
     constexpr int third = 16 * R2;
@@ -174,11 +176,11 @@ cudaError_t fft_fixed_go(const cpx<float> *in, cpx<float> *out, int rows, const 
     if (e != cudaSuccess) return e;
     if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
     if (!attr_set[dev]) {
-        e = cudaFuncSetAttribute(k_fft_fixed<R2, R3>, cudaFuncAttributeMaxDynamicSharedMemorySize, F::smem);
+        e = cudaFuncSetAttribute(k_fft_fixed<G, R2, R3>, cudaFuncAttributeMaxDynamicSharedMemorySize, F::smem);
         if (e != cudaSuccess) return e;
         attr_set[dev] = true;
     }
-    k_fft_fixed<R2, R3><<<(rows + F::R - 1) / F::R, F::T, F::smem, st>>>(in, out, rows, dg.nf1, dg.H, dg.B, P, sP, nz,
+    k_fft_fixed<G, R2, R3><<<(rows + F::R - 1) / F::R, F::T, F::smem, st>>>(in, out, rows, dg.nf1, dg.H, dg.B, P, sP, nz,
                                                                         nzp, twB, twB + 16 * R2);
     return cudaGetLastError();
 }

@@ -1,5 +1,5 @@
-// Instances of the compile-time-length FFT pass, lengths 1920 to 2560 (one translation unit of several, so that
-// they compile side by side).
+// Instances of the compile-time-length FFT pass, lengths 1920 to 2560 (one translation unit of several, so
+// that they compile side by side).
 #include "fv_fft_fixed.cuh"
 
 namespace fv {
@@ -8,12 +8,12 @@ cudaError_t fft_fixed_c(const cpx<float> *in, cpx<float> *out, int rows, const D
                         int nzp, const cpx<float> *twB, cudaStream_t st)
 {
     switch (dg.M) {
-    case 1920: return fft_fixed_go<12, 10>(in, out, rows, dg, P, sP, nz, nzp, twB, st);
-    case 2048: return fft_fixed_go<16, 8>(in, out, rows, dg, P, sP, nz, nzp, twB, st);
-    case 2160: return fft_fixed_go<15, 9>(in, out, rows, dg, P, sP, nz, nzp, twB, st);
-    case 2304: return fft_fixed_go<12, 12>(in, out, rows, dg, P, sP, nz, nzp, twB, st);
-    case 2400: return fft_fixed_go<15, 10>(in, out, rows, dg, P, sP, nz, nzp, twB, st);
-    case 2560: return fft_fixed_go<16, 10>(in, out, rows, dg, P, sP, nz, nzp, twB, st);
+    case 1920: return fft_fixed_go<float, 12, 10>(in, out, rows, dg, P, sP, nz, nzp, twB, st);
+    case 2048: return fft_fixed_go<float, 16, 8>(in, out, rows, dg, P, sP, nz, nzp, twB, st);
+    case 2160: return fft_fixed_go<float, 15, 9>(in, out, rows, dg, P, sP, nz, nzp, twB, st);
+    case 2304: return fft_fixed_go<float, 12, 12>(in, out, rows, dg, P, sP, nz, nzp, twB, st);
+    case 2400: return fft_fixed_go<float, 15, 10>(in, out, rows, dg, P, sP, nz, nzp, twB, st);
+    case 2560: return fft_fixed_go<float, 16, 10>(in, out, rows, dg, P, sP, nz, nzp, twB, st);
     default: return cudaErrorInvalidValue;
     }
 }

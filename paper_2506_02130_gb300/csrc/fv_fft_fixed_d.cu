@@ -1,5 +1,5 @@
-// Instances of the compile-time-length FFT pass, lengths 2880 to 4096 (one translation unit of several, so that
-// they compile side by side).
+// Instances of the compile-time-length FFT pass, lengths 2880 to 4096 (one translation unit of several, so
+// that they compile side by side).
 #include "fv_fft_fixed.cuh"
 
 namespace fv {
@@ -8,11 +8,11 @@ cudaError_t fft_fixed_d(const cpx<float> *in, cpx<float> *out, int rows, const D
                         int nzp, const cpx<float> *twB, cudaStream_t st)
 {
     switch (dg.M) {
-    case 2880: return fft_fixed_go<15, 12>(in, out, rows, dg, P, sP, nz, nzp, twB, st);
-    case 3072: return fft_fixed_go<16, 12>(in, out, rows, dg, P, sP, nz, nzp, twB, st);
-    case 3600: return fft_fixed_go<15, 15>(in, out, rows, dg, P, sP, nz, nzp, twB, st);
-    case 3840: return fft_fixed_go<16, 15>(in, out, rows, dg, P, sP, nz, nzp, twB, st);
-    case 4096: return fft_fixed_go<16, 16>(in, out, rows, dg, P, sP, nz, nzp, twB, st);
+    case 2880: return fft_fixed_go<float, 15, 12>(in, out, rows, dg, P, sP, nz, nzp, twB, st);
+    case 3072: return fft_fixed_go<float, 16, 12>(in, out, rows, dg, P, sP, nz, nzp, twB, st);
+    case 3600: return fft_fixed_go<float, 15, 15>(in, out, rows, dg, P, sP, nz, nzp, twB, st);
+    case 3840: return fft_fixed_go<float, 16, 15>(in, out, rows, dg, P, sP, nz, nzp, twB, st);
+    case 4096: return fft_fixed_go<float, 16, 16>(in, out, rows, dg, P, sP, nz, nzp, twB, st);
     default: return cudaErrorInvalidValue;
     }
 }

@@ -1,0 +1,27 @@
+// Instances of the compile-time-length FFT pass on pairs of floats, lengths 256 to 864 (one translation unit of several, so
+// that they compile side by side).
+#include "fv_fft_fixed.cuh"
+
+namespace fv {
+
+cudaError_t fft_pairs_a(const cpx<Pf> *in, cpx<Pf> *out, int rows, const DimGeom &dg, int P, int sP, int nz,
+                        int nzp, const cpx<Pf> *twB, cudaStream_t st)
+{
+    switch (dg.M) {
+    case 256: return fft_fixed_go<Pf, 4, 4>(in, out, rows, dg, P, sP, nz, nzp, twB, st);
+    case 320: return fft_fixed_go<Pf, 5, 4>(in, out, rows, dg, P, sP, nz, nzp, twB, st);
+    case 384: return fft_fixed_go<Pf, 6, 4>(in, out, rows, dg, P, sP, nz, nzp, twB, st);
+    case 400: return fft_fixed_go<Pf, 5, 5>(in, out, rows, dg, P, sP, nz, nzp, twB, st);
+    case 480: return fft_fixed_go<Pf, 6, 5>(in, out, rows, dg, P, sP, nz, nzp, twB, st);
+    case 512: return fft_fixed_go<Pf, 8, 4>(in, out, rows, dg, P, sP, nz, nzp, twB, st);
+    case 576: return fft_fixed_go<Pf, 6, 6>(in, out, rows, dg, P, sP, nz, nzp, twB, st);
+    case 640: return fft_fixed_go<Pf, 8, 5>(in, out, rows, dg, P, sP, nz, nzp, twB, st);
+    case 720: return fft_fixed_go<Pf, 9, 5>(in, out, rows, dg, P, sP, nz, nzp, twB, st);
+    case 768: return fft_fixed_go<Pf, 8, 6>(in, out, rows, dg, P, sP, nz, nzp, twB, st);
+    case 800: return fft_fixed_go<Pf, 10, 5>(in, out, rows, dg, P, sP, nz, nzp, twB, st);
+    case 864: return fft_fixed_go<Pf, 9, 6>(in, out, rows, dg, P, sP, nz, nzp, twB, st);
+    default: return cudaErrorInvalidValue;
+    }
+}
+
+}  // namespace fv

@@ -528,12 +528,14 @@ cudaError_t launch_fft_pass(const cpx<G> *in, cpx<G> *out, long rows, const DimG
 // The same pass for FP32 rows of a compile-time length (dg.fixed; M >= 2 N, no prescale): row r = (y, p) with
 // P = rows per y, its value l at in[(y N + l) sP + (p / nz) nzp + p % nz] (P = sP = nz = nzp = 1: contiguous rows).
 // tw: the tables of launch_fixed_twiddles (fft_fixed_table complex values).
-cudaError_t launch_fft_fixed(const cpx<float> *in, cpx<float> *out, long rows, const DimGeom &dg, int P, int sP, int nz,
-                             int nzp, const cpx<float> *tw, cudaStream_t st);
+// G: float, or Pf for grids of float pairs.
+template <class G>
+cudaError_t launch_fft_fixed(const cpx<G> *in, cpx<G> *out, long rows, const DimGeom &dg, int P, int sP, int nz, int nzp,
+                             const cpx<G> *tw, cudaStream_t st);
 // The smallest compile-time length M >= target, or false (target above 4096).
 bool fft_choose_fixed(int target, int *radix, int &nstages, int &M);
 size_t fft_fixed_table(const DimGeom &dg);
-cudaError_t launch_fixed_twiddles(cpx<float> *tw, const DimGeom &dg, cudaStream_t st);
+template <class G> cudaError_t launch_fixed_twiddles(cpx<G> *tw, const DimGeom &dg, cudaStream_t st);
 
 // Interpolation at the unique targets, deconvolution and postphase: Vu[u][pol] (FP64).
 template <class G>
@@ -548,6 +550,34 @@ struct SliceOut {
     const int *u_off, *u_bl;
     int u_base;
 };
+
+// The NP values of a target to its nb baselines u_bl[b0 ..): out[b][p].  Four indexes are read ahead of their
+// stores: the shortest baseline of a regular array has hundreds of copies, and its warp sets the launch's length.
+template <class G, int NP>
+__device__ __forceinline__ void write_target(const SliceOut &so, int b0, int nb, const G *rx, const G *ry, int lane)
+{
+    cpx<G> *o = reinterpret_cast<cpx<G> *>(so.out);
+    const int p = NP == 1 ? 0 : lane & 3;            // the same for every value of a lane
+    G vx = rx[0], vy = ry[0];
+#pragma unroll
+    for (int q = 1; q < NP; ++q)
+        if (p == q) {
+            vx = rx[q];
+            vy = ry[q];
+        }
+    const int n = nb * NP;
+    for (int k = lane; k < n; k += 128) {
+        int b[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const int kk = k + 32 * j;
+            b[j] = kk < n ? so.u_bl[b0 + (NP == 1 ? kk : kk >> 2)] : -1;
+        }
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+            if (b[j] >= 0) o[(size_t)b[j] * NP + p] = cmk<G>(vx, vy);
+    }
+}
 
 // Whether launch_interp_zdirect can write a slice's output itself for this geometry and grid precision
 // (two-dimensional grids without height terms; FP32 grids with an even number of planes per cell).

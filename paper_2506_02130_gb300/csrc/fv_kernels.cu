@@ -575,34 +575,6 @@ __device__ __forceinline__ void target_setup(const SliceGeom &g, long u, int &m0
     phr = fmaf(-k, -1.7484555e-7f, fmaf(-k, 6.2831855f, qh)) - ql;
 }
 
-// The NP values of a target to its nb baselines u_bl[b0 ..): out[b][p].  Four indexes are read ahead of their
-// stores: the shortest baseline of a regular array has hundreds of copies, and its warp sets the launch's length.
-template <class G, int NP>
-__device__ __forceinline__ void write_target(const SliceOut &so, int b0, int nb, const G *rx, const G *ry, int lane)
-{
-    cpx<G> *o = reinterpret_cast<cpx<G> *>(so.out);
-    const int p = NP == 1 ? 0 : lane & 3;            // the same for every value of a lane
-    G vx = rx[0], vy = ry[0];
-#pragma unroll
-    for (int q = 1; q < NP; ++q)
-        if (p == q) {
-            vx = rx[q];
-            vy = ry[q];
-        }
-    const int n = nb * NP;
-    for (int k = lane; k < n; k += 128) {
-        int b[4];
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const int kk = k + 32 * j;
-            b[j] = kk < n ? so.u_bl[b0 + (NP == 1 ? kk : kk >> 2)] : -1;
-        }
-#pragma unroll
-        for (int j = 0; j < 4; ++j)
-            if (b[j] >= 0) o[(size_t)b[j] * NP + p] = cmk<G>(vx, vy);
-    }
-}
-
 // 2-D interpolation with one warp per target.  Lane 0 computes the target's FP64 quantities (coordinate
 // on the FFT grid, first footprint cell, offset, postphase argument reduced to [-pi, pi]); lanes
 // (dx, j) = (lane / J, lane % J), J = 32 / w, then cover footprint column dx and, with four products,

@@ -33,14 +33,6 @@ namespace {
 constexpr int kDenseThreads = 256;
 constexpr int kDenseChain = 256;          // sources an FP32 sum takes before it goes to the FP64 sums
 
-__device__ __forceinline__ float2 dup(float v) { return make_float2(v, v); }
-__device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a, b); }
-__device__ __forceinline__ float2 sub2(float2 a, float2 b) { return __ffma2_rn(b, make_float2(-1.0f, -1.0f), a); }
-__device__ __forceinline__ float2 neg2(float2 a) { return __fmul2_rn(a, make_float2(-1.0f, -1.0f)); }
-
-// two pairs of floats side by side (the real and imaginary part)
-struct Pair2 { float2 h, l; };
-
 // the arithmetic of one precision: values in shared memory and the thread's sums
 template <class G> struct Dense;
 template <> struct Dense<float> {
@@ -64,23 +56,13 @@ template <> struct Dense<double> {
     using Acc = Pair2;
     using E = Pair2;
     static __device__ __forceinline__ Acc zero() { return Pair2{make_float2(0.0f, 0.0f), make_float2(0.0f, 0.0f)}; }
-    // p = a b: the rounded product and its error, with the low parts' cross terms
-    static __device__ __forceinline__ Pair2 times(float2 ah, float2 al, float2 bh, float2 bl)
-    {
-        Pair2 r;
-        r.h = __fmul2_rn(ah, bh);
-        r.l = __ffma2_rn(ah, bh, neg2(r.h));
-        r.l = __ffma2_rn(ah, bl, r.l);
-        r.l = __ffma2_rn(al, bh, r.l);
-        return r;
-    }
     static __device__ __forceinline__ E product(const float4 *e, const float4 *b)
     {
         const float4 eh = e[0], el = e[1], bh = b[0], bl = b[1];
-        const Pair2 p = times(make_float2(eh.x, eh.y), make_float2(el.x, el.y), make_float2(bh.x, bh.y),
-                              make_float2(bl.x, bl.y));
-        const Pair2 q = times(make_float2(eh.z, eh.w), make_float2(el.z, el.w), make_float2(bh.z, bh.w),
-                              make_float2(bl.z, bl.w));
+        const Pair2 p = pair2_times(make_float2(eh.x, eh.y), make_float2(el.x, el.y), make_float2(bh.x, bh.y),
+                                    make_float2(bl.x, bl.y));
+        const Pair2 q = pair2_times(make_float2(eh.z, eh.w), make_float2(el.z, el.w), make_float2(bh.z, bh.w),
+                                    make_float2(bl.z, bl.w));
         const float2 s = add2(p.h, q.h), t = sub2(s, p.h);
         const float2 l = add2(add2(add2(sub2(p.h, sub2(s, t)), sub2(q.h, t)), p.l), q.l);
         E r;
@@ -90,17 +72,9 @@ template <> struct Dense<double> {
     }
     static __device__ __forceinline__ void add(Acc &a, const float2 *w, const E &e)
     {
-        const Pair2 p = times(w[0], w[1], e.h, e.l);
-        const float2 s = add2(a.h, p.h), t = sub2(s, a.h);
-        a.l = add2(a.l, add2(add2(sub2(a.h, sub2(s, t)), sub2(p.h, t)), p.l));
-        a.h = s;
+        pair2_add(a, pair2_times(w[0], w[1], e.h, e.l));
     }
-    static __device__ __forceinline__ void join(Acc &a, const Acc &b)
-    {
-        const float2 s = add2(a.h, b.h), t = sub2(s, a.h);
-        a.l = add2(add2(a.l, b.l), add2(sub2(a.h, sub2(s, t)), sub2(b.h, t)));
-        a.h = s;
-    }
+    static __device__ __forceinline__ void join(Acc &a, const Acc &b) { pair2_add(a, b); }
     static __device__ __forceinline__ cpx<double> value(const Acc &a)
     {
         return cmk<double>((double)a.h.x + (double)a.l.x, (double)a.h.y + (double)a.l.y);
@@ -162,6 +136,44 @@ __global__ void __launch_bounds__(kDenseThreads, 2)
 #pragma unroll
             for (int b = 0; b < TB; ++b) acc[j][a][b] = D::zero();
     int held = 0;                                                          // sources in the thread's sums
+    // FP64: the sums' power of two (pair_shift of each block of sources; a block with another one starts new sums)
+    __shared__ unsigned s_key[2];
+    int shift = 0, par = 0;
+    double up = 1.0, down = 1.0;
+    if constexpr (sizeof(G) == 8) {
+        if (threadIdx.x < 2) s_key[threadIdx.x] = 0u;
+        __syncthreads();
+    }
+    // the sums to the FP64 sums in memory: the groups' are added up through shared memory first (over the tables),
+    // since every group and CTA adds to the same few hundred modes
+    auto flush = [&]() {
+        typename D::Acc *buf = reinterpret_cast<typename D::Acc *>(smem_raw);
+#pragma unroll
+        for (int j = 0; j < JB; ++j) {
+            if (j >= nj) break;
+#pragma unroll
+            for (int i = 0; i < TA; ++i) {
+                __syncthreads();
+#pragma unroll
+                for (int k = 0; k < TB; ++k) {
+                    if (work) buf[threadIdx.x * TB + k] = acc[j][i][k];
+                    acc[j][i][k] = D::zero();
+                }
+                __syncthreads();
+                for (int o = threadIdx.x; o < tiles * TB; o += kDenseThreads) {
+                    const int t = dg.tiles[tile0 + o / TB];
+                    const int row = (t & 0xffff) + i, col = (t >> 16) + o % TB;
+                    if (row >= n2 || col >= n1) continue;
+                    typename D::Acc v = buf[o];
+                    for (int q = 1; q < groups; ++q) D::join(v, buf[q * tiles * TB + o]);
+                    const cpx<double> r = D::value(v);
+                    cpx<double> *d = out + ((size_t)(j0 + j) * n2 + row) * n1 + col;
+                    atomicAdd(&d->x, sizeof(G) == 8 ? r.x * down : r.x);
+                    atomicAdd(&d->y, sizeof(G) == 8 ? r.y * down : r.y);
+                }
+            }
+        }
+    };
 
     for (int block = first; block < last; block += kDenseThreads) {
         const int nblk = min(kDenseThreads, last - block);
@@ -206,6 +218,13 @@ __global__ void __launch_bounds__(kDenseThreads, 2)
                 r[2] = c[1].x;                    // U'
                 r[3] = c[1].y;                    // V
             }
+            if constexpr (sizeof(G) == 8) {
+                const unsigned e = max(max(exponent_key(r[0]), exponent_key(r[1])),
+                                       max(exponent_key(r[2]), exponent_key(r[3])));
+                const unsigned lanes = __activemask();
+                const unsigned m = __reduce_max_sync(lanes, e);
+                if ((threadIdx.x & 31) == __ffs(lanes) - 1) atomicMax(&s_key[par], m);
+            }
             int p = j0 / dg.K, q = j0 - p * dg.K;
             G tm = u, t = (G)1;                   // T_{-1} = T_1, T_0
             for (int k = 0; k < q; ++k) {
@@ -230,6 +249,21 @@ __global__ void __launch_bounds__(kDenseThreads, 2)
             }
         }
         __syncthreads();
+        if constexpr (sizeof(G) == 8) {
+            const int sh = pair_shift(s_key[par]);
+            par ^= 1;
+            if (threadIdx.x == 0) s_key[par] = 0u;       // last read before the chunks' barriers of the block before
+            if (sh != shift) {                           // the same on every thread
+                if (held > 0) {
+                    flush();
+                    held = 0;
+                    __syncthreads();                     // the sums have been read: the tables may be written
+                }
+                shift = sh;
+                up = scalbn(1.0, sh);
+                down = scalbn(1.0, -sh);
+            }
+        }
         for (int base = 0; base < nblk; base += CS) {
             const int n = min(CS, nblk - base);
             // the chunk's tables: strengths, n_2 factors as (re, re, im, im), n_1 factors as (re, im, -im, re)
@@ -239,7 +273,7 @@ __global__ void __launch_bounds__(kDenseThreads, 2)
                 if constexpr (sizeof(G) == 4) {
                     w[0] = dup((float)v);
                 } else {
-                    const Pf y = pf((double)v);
+                    const Pf y = pf((double)v * up);
                     w[0] = dup(y.h);
                     w[1] = dup(y.l);
                 }
@@ -355,37 +389,10 @@ __global__ void __launch_bounds__(kDenseThreads, 2)
                 }
             }
             held += (n + groups - 1) / groups;
-            // to the FP64 sums in memory at the end, and in FP32 before a sum grows long (its rounding grows with the
-            // number of its terms): the groups' sums are added up through shared memory first, since every group and
-            // CTA adds to the same few hundred modes
+            // at the end, and in FP32 before a sum grows long (its rounding grows with the number of its terms)
             if (block + base + CS >= last || (sizeof(G) == 4 && held >= kDenseChain)) {
                 held = 0;
-                typename D::Acc *buf = reinterpret_cast<typename D::Acc *>(smem_raw);     // over the tables
-#pragma unroll
-                for (int j = 0; j < JB; ++j) {
-                    if (j >= nj) break;
-#pragma unroll
-                    for (int i = 0; i < TA; ++i) {
-                        __syncthreads();
-#pragma unroll
-                        for (int k = 0; k < TB; ++k) {
-                            if (work) buf[threadIdx.x * TB + k] = acc[j][i][k];
-                            acc[j][i][k] = D::zero();
-                        }
-                        __syncthreads();
-                        for (int o = threadIdx.x; o < tiles * TB; o += kDenseThreads) {
-                            const int t = dg.tiles[tile0 + o / TB];
-                            const int row = (t & 0xffff) + i, col = (t >> 16) + o % TB;
-                            if (row >= n2 || col >= n1) continue;
-                            typename D::Acc v = buf[o];
-                            for (int q = 1; q < groups; ++q) D::join(v, buf[q * tiles * TB + o]);
-                            const cpx<double> r = D::value(v);
-                            cpx<double> *d = out + ((size_t)(j0 + j) * n2 + row) * n1 + col;
-                            atomicAdd(&d->x, r.x);
-                            atomicAdd(&d->y, r.y);
-                        }
-                    }
-                }
+                flush();
             }
             __syncthreads();                          // the chunk's tables have been read
         }

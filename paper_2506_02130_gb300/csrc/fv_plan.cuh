@@ -4,6 +4,7 @@
 #include "../../include/fv.h"
 #include "fv_internal.cuh"
 #include "fv_lattice_dense.cuh"
+#include "fv_pairs.cuh"
 
 #include <string>
 #include <utility>
@@ -112,6 +113,7 @@ struct fv_plan_s {
         double *sdir = nullptr;
         void *frac = nullptr, *cs = nullptr;
         float4 *rec = nullptr;    // per-time records of the direct mode sums (launch_time_compact)
+        void *pairs = nullptr;    // FP64 in pairs: the strengths' exponent (256 bytes), then targets and their weights
         float4 *tc = nullptr;     // per-time coordinate records of the sorted sources (FP32 grids)
         int *tiles = nullptr;     // ring gather: ticket and work-list counts (reset by the prep kernel)
         // ring gather work list (fv_spread_ring.cu): tiles' bin rectangles, unsplit tiles, parts of split
@@ -132,6 +134,8 @@ struct fv_plan_s {
         bool tc = false;                               // per-time coordinate records (48 bytes per source)
         bool rec = false;                              // direct mode sums in FP32: their records (32 bytes per source)
         bool dirs = true;                              //   in place of directions and cells
+        bool cells = true;                             // cells beside the directions (not for FP64 pairs' records)
+        size_t pairs = 0;                              // FP64 in pairs: targets of one launch and strengths' exponent
         int ring_tiles = 0, ring_slots = 0, ring_np = 0; // ring gather: tiles of the largest grid, part slots, n_pol
     } need;
     int n_streams = 1;
@@ -143,7 +147,12 @@ struct fv_plan_s {
     int spread_req = 0;         // fv_opts.spread_method
     int fft_max_radix = 16;
     int spread_method = 0;      // resolved method
+    int general_method = 0;     //   before the forms that fix it (pairs), for general_bytes
+    bool ring_ok = false;       //   the general form's gather is the ring
     bool ring = false;          // FP32 2-D gather through the shared-memory ring (fv_spread_ring.cu)
+    bool pairs = false;         // FP64 slices in pairs of floats (fv_pairs.cu)
+    fv::PairPoly pair_poly{};   //   their kernel values as polynomials
+    int pair_chunk = 0;         //   targets one interpolation launch takes
     bool xy_fixed = false;      // every channel's x and y FFT lengths are compile-time lengths (launch_fft_fixed)
     bool strip = false;         // FP32 gather plans, w <= 7: preparation and spreading in one pass (fv_spread_strip.cu)
     fv::EsPoly es_poly{};       //   its kernel values as polynomials
@@ -205,6 +214,7 @@ struct fv_plan_s {
     unsigned long long gen = 0;
 
     long long ws_bytes = 0;
+    size_t static_need = 0;          // bytes by which the static scratch takes or refuses the plan (general_bytes)
     std::vector<long> geo_sig;       // sizes behind the current tables and workspaces
     int nf1_max[3] = {1, 1, 1}, M_max[3] = {1, 1, 1};
 

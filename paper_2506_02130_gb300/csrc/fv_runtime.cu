@@ -158,9 +158,9 @@ size_t workspace_layout(const fv_plan_s::WsNeed &need, char *base, fv_plan_s::Wo
     };
     fv_plan_s::Workspace tmp;
     fv_plan_s::Workspace &o = w ? *w : tmp;
-    o.grid = take(need.grid);
+    // the grid is dead once the first FFT pass has read it: the second band takes its place
+    o.grid = o.bufB = take(std::max(need.grid, need.bufB));
     o.bufA = take(need.bufA);
-    o.bufB = take(need.bufB);
     o.Vu = (cpx<double> *)take(need.vu);
     if (need.tiled) {
         const size_t ns = (size_t)need.n_src, nb = (size_t)need.nb;
@@ -169,7 +169,7 @@ size_t workspace_layout(const fv_plan_s::WsNeed &need, char *base, fv_plan_s::Wo
         o.offsets = (int *)take((nb + 1) * sizeof(int));
         o.cursor = (int *)take(nb * sizeof(int));
         o.sidx = (int *)take(ns * sizeof(int));
-        o.cell = need.dirs ? (int *)take(3 * ns * sizeof(int)) : nullptr;
+        o.cell = need.dirs && need.cells ? (int *)take(3 * ns * sizeof(int)) : nullptr;
         o.sdir = need.dirs ? (double *)take(3 * ns * sizeof(double)) : nullptr;
         o.rec = need.rec ? (float4 *)take(ns * 2 * sizeof(float4)) : nullptr;
         // 64 bytes of slack: the band spreader's bulk copies round their ends up to 16 bytes
@@ -177,6 +177,7 @@ size_t workspace_layout(const fv_plan_s::WsNeed &need, char *base, fv_plan_s::Wo
         o.cs = take(ns * need.cs_per_src + 64);
         o.tc = need.tc ? (float4 *)take(ns * 3 * sizeof(float4)) : nullptr;
         o.tiles = (int *)take(4 * sizeof(int));
+        o.pairs = need.pairs ? take(need.pairs) : nullptr;
         if (need.ring_tiles > 0) {
             const size_t nt = (size_t)need.ring_tiles, sl = (size_t)need.ring_slots;
             o.ring_tiles = need.ring_tiles;
@@ -186,6 +187,33 @@ size_t workspace_layout(const fv_plan_s::WsNeed &need, char *base, fv_plan_s::Wo
             o.ring_cnt = (int *)take(nt * kRingBlocks * sizeof(int));
             o.ring_parts = (int4 *)take(sl * sizeof(int4));
             o.ring_partial = (float4 *)take(sl * kRingBlocks * need.ring_np * 32 * sizeof(float4));
+        }
+    }
+    return off;
+}
+
+// Bytes of a slice in the general form: the grid and both bands side by side at the general FFT lengths, coordinates and
+// strengths per source for the spreading on that grid.  The static scratch takes or refuses a plan by this size, so
+// that which plans it takes does not depend on the form a plan's slices have.
+static size_t general_bytes(const fv_plan_s::WsNeed &need)
+{
+    size_t off = 0;
+    auto take = [&](size_t bytes) { off = ((off + 255) & ~(size_t)255) + bytes; };
+    take(need.grid);
+    take(need.bufA);
+    take(need.bufB);
+    take(need.vu);
+    if (need.tiled) {
+        const size_t ns = (size_t)need.n_src, nb = (size_t)need.nb;
+        for (const size_t bytes : {ns * 4, nb * 4, (nb + 1) * 4, nb * 4, ns * 4, ns * 12, ns * 24}) take(bytes);
+        take(ns * need.frac_per_src + 64);
+        take(ns * need.cs_per_src + 64);
+        if (need.tc) take(ns * 3 * sizeof(float4));
+        take(16);
+        if (need.ring_tiles > 0) {
+            const size_t nt = (size_t)need.ring_tiles, sl = (size_t)need.ring_slots;
+            for (const size_t bytes : {nt * 16, nt * 4, nt * kRingBlocks * 4, sl * 16, sl * kRingBlocks * need.ring_np * 512})
+                take(bytes);
         }
     }
     return off;
@@ -263,7 +291,7 @@ static void resolve_spread(fv_plan_s *p, int gs, int w)
     // the other methods for the per-channel slices, so auto takes them only where nothing else exists
     const bool gather_auto = gather_ok && !(gs == 8 && nz_t > 8);
     // the ring gather (and its tensor-core form): FP32 two-dimensional grids without height terms
-    const bool ring_ok = gather_ok && gs == 4 && p->d == 2 && p->hK == 0 && (p->n_pol == 1 || p->n_pol == 4) &&
+    const bool ring_ok = p->ring_ok = gather_ok && gs == 4 && p->d == 2 && p->hK == 0 && (p->n_pol == 1 || p->n_pol == 4) &&
                          w <= kRingWmax && p->precision == FV_MIXED;
     int m = p->spread_req;
     if (m == FV_SPREAD_TENSOR && !ring_ok) m = FV_SPREAD_GATHER;
@@ -272,6 +300,8 @@ static void resolve_spread(fv_plan_s *p, int gs, int w)
     if (p->hK > 0) m = FV_SPREAD_GATHER;    // the height terms are spread by the gather kernel only (checked)
     if (m == FV_SPREAD_GATHER && !gather_ok) m = FV_SPREAD_ATOMIC;
     if (m == FV_SPREAD_SCATTER && !scatter_ok) m = FV_SPREAD_ATOMIC;
+    p->general_method = m;
+    if (p->pairs) m = FV_SPREAD_GATHER;
     p->spread_method = m;
     // FP32 gather plans with a kernel of at most 7 points: sources prepared and added in one pass, sorted by
     // strips (fv_spread_strip.cu); an 8-point kernel fills the window's eight rows, so that every change of row
@@ -421,6 +451,9 @@ static fv_status prepare_lattice(fv_plan_s *p)
     nd.bufB = (size_t)(2 * lg.H[1] + 1) * (2 * lg.H[0] + 1) * K * np * es;
     nd.frac_per_src = (3 + 2 * (size_t)w) * gs;         // fx, fy, u and the 2w kernel values
     nd.cs_per_src = (size_t)np * es;
+    fv_plan_s::WsNeed general = nd;
+    general.nb = 1;
+    p->static_need = general_bytes(general);
     if (p->lat_dense) {
         // at most what the type-1 transform would hold, so that the static scratch takes every plan it took with it
         const size_t one = dense_modes(p->dense) * sizeof(cpx<double>);
@@ -441,7 +474,8 @@ static fv_status prepare_lattice(fv_plan_s *p)
 // Per-channel geometry, tables and workspace; needs the array and the sky.
 // Grid and FFT geometry of one dimension of a transform whose targets have half-extent X and whose
 // sources have half-extent S (Eq. 5: nf1 >= 2 sigma X S / pi + w); D and C are left to the caller.
-static fv_status dim_geometry(fv_plan_s *p, double X, double S, DimGeom &dg)
+// xy: an axis of the FFT passes along x or y (a compile-time length where there is one).
+static fv_status dim_geometry(fv_plan_s *p, double X, double S, DimGeom &dg, bool xy = true)
 {
     const int w = p->w;
     const int maxM = fft_max_M((int)(p->precision == FV_FP64 ? sizeof(double) : sizeof(float)));
@@ -451,9 +485,9 @@ static fv_status dim_geometry(fv_plan_s *p, double X, double S, DimGeom &dg)
     if (nf1 < w + 1) nf1 = w + 1;     // Eq. 5 is the requirement; no 2w floor is needed
     if (nf1 > (1L << 20)) return p->fail(FV_ERR_UNSUPPORTED, "spreading grid too large");
     dg.nf1 = next235even(nf1);
-    // FP32 grids at sigma >= 2: a compile-time length where there is one (up to 4,096 points)
+    // FP32 grids at sigma >= 2 and FP64 in pairs: a compile-time length where there is one (up to 4,096 points)
     const int target = (int)std::ceil(p->sigma * dg.nf1 - 1e-9);
-    dg.fixed = p->precision == FV_MIXED && p->sigma >= 2.0 && p->fft_max_radix == 16 &&
+    dg.fixed = xy && (p->precision == FV_MIXED ? p->sigma >= 2.0 : p->pairs) && p->fft_max_radix == 16 &&
                fft_choose_fixed(target, dg.radix, dg.nstages, dg.M);
     if (!dg.fixed) dg.M = fft_choose_length(target, dg.radix, dg.nstages, p->fft_max_radix);
     if (dg.M < 0 || dg.M > maxM)
@@ -519,7 +553,7 @@ static fv_status choose_heights(fv_plan_s *p)
         if (take && !asked) {
             // the up planes the three-dimensional grid of the top channel would take
             DimGeom dz{};
-            const fv_status ds = dim_geometry(p, kappa_top * p->bhalf[2], p->S[2], dz);
+            const fv_status ds = dim_geometry(p, kappa_top * p->bhalf[2], p->S[2], dz, false);
             take = ds != FV_OK || K <= dz.nf1;
             p->err.clear();
         }
@@ -536,11 +570,38 @@ static fv_status choose_heights(fv_plan_s *p)
     return FV_OK;
 }
 
+// FP64 slices in pairs of floats (fv_pairs.cu): sigma = 2, gather spreading (AUTO or asked for), products and planes
+// that its kernels hold, and x and y FFT lengths with a compile-time form in every channel (so in the top one).
+static fv_status choose_pairs(fv_plan_s *p)
+{
+    p->pairs = false;
+    if (p->precision != FV_FP64 || p->use_basis || std::fabs(p->sigma - 2.0) > 1e-12 || p->fft_max_radix != 16 ||
+        (p->spread_req != FV_SPREAD_AUTO && p->spread_req != FV_SPREAD_GATHER) || p->n_u <= 0 || !p->d_u_off)
+        return FV_OK;
+    const double nu_top = *std::max_element(p->freq.begin(), p->freq.end());
+    DimGeom d[3]{};
+    p->pairs = true;
+    for (int i = 0; i < p->d; ++i) {
+        if (dim_geometry(p, 2.0 * M_PI * nu_top / FV_C_LIGHT * p->bhalf[i], p->S[i], d[i], i < 2) != FV_OK) {
+            p->err.clear();
+            p->pairs = false;
+            return FV_OK;              // prepare reports it
+        }
+    }
+    const int nz = p->d == 3 ? d[2].nf1 : std::max(p->hK, 1);
+    p->pairs = d[0].fixed && d[1].fixed && pairs_fit(p->w, p->n_pol, nz);
+    if (p->pairs) p->pair_poly = pair_polynomials(p->w, p->beta);
+    return FV_OK;
+}
+
 static fv_status prepare(fv_plan_s *p)
 {
+    p->pairs = false;
     const fv_status hs = choose_heights(p);
     if (hs != FV_OK) return hs;
     if (p->use_basis) return prepare_basis(p);
+    const fv_status cps = choose_pairs(p);
+    if (cps != FV_OK) return cps;
     const int nf = (int)p->freq.size();
     const int w = p->w;
     p->gf.assign(nf, SliceGeom{});
@@ -549,6 +610,13 @@ static fv_status prepare(fv_plan_s *p)
     size_t pre_total = 0, tw_total = 0;
     for (int i = 0; i < 3; ++i) { p->nf1_max[i] = 1; p->M_max[i] = 1; }
     size_t grid_e = 0, bufA_e = 0, bufB_e = 0;
+    fv_plan_s::WsNeed general;                // general_bytes, in elements here
+    const auto general_B = [&](const DimGeom &dg) {
+        if (!dg.fixed) return (size_t)dg.B;
+        DimGeom o{};
+        const int M = fft_choose_length((int)std::ceil(p->sigma * dg.nf1 - 1e-9), o.radix, o.nstages, p->fft_max_radix);
+        return 2 * ((size_t)std::ceil(M / (2.0 * p->sigma) + 0.5 * w) + 1) + 1;
+    };
     std::map<int, size_t> tw_of;
     p->xy_fixed = true;
     for (int f = 0; f < nf; ++f) {
@@ -579,7 +647,7 @@ static fv_status prepare(fv_plan_s *p)
                 dg.nstages = 0;
                 continue;
             }
-            const fv_status ds = dim_geometry(p, g.kappa * p->bhalf[i], p->S[i], dg);
+            const fv_status ds = dim_geometry(p, g.kappa * p->bhalf[i], p->S[i], dg, i < 2);
             if (ds != FV_OK) return ds;
             dg.D = -g.kappa * p->bcen[i];
             dg.C = p->C[i];
@@ -606,7 +674,11 @@ static fv_status prepare(fv_plan_s *p)
         size_t grid_c = (size_t)p->n_pol * D[0].nf1 * D[1].nf1 * strip_planes(D[2].nf1);
         size_t pass1 = (size_t)D[0].B * p->n_pol * D[2].nf1 * D[1].nf1;
         size_t pass2 = (size_t)D[1].B * D[0].B * p->n_pol * D[2].nf1;
-        size_t pass3 = p->d == 3 ? (size_t)D[2].B * D[1].B * D[0].B * p->n_pol : 0;
+        size_t pass3 = p->d == 3 && D[2].nf1 > FV_ZDIRECT_MAX ? (size_t)D[2].B * D[1].B * D[0].B * p->n_pol : 0;
+        const size_t gb[3] = {general_B(D[0]), general_B(D[1]), general_B(D[2])}, npl = (size_t)p->n_pol * D[2].nf1;
+        general.grid = std::max(general.grid, npl * D[0].nf1 * D[1].nf1);
+        general.bufA = std::max({general.bufA, gb[0] * npl * D[1].nf1, p->d == 3 ? gb[2] * gb[1] * gb[0] * p->n_pol : 0});
+        general.bufB = std::max(general.bufB, gb[1] * gb[0] * npl);
         grid_e = std::max(grid_e, grid_c);
         bufA_e = std::max(bufA_e, std::max(pass1, pass3));
         bufB_e = std::max(bufB_e, pass2);
@@ -616,7 +688,7 @@ static fv_status prepare(fv_plan_s *p)
     // a new sky with the same grid sizes (the usual case: same array, same channels) keeps the
     // tables and workspaces of the previous one
     std::vector<long> sig = {(long)p->n_src, (long)p->n_pol, (long)p->n_streams, (long)p->spread_req, (long)p->d,
-                             (long)p->hK,
+                             (long)p->hK, (long)p->pairs,
                              (long)grid_e, (long)bufA_e, (long)bufB_e, (long)p->lat_ok, (long)p->lat_H[0],
                              (long)p->lat_H[1], (long)p->n_u, (long)p->n_bl};
     for (int k = 0; k < 4; ++k) {
@@ -684,12 +756,14 @@ static fv_status prepare(fv_plan_s *p)
                 CK(launch_prescale_table<double>((double *)p->d_pre + p->pre_off[(size_t)f * 3 + i], dg.nf1, dg.M, w,
                                                  p->beta, p->d_glx, p->d_glw, p->nq, p->stream));
                 if (first) CK(launch_twiddles<double>((cpx<double> *)p->d_tw + to, dg.M, p->stream));
+                if (first && dg.fixed)                          // cpx<Pf> and cpx<double> are of one size
+                    CK(launch_fixed_twiddles<Pf>((cpx<Pf> *)p->d_tw + to + dg.M, dg, p->stream));
             } else {
                 CK(launch_prescale_table<float>((float *)p->d_pre + p->pre_off[(size_t)f * 3 + i], dg.nf1, dg.M, w,
                                                 p->beta, p->d_glx, p->d_glw, p->nq, p->stream));
                 if (first) CK(launch_twiddles<float>((cpx<float> *)p->d_tw + to, dg.M, p->stream));
                 if (first && dg.fixed)
-                    CK(launch_fixed_twiddles((cpx<float> *)p->d_tw + to + dg.M, dg, p->stream));
+                    CK(launch_fixed_twiddles<float>((cpx<float> *)p->d_tw + to + dg.M, dg, p->stream));
             }
         }
     }
@@ -711,12 +785,35 @@ static fv_status prepare(fv_plan_s *p)
         p->strip ? 0 : (staged ? (size_t)staged_cs_stride((int)gs, p->n_pol) * es : (size_t)p->n_pol * es);
     // FP32 grids take each slice's coordinates and prephase from per-time records (no FP64 per slice)
     p->need.tc = p->precision == FV_MIXED && p->tiled;
-    const size_t bin_bytes = p->tiled ? workspace_layout(p->need, nullptr, nullptr) -
-                                            (p->need.grid + p->need.bufA + p->need.bufB + p->need.vu)
-                                      : 0;
-    p->ws_bytes = (long long)(pre_total * gs + tw_total * es +
-                              p->n_streams * ((grid_e + bufA_e + bufB_e) * es +
-                                              (size_t)p->n_u * p->n_pol * sizeof(cpx<double>) + bin_bytes));
+    // pairs: about 2 MB of targets a launch; no visibilities per target (the output is written directly) and no cells
+    p->need.cells = !p->pairs;
+    p->need.pairs = 0;
+    if (p->pairs) {
+        const size_t per = sizeof(PairTarget) + sizeof(cpx<Pf>) * p->nf1_max[2] * (p->d == 3 ? 1 : 0) +
+                           sizeof(cpx<Pf>) * std::max(p->hK, 1);
+        p->pair_chunk = (int)std::min<size_t>(p->n_u, ((size_t)2 << 20) / per);
+        p->need.pairs = 256 + p->pair_chunk * per;
+        p->need.vu = sizeof(cpx<double>);
+    }
+    p->ws_bytes = (long long)(pre_total * gs + tw_total * es + p->n_streams * workspace_layout(p->need, nullptr, nullptr));
+    // the general form: its spreading method, bins of 8 x 4 cells and records
+    general.grid *= es;
+    general.bufA *= es;
+    general.bufB *= es;
+    general.vu = std::max<size_t>((size_t)p->n_u * p->n_pol, 1) * sizeof(cpx<double>);
+    const bool g_staged = p->general_method == FV_SPREAD_GATHER || p->general_method == FV_SPREAD_TENSOR;
+    const bool g_ring = p->ring_ok && g_staged;
+    const int gT[2] = {p->bin_req[0] > 0 ? p->bin_req[0] : 8, p->bin_req[1] > 0 ? p->bin_req[1] : 4};
+    general.tiled = p->general_method != FV_SPREAD_ATOMIC;
+    general.n_src = std::max<long>(p->n_src, 1);
+    general.nb = ((p->nf1_top[0] + gT[0] - 1) / gT[0]) * ((p->nf1_top[1] + gT[1] - 1) / gT[1]);
+    general.frac_per_src = g_ring ? sizeof(RingRec) : (g_staged ? 4 * gs : 3 * gs);
+    general.cs_per_src = g_staged ? (size_t)staged_cs_stride((int)gs, p->n_pol) * es : (size_t)p->n_pol * es;
+    general.tc = p->precision == FV_MIXED && general.tiled;
+    general.ring_tiles = g_ring ? ring_tiles(p->nf1_max[0], p->nf1_max[1]) : 0;
+    general.ring_slots = g_ring ? (int)std::min<long>(kRingSlotsMax, 8 * std::max<long>(p->n_src, 1) / kRingPart + 1) : 0;
+    general.ring_np = g_ring ? p->n_pol : 0;
+    p->static_need = general_bytes(general);
     fv_status ls = prepare_lattice(p);
     if (ls != FV_OK) return ls;
     CK(cudaStreamSynchronize(p->stream));
@@ -920,7 +1017,9 @@ fv_status run_slices(fv_plan_s *p, fv_plan_s::Workspace &wk, cudaStream_t st, ch
         char *out = vis + ((size_t)(f - om.f0) * ntm + (t - om.t0)) * slice_bytes;
         // the interpolation writes the baselines' output itself (no scatter) where its kernel can
         const bool fused = p->d_u_off && p->tgt_n == p->n_u && (p->d == 2 || p->gf[f].dim[2].nf1 <= FV_ZDIRECT_MAX) &&
-                           interp_fuses_scatter(p->gf[f], (int)sizeof(G));
+                           (p->pairs || interp_fuses_scatter(p->gf[f], (int)sizeof(G)));
+        if (p->pairs && !fused) return p->fail(FV_ERR_STATE, "pair slices need their targets' baselines");
+        unsigned *key = (unsigned *)wk.pairs;
         // one transform per beam group: strengths with the group's two beams, targets [u0, u1)
         for (const auto &gr : p->groups) {
             if (gr.u1 <= gr.u0) continue;
@@ -956,9 +1055,11 @@ fv_status run_slices(fv_plan_s *p, fv_plan_s::Workspace &wk, cudaStream_t st, ch
                                       wk.cell, (float *)frac, (cpx<float> *)cs,
                                       staged && !ring ? (SrcRec<float> *)rec : nullptr,
                                       ring ? (RingRec *)wk.frac : nullptr, ring ? wk.tiles : nullptr, st));
-                else if (staged)
+                else if (staged) {
+                    if (p->pairs) CK(cudaMemsetAsync(key, 0, sizeof(unsigned), st));
                     CK(launch_prep_staged<G>(wk.sdir, wk.sidx, wk.offsets + nb, p->n_src, p->flux, p->flux_fp64, nf,
-                                             f, g, rec, cs, st));
+                                             f, g, rec, cs, st, p->pairs ? key : nullptr));
+                }
                 else
                     CK(launch_prep<G>(wk.sdir, wk.sidx, wk.offsets + nb, p->n_src, p->flux, p->flux_fp64, nf, f, g,
                                       wk.cell, frac, cs, st));
@@ -972,6 +1073,9 @@ fv_status run_slices(fv_plan_s *p, fv_plan_s::Workspace &wk, cudaStream_t st, ch
                                           RingWork{wk.tiles, wk.ring_bins, wk.ring_light, wk.ring_parts, wk.ring_cnt,
                                                    wk.ring_partial, wk.ring_tiles, wk.ring_slots},
                                           p->d_status, (cpx<float> *)grid, p->spread_method == FV_SPREAD_TENSOR, st));
+                else if (p->pairs)
+                    CK(launch_spread_pairs(wk.offsets, (const SrcRec<double> *)wk.frac, (const cpx<double> *)wk.cs, g, tb,
+                                           r0, r1, p->pair_poly, key, (cpx<Pf> *)grid, st));
                 else if (p->spread_method == FV_SPREAD_GATHER || p->spread_method == FV_SPREAD_TENSOR)
                     CK(launch_spread_gather_rec<G>(wk.offsets, rec, cs, g, tb, r0, r1, p->d_status, grid, st));
                 else if (p->spread_method == FV_SPREAD_SCATTER)
@@ -999,12 +1103,18 @@ fv_status run_slices(fv_plan_s *p, fv_plan_s::Workspace &wk, cudaStream_t st, ch
             const long r1 = (long)np * nz * D[1].nf1;
             CK(prof_begin(p, PC_FFT_X, st));
             if (p->strip) CK(fft_pass<G>(grid, A, r1, D[0], nullptr, tw + p->tw_off[o0], st, np * nz, np * nzp, nz, nzp));
+            else if (p->pairs)
+                CK(launch_fft_fixed<Pf>((const cpx<Pf> *)grid, (cpx<Pf> *)A, r1, D[0], 1, 1, 1, 1,
+                                        (const cpx<Pf> *)p->d_tw + p->tw_off[o0] + D[0].M, st));
             else CK(fft_pass<G>(grid, A, r1, D[0], pre_x, tw + p->tw_off[o0], st));
             CK(prof_end(p, (double)r1 * (D[0].nf1 + D[0].B) * es));
             // pass 2 along y: rows (bx, pol, z)
             const long r2 = (long)D[0].B * np * nz;
             CK(prof_begin(p, PC_FFT_Y, st));
             if (p->strip) CK(fft_pass<G>(A, Bb, r2, D[1], nullptr, tw + p->tw_off[o0 + 1], st, np * nz, np * nz, np * nz, np * nz));
+            else if (p->pairs)
+                CK(launch_fft_fixed<Pf>((const cpx<Pf> *)A, (cpx<Pf> *)Bb, r2, D[1], 1, 1, 1, 1,
+                                        (const cpx<Pf> *)p->d_tw + p->tw_off[o0 + 1] + D[1].M, st));
             else CK(fft_pass<G>(A, Bb, r2, D[1], pre_y, tw + p->tw_off[o0 + 1], st));
             CK(prof_end(p, (double)r2 * (D[1].nf1 + D[1].B) * es));
             if (p->d == 2 || D[2].nf1 <= FV_ZDIRECT_MAX) {
@@ -1012,8 +1122,16 @@ fv_status run_slices(fv_plan_s *p, fv_plan_s::Workspace &wk, cudaStream_t st, ch
                 const double wd = (double)p->w * p->w * D[2].nf1;
                 CK(prof_begin(p, PC_INTERP, st));
                 const SliceOut so{out, p->d_u_off, p->d_u_bl, gr.u0};
-                CK(launch_interp_zdirect<G>(Bb, bug, nug, decg, g, pre + p->pre_off[o0 + 2],
-                                            tw + p->tw_off[o0 + 2], Vug, st, fused ? &so : nullptr));
+                if (p->pairs) {
+                    PairTarget *tgt = (PairTarget *)((char *)wk.pairs + 256);
+                    CK(launch_interp_pairs((const cpx<Pf> *)Bb, bug, nug, decg, g,
+                                           (const double *)p->d_pre + p->pre_off[o0 + 2],
+                                           (const cpx<double> *)p->d_tw + p->tw_off[o0 + 2], p->pair_poly, key,
+                                           p->pair_chunk, tgt, (cpx<Pf> *)(tgt + p->pair_chunk), so, st));
+                } else {
+                    CK(launch_interp_zdirect<G>(Bb, bug, nug, decg, g, pre + p->pre_off[o0 + 2],
+                                                tw + p->tw_off[o0 + 2], Vug, st, fused ? &so : nullptr));
+                }
                 // with the scatter fused in, the baselines' output is written here
                 const double nbl_g = gr.bl1 - gr.bl0;
                 CK(prof_end(p, (double)nug * (wd * p->n_pol * es + 4 * sizeof(double) + p->n_pol * 16.0) +
@@ -1166,7 +1284,7 @@ static fv_status prepare_basis(fv_plan_s *p)
         }
         const double blo = p->bcen[i] - p->bhalf[i], bhi = p->bcen[i] + p->bhalf[i];
         const double xlo = std::min(-kmin * bhi, -kmax * bhi), xhi = std::max(-kmin * blo, -kmax * blo);
-        const fv_status ds = dim_geometry(p, 0.5 * (xhi - xlo), p->S[i], dg);
+        const fv_status ds = dim_geometry(p, 0.5 * (xhi - xlo), p->S[i], dg, i < 2);
         if (ds != FV_OK) return ds;
         dg.D = 0.5 * (xhi + xlo);
         dg.C = p->C[i];
@@ -1222,7 +1340,7 @@ static fv_status prepare_basis(fv_plan_s *p)
             CK(launch_prescale_table<float>((float *)p->d_pre + p->pre_off[i], dg.nf1, dg.M, w, p->beta, p->d_glx,
                                             p->d_glw, p->nq, p->stream));
             CK(launch_twiddles<float>((cpx<float> *)p->d_tw + p->tw_off[i], dg.M, p->stream));
-            if (dg.fixed) CK(launch_fixed_twiddles((cpx<float> *)p->d_tw + p->tw_off[i] + dg.M, dg, p->stream));
+            if (dg.fixed) CK(launch_fixed_twiddles<float>((cpx<float> *)p->d_tw + p->tw_off[i] + dg.M, dg, p->stream));
         }
     }
     CK(cudaMalloc(&p->d_bas_M, M.size() * sizeof(double)));

@@ -375,7 +375,8 @@ __global__ void __launch_bounds__(256) k_prep(const double *__restrict__ sdir, c
                                               const int *__restrict__ nv_ptr, long n_src,
                                               const void *__restrict__ flux, int flux_fp64, int n_freq, int f,
                                               SliceGeom g, int *__restrict__ cell, G *__restrict__ frac,
-                                              cpx<G> *__restrict__ cs, SrcRec<G> *__restrict__ rec)
+                                              cpx<G> *__restrict__ cs, SrcRec<G> *__restrict__ rec,
+                                              unsigned *__restrict__ key)
 {
     const long i = blockIdx.x * (long)blockDim.x + threadIdx.x;
     if (i >= *nv_ptr) return;
@@ -396,6 +397,16 @@ __global__ void __launch_bounds__(256) k_prep(const double *__restrict__ sdir, c
         if (p < np)
             cs[STAGED ? (size_t)i * staged_cs_stride((int)sizeof(G), np) + p : (size_t)p * n_src + i] =
                 cmul(c[p], cmk<G>(cp, sp));
+    if (STAGED && sizeof(G) == 8 && key) {
+        // the slice's largest exponent of a strength (pair_shift)
+        unsigned e = 0;
+#pragma unroll
+        for (int p = 0; p < 4; ++p)
+            if (p < np) e = max(e, max(exponent_key((double)c[p].x), exponent_key((double)c[p].y)));
+        const unsigned lanes = __activemask();
+        e = __reduce_max_sync(lanes, e);
+        if ((threadIdx.x & 31) == __ffs(lanes) - 1) atomicMax(key, e);
+    }
     // grid coordinates: first footprint cell l0 = ceil(q - w/2) and offset l0 - q of q = (s - C) qscale,
     // the product in FP64.  FP64 grids split in FP64; FP32 grids split q into q_hi + q_lo (floats, q_lo
     // the FP64 remainder) and take l0 and l0 - q_hi in FP32, exact but where q_hi - w/2 rounds onto an
@@ -555,18 +566,18 @@ cudaError_t launch_prep(const double *sdir, const int *sidx, const int *nv_ptr, 
 {
     if (n_src <= 0) return cudaSuccess;
     k_prep<G, false><<<(unsigned)((n_src + 255) / 256), 256, 0, st>>>(sdir, sidx, nv_ptr, n_src, flux, flux_fp64,
-                                                                      n_freq, f, g, cell, frac, cs, nullptr);
+                                                                      n_freq, f, g, cell, frac, cs, nullptr, nullptr);
     return cudaGetLastError();
 }
 
 template <class G>
 cudaError_t launch_prep_staged(const double *sdir, const int *sidx, const int *nv_ptr, long n_src,
                                const void *flux, int flux_fp64, int n_freq, int f, const SliceGeom &g,
-                               SrcRec<G> *rec, cpx<G> *cs, cudaStream_t st)
+                               SrcRec<G> *rec, cpx<G> *cs, cudaStream_t st, unsigned *key)
 {
     if (n_src <= 0) return cudaSuccess;
     k_prep<G, true><<<(unsigned)((n_src + 255) / 256), 256, 0, st>>>(sdir, sidx, nv_ptr, n_src, flux, flux_fp64,
-                                                                     n_freq, f, g, nullptr, nullptr, cs, rec);
+                                                                     n_freq, f, g, nullptr, nullptr, cs, rec, key);
     return cudaGetLastError();
 }
 
@@ -1148,10 +1159,10 @@ template cudaError_t launch_prep<float>(const double *, const int *, const int *
                                         const SliceGeom &, int *, float *, cpx<float> *, cudaStream_t);
 template cudaError_t launch_prep_staged<double>(const double *, const int *, const int *, long, const void *, int,
                                                 int, int, const SliceGeom &, SrcRec<double> *, cpx<double> *,
-                                                cudaStream_t);
+                                                cudaStream_t, unsigned *);
 template cudaError_t launch_prep_staged<float>(const double *, const int *, const int *, long, const void *, int,
                                                int, int, const SliceGeom &, SrcRec<float> *, cpx<float> *,
-                                               cudaStream_t);
+                                               cudaStream_t, unsigned *);
 template cudaError_t launch_spread_tile<double>(const int *, const int *, const double *, const cpx<double> *, long,
                                                 const SliceGeom &, const TimeBin &, double, double, cpx<double> *,
                                                 cudaStream_t);

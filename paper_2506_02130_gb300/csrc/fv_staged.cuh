@@ -144,11 +144,12 @@ cudaError_t launch_spread_ring(const int *offsets, const RingRec *rec, const cpx
                                cpx<float> *grid, bool tensor, cudaStream_t st);
 
 // Per slice: strengths with prephase and packed grid coordinates of the sorted sources, as staged
-// records (the same arithmetic as launch_prep).
+// records (the same arithmetic as launch_prep).  key (FP64, or nullptr; zero at launch): raised to the largest
+// exponent field of a strength (pair_shift).
 template <class G>
 cudaError_t launch_prep_staged(const double *sdir, const int *sidx, const int *nv_ptr, long n_src,
                                const void *flux, int flux_fp64, int n_freq, int f, const SliceGeom &g,
-                               SrcRec<G> *rec, cpx<G> *cs, cudaStream_t st);
+                               SrcRec<G> *rec, cpx<G> *cs, cudaStream_t st, unsigned *key = nullptr);
 
 // FP32 grids: the same, from the per-time records tc of launch_time_binning (no FP64 arithmetic); writes
 // ring records when ring_rec is given (two-dimensional grids, w <= 8), else staged records when rec is

@@ -108,7 +108,7 @@ extern "C" fv_status fv_execute_static(fv_plan_t p, void *vis)
     fv_status prev = plan_take_status(p, false);
     if (prev != FV_OK) return prev;
     // the same carving as a plan's own execution workspace (fv_plan_s::need), over the static array
-    const size_t need = workspace_layout(p->need, nullptr, nullptr);
+    const size_t need = std::max(workspace_layout(p->need, nullptr, nullptr), p->static_need);
     if (need > FV_STATIC_SCRATCH_BYTES)
         return p->fail(FV_ERR_UNSUPPORTED, "this plan needs " + std::to_string(need) +
                                                " bytes of scratch; the static scratch holds " +
