@@ -34,7 +34,10 @@ namespace {
 
 constexpr int kStripThreads = 128;                     // four warps, independent of one another
 constexpr int kWinX = 16, kWinY = 8;
-constexpr int kStripMin = 8;
+// least sources of a warp's run: 8 (a nearly empty grid takes them; the warp's latency is its run's length), with eight
+// planes 32 (each run ends with a window of 128 cells x 8 planes to add to the grid)
+// (hex array of 127 antennas, 128 channels x 8 terms, 31.0 -> 28.1 ms; with fewer planes 32 leaves SMs idle)
+__host__ __device__ constexpr int strip_min(int npl) { return npl == 8 ? 32 : 8; }
 
 // resident CTAs per SM (without spills in the loop over the sources)
 __host__ __device__ constexpr int strip_ctas(int npl) { return npl == 8 ? 4 : (npl == 4 ? 5 : 6); }
@@ -165,10 +168,9 @@ __global__ void __launch_bounds__(kStripThreads, strip_ctas(NPL))
     __shared__ __align__(16) float s_rec[kStripThreads / 32][32 * W];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int nv = *nv_ptr;
-    // contiguous runs of equally many sources, one per warp (at least 8, which a nearly empty grid takes: the
-    // warp's latency is then its run's length), cut into equal batches of at most 32
+    // contiguous runs of equally many sources, one per warp (at least strip_min), cut into equal batches of at most 32
     const int warps = gridDim.x * (kStripThreads / 32), wid = blockIdx.x * (kStripThreads / 32) + warp;
-    const int per = max(kStripMin, (nv + warps - 1) / warps);
+    const int per = max(strip_min(NPL), (nv + warps - 1) / warps);
     const int first = wid * per, last = min(nv, first + per);
     if (first >= last) return;                      // whole warps; nothing below synchronises the CTA
     const int batches = (last - first + 31) / 32, step = (last - first + batches - 1) / batches;
@@ -382,9 +384,9 @@ cudaError_t launch_spread_strip(const float4 *tc, const int *sidx, const int *nv
     }
     const bool pol4 = g.n_pol == 4 && nz == 1;
     const int npl = pol4 ? 4 : (nz == 1 ? 1 : (nz <= 4 ? 4 : 8));
-    // one wave of CTAs, each warp one run of at least kStripMin sources
-    constexpr int kMinCta = kStripMin * (kStripThreads / 32);
-    const long want = (n_src + kMinCta - 1) / kMinCta;
+    // one wave of CTAs, each warp one run of at least strip_min sources
+    const int min_cta = strip_min(npl) * (kStripThreads / 32);
+    const long want = (n_src + min_cta - 1) / min_cta;
     const unsigned groups = pol4 ? 1u : (unsigned)((nz + npl - 1) / npl), pols = pol4 ? 1u : (unsigned)g.n_pol;
     const long slots = (long)strip_ctas(npl) * sms[dev];
     const unsigned gx = (unsigned)std::min<long>(want, std::max<long>(1, slots / (groups * pols)));
