@@ -35,7 +35,10 @@ template <class G, int R2, int R3> struct FixedFft {
     static constexpr int rounds = items <= 320 ? 1 : (items <= 768 ? 2 : 3);
     static constexpr int T = (items + 32 * rounds - 1) / (32 * rounds) * 32;
     static constexpr int smem = R * S0 * 2 * (int)sizeof(G);
-    static constexpr int by_smem = 225000 / (smem + 1024), by_regs = 65536 / (T * (P ? 160 : 80));
+    // registers a thread: pairs 160, above 1,152 points 128 (a second CTA per SM: 1,728 and 1,920 points 102 -> 92 us;
+    // at 576 to 864 points 128 is slower, 77 against 74 us)
+    static constexpr int regs = P ? (M > 1152 ? 128 : 160) : 80;
+    static constexpr int by_smem = 225000 / (smem + 1024), by_regs = 65536 / (T * regs);
     static constexpr int blocks = by_smem < by_regs ? (by_smem > 0 ? by_smem : 1) : (by_regs > 0 ? by_regs : 1);
     static constexpr int keep = R3 / 4;                          // outputs m3 <= keep and m3 >= R3 - 1 - keep
 };

@@ -2,7 +2,7 @@
 //
 // GB300 has 64 FP32 multiply-adds for one of FP64, so an FP64 slice was bound by the FP64 pipe in every step: on the
 // 127-antenna workload (35,000 sources, 10 height terms, 12-point kernel) 1,050 us of spreading, 515 + 420 us of FFT
-// passes and 400 us of interpolation.  A pair of floats carries 48 bits, and a multiply-add of pairs takes about 13
+// passes and 400 us of interpolation (now 210, 90 + 74 and 62 us).  A pair of floats carries 48 bits, and a multiply-add of pairs takes about 13
 // operations.  FP64 plans take this path at sigma = 2 and kernels of at most 13 points, whose own error (1.7e-12 at
 // w = 13) stays well above the pairs' (about 1e-14 an operation); wider kernels and other sigma keep FP64 throughout.
 // FP64 remains in the per-time directions, the strengths, coordinates and phases (k_prep), the per-target set-up and
@@ -59,8 +59,8 @@ PairPoly pair_polynomials(int w, double beta)
 
 namespace {
 
-constexpr int kPsThreads = 256, kPsChunk = 64;
-constexpr int kPsTileX = 32, kPsTileY = 8, kPsPatches = 8;          // a warp: 8 x 4 cells
+constexpr int kPsTileX = 16, kPsTileY = 8, kPsPatchX = kPsTileX / 8;    // a warp: 8 x 4 cells
+constexpr int kPsPatches = kPsPatchX * (kPsTileY / 4), kPsThreads = 32 * kPsPatches, kPsChunk = 64;
 
 // Horner in pairs; value p (even + s odd) and its mirror (even - s odd)
 __device__ __forceinline__ void pair_kernel(const Pf *es, int p, Pf s, Pf s2, Pf &v, Pf &mirror)
@@ -79,12 +79,15 @@ __device__ __forceinline__ void pair_kernel(const Pf *es, int p, Pf s, Pf s2, Pf
 
 }  // namespace
 
-// A CTA of 8 warps owns a 32 x 8 tile of (x, y) columns, a warp an 8 x 4 patch, a lane one column with its NZ planes x
-// NP products in registers (as the FP64 register gather).  Candidates are taken 64 at a time: their kernel values and
-// height terms are computed once per chunk into shared memory, each is listed for the patches its footprint meets, and
-// every warp adds its list's sources.  Every cell is stored once.
+// A CTA of 4 warps owns a 16 x 8 tile of (x, y) columns, a warp an 8 x 4 patch, a lane one column with its NZ planes x
+// NP products in registers (as the FP64 register gather).  The sources of the tile's bins that reach it (about half) are taken
+// kPsChunk at a time: their kernel values and height terms are computed once per chunk into shared memory, each is
+// listed for the patches its footprint meets, and every warp adds its list's sources.  The warps of a CTA wait for the
+// longest list of a chunk, so small tiles win although a source's values are computed in more of them (12-point kernel,
+// 10 height terms): 208 us a slice, 246 with 32 x 8, 225 with 8 x 8, 231 with 16 x 4 and 16 x 16 cells; chunks of 32
+// instead of 64 sources 222.  Every cell is stored once.
 template <int NP, int NZ>
-__global__ void __launch_bounds__(kPsThreads, 2) k_spread_pairs(const int *__restrict__ offsets,
+__global__ void __launch_bounds__(kPsThreads, 512 / kPsThreads) k_spread_pairs(const int *__restrict__ offsets,
                                                                 const SrcRec<double> *__restrict__ rec,
                                                                 const cpx<double> *__restrict__ cs, SliceGeom g, TimeBin tb,
                                                                 double r0, double r1, PairPoly es,
@@ -97,13 +100,13 @@ __global__ void __launch_bounds__(kPsThreads, 2) k_spread_pairs(const int *__res
     __shared__ Pf s_s[2][kPsChunk], s_z[NZ > 1 ? kPsChunk : 1];
     __shared__ int s_cz[NZ > 1 ? kPsChunk : 1];
     __shared__ int s_list[kPsPatches][kPsChunk], s_cnt[kPsPatches];
-    __shared__ int s_row0[32], s_pre[32], s_total, s_bins[4];
+    __shared__ int s_row0[32], s_pre[32], s_total, s_bins[4], s_idx[kPsChunk + kPsThreads], s_have;
     __shared__ double s_up;
     const int nx = g.dim[0].nf1, ny = g.dim[1].nf1, nz = g.d == 3 || g.K ? g.dim[2].nf1 : 1;
     const int w = g.w;
     const int x0 = blockIdx.x * kPsTileX, y0 = blockIdx.y * kPsTileY;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int gx = x0 + (warp & 3) * 8 + (lane & 7), gy = y0 + (warp >> 2) * 4 + (lane >> 3);
+    const int gx = x0 + warp % kPsPatchX * 8 + (lane & 7), gy = y0 + warp / kPsPatchX * 4 + (lane >> 3);
     Pair2 acc[NP][NZ];
 #pragma unroll
     for (int p = 0; p < NP; ++p)
@@ -112,6 +115,7 @@ __global__ void __launch_bounds__(kPsThreads, 2) k_spread_pairs(const int *__res
     for (int k = threadIdx.x; k < kPairPoly; k += kPsThreads) s_es[k] = es.v[k];
     if (threadIdx.x < kPsPatches) s_cnt[threadIdx.x] = 0;
     if (threadIdx.x == 0) {
+        s_have = 0;
         s_up = scalbn(1.0, pair_shift(*key));
         // bins whose sources can reach the tile (one top cell of margin)
         const double qx_lo = (x0 - nx / 2 - 0.5 * w) / r0, qx_hi = (x0 + kPsTileX - nx / 2 + 0.5 * w - 1) / r0;
@@ -146,15 +150,32 @@ __global__ void __launch_bounds__(kPsThreads, 2) k_spread_pairs(const int *__res
         }
         __syncthreads();
         const int total = s_total;
-        for (int base = 0; base < total; base += kPsChunk) {
-            const int n = min(kPsChunk, total - base);
-            if (threadIdx.x < n) {
-                const int t = threadIdx.x, v = base + t;
-                int r = 0;                          // the last row whose prefix is <= v
+        int base = 0, have = 0;
+        while (true) {
+            // the bins' sources that reach the tile, until there is a chunk of them
+            while (have < kPsChunk && base < total) {
+                const int v = base + threadIdx.x;
+                if (v < total) {
+                    int r = 0;                          // the last row whose prefix is <= v
 #pragma unroll
-                for (int step = 16; step > 0; step >>= 1)
-                    if (r + step < nrows && s_pre[r + step] <= v) r += step;
-                const long i = s_row0[r] + (v - s_pre[r]);
+                    for (int step = 16; step > 0; step >>= 1)
+                        if (r + step < nrows && s_pre[r + step] <= v) r += step;
+                    const int i = s_row0[r] + (v - s_pre[r]);
+                    const unsigned cell = rec[i].cell;
+                    const int cx = (int)(cell & 0x3fffu) - x0, cy = (int)((cell >> 14) & 0x3fffu) - y0;
+                    if (cx < kPsTileX && cx + w > 0 && cy < kPsTileY && cy + w > 0) s_idx[atomicAdd(&s_have, 1)] = i;
+                }
+                base += kPsThreads;
+                __syncthreads();
+                have = s_have;
+                __syncthreads();
+            }
+            const int n = min(kPsChunk, have);
+            if (n == 0) break;
+            have -= n;
+            if (threadIdx.x < n) {
+                const int t = threadIdx.x;
+                const long i = s_idx[have + t];
                 const SrcRec<double> rr = rec[i];
                 const int cx = (int)(rr.cell & 0x3fffu), cy = (int)((rr.cell >> 14) & 0x3fffu);
                 s_s[0][t] = pf(2.0 * rr.fx + (double)(w - 1));
@@ -171,13 +192,13 @@ __global__ void __launch_bounds__(kPsThreads, 2) k_spread_pairs(const int *__res
                 }
                 const int ax = max(cx - x0, 0), bx = min(cx + w - 1 - x0, kPsTileX - 1);
                 const int ay = max(cy - y0, 0), by2 = min(cy + w - 1 - y0, kPsTileY - 1);
-                if (ax <= bx && ay <= by2)
-                    for (int qy = ay / 4; qy <= by2 / 4; ++qy)
-                        for (int qx = ax / 8; qx <= bx / 8; ++qx) {
-                            const int q = qy * 4 + qx, pos = atomicAdd(&s_cnt[q], 1);
-                            s_list[q][pos] = t | ((cx - x0 + 16) << 8) | ((cy - y0 + 16) << 16);
-                        }
+                for (int qy = ay / 4; qy <= by2 / 4; ++qy)
+                    for (int qx = ax / 8; qx <= bx / 8; ++qx) {
+                        const int q = qy * kPsPatchX + qx, pos = atomicAdd(&s_cnt[q], 1);
+                        s_list[q][pos] = t | ((cx - x0 + 16) << 8) | ((cy - y0 + 16) << 16);
+                    }
             }
+            if (threadIdx.x == 0) s_have = have;
             __syncthreads();
             // kernel values: (source fastest, axis, mirrored pair)
             for (int v = threadIdx.x; v < kPsChunk * 2 * half; v += kPsThreads) {
@@ -242,6 +263,7 @@ __global__ void __launch_bounds__(kPsThreads, 2) k_spread_pairs(const int *__res
             }
             __syncthreads();
             if (threadIdx.x < kPsPatches) s_cnt[threadIdx.x] = 0;
+            __syncthreads();
         }
         __syncthreads();
     }
