@@ -63,7 +63,7 @@ static void drop_graph(fv_batch_s *b)
 
 static bool covers(const fv_plan_s::WsNeed &have, const fv_plan_s::WsNeed &need)
 {
-    return have.grid >= need.grid && have.bufA >= need.bufA && have.bufB >= need.bufB && have.vu >= need.vu &&
+    return (have.apart || !need.apart) && have.grid >= need.grid && have.bufA >= need.bufA && have.bufB >= need.bufB && have.vu >= need.vu &&
            (!need.tiled || (have.tiled && have.n_src >= need.n_src && have.nb >= need.nb &&
                             have.frac_per_src >= need.frac_per_src && have.cs_per_src >= need.cs_per_src &&
                             (have.tc || !need.tc) && (have.rec || !need.rec) && (have.dirs || !need.dirs) &&
@@ -255,6 +255,7 @@ fv_status fv_batch_execute(fv_batch_t b, int use_graph)
         need.bufA = std::max(need.bufA, n.bufA);
         need.bufB = std::max(need.bufB, n.bufB);
         need.vu = std::max(need.vu, n.vu);
+        need.apart = need.apart || n.apart;
         if (n.tiled) {
             need.tiled = true;
             need.n_src = std::max(need.n_src, n.n_src);

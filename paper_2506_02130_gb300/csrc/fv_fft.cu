@@ -302,7 +302,7 @@ template cudaError_t launch_fft_pass<float>(const cpx<float> *, cpx<float> *, lo
 
 // ---------------------------------------------------------------- compile-time lengths (fv_fft_fixed.cuh)
 #define FV_FIXED_ARGS(G) const cpx<G> *in, cpx<G> *out, int rows, const DimGeom &dg, int P, int sP, int nz, int nzp, \
-                         const cpx<G> *twB, cudaStream_t st
+                         const cpx<G> *twB, cpx<G> *clr, cudaStream_t st
 cudaError_t fft_fixed_a(FV_FIXED_ARGS(float));      // lengths up to 864
 cudaError_t fft_fixed_b(FV_FIXED_ARGS(float));      // up to 1728
 cudaError_t fft_fixed_c(FV_FIXED_ARGS(float));      // up to 2560
@@ -365,27 +365,27 @@ template cudaError_t launch_fixed_twiddles<Pf>(cpx<Pf> *, const DimGeom &, cudaS
 
 template <class G>
 cudaError_t launch_fft_fixed(const cpx<G> *in, cpx<G> *out, long rows, const DimGeom &dg, int P, int sP, int nz, int nzp,
-                             const cpx<G> *tw, cudaStream_t st)
+                             const cpx<G> *tw, cudaStream_t st, cpx<G> *clr)
 {
     if (rows <= 0) return cudaSuccess;
     if (rows > (1L << 30) || P < 1 || nz < 1) return cudaErrorInvalidValue;
     const int r = (int)rows;
     if constexpr (sizeof(G) == 4) {
-        if (dg.M <= 864) return fft_fixed_a(in, out, r, dg, P, sP, nz, nzp, tw, st);
-        if (dg.M <= 1728) return fft_fixed_b(in, out, r, dg, P, sP, nz, nzp, tw, st);
-        if (dg.M <= 2560) return fft_fixed_c(in, out, r, dg, P, sP, nz, nzp, tw, st);
-        return fft_fixed_d(in, out, r, dg, P, sP, nz, nzp, tw, st);
+        if (dg.M <= 864) return fft_fixed_a(in, out, r, dg, P, sP, nz, nzp, tw, clr, st);
+        if (dg.M <= 1728) return fft_fixed_b(in, out, r, dg, P, sP, nz, nzp, tw, clr, st);
+        if (dg.M <= 2560) return fft_fixed_c(in, out, r, dg, P, sP, nz, nzp, tw, clr, st);
+        return fft_fixed_d(in, out, r, dg, P, sP, nz, nzp, tw, clr, st);
     } else {
-        if (dg.M <= 864) return fft_pairs_a(in, out, r, dg, P, sP, nz, nzp, tw, st);
-        if (dg.M <= 1728) return fft_pairs_b(in, out, r, dg, P, sP, nz, nzp, tw, st);
-        if (dg.M <= 2560) return fft_pairs_c(in, out, r, dg, P, sP, nz, nzp, tw, st);
-        return fft_pairs_d(in, out, r, dg, P, sP, nz, nzp, tw, st);
+        if (dg.M <= 864) return fft_pairs_a(in, out, r, dg, P, sP, nz, nzp, tw, clr, st);
+        if (dg.M <= 1728) return fft_pairs_b(in, out, r, dg, P, sP, nz, nzp, tw, clr, st);
+        if (dg.M <= 2560) return fft_pairs_c(in, out, r, dg, P, sP, nz, nzp, tw, clr, st);
+        return fft_pairs_d(in, out, r, dg, P, sP, nz, nzp, tw, clr, st);
     }
 }
 template cudaError_t launch_fft_fixed<float>(const cpx<float> *, cpx<float> *, long, const DimGeom &, int, int, int, int,
-                                             const cpx<float> *, cudaStream_t);
+                                             const cpx<float> *, cudaStream_t, cpx<float> *);
 template cudaError_t launch_fft_fixed<Pf>(const cpx<Pf> *, cpx<Pf> *, long, const DimGeom &, int, int, int, int,
-                                          const cpx<Pf> *, cudaStream_t);
+                                          const cpx<Pf> *, cudaStream_t, cpx<Pf> *);
 
 // ---------------------------------------------------------------- host planning
 static const int kRadices[] = {16, 15, 12, 10, 9, 8, 6, 5, 4, 3, 2};

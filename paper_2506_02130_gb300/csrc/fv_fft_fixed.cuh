@@ -77,10 +77,12 @@ template <class G> __device__ __forceinline__ void dft16_half(const cpx<G> *v, c
     }
 }
 
-// rows (y, p), y = row / P, p = row % P: value l at in[(y N + l) sP + (p / nz) nzp + p % nz]
-template <class G, int R2, int R3>
+// rows (y, p), y = row / P, p = row % P: value l at in[(y N + l) sP + (p / nz) nzp + p % nz].  CLEAR: read from clr
+// (the same rows), which is left zero for the next slice's spreading (with its padding plane): a memset launch less,
+// for small grids (a 22 MB grid costs the pass more, 22 -> 33 us, than its memset, 8 us).
+template <class G, int R2, int R3, bool CLEAR>
 __global__ void __launch_bounds__((FixedFft<G, R2, R3>::T), (FixedFft<G, R2, R3>::blocks))
-    k_fft_fixed(const cpx<G> *__restrict__ in, cpx<G> *__restrict__ out, int rows, int N, int H, int B, int P,
+    k_fft_fixed(const cpx<G> *__restrict__ in, cpx<G> *clr, cpx<G> *__restrict__ out, int rows, int N, int H, int B, int P,
                 int sP, int nz, int nzp, const cpx<G> *__restrict__ twB, const cpx<G> *__restrict__ twC)
 {
     using F = FixedFft<G, R2, R3>;
@@ -95,7 +97,11 @@ __global__ void __launch_bounds__((FixedFft<G, R2, R3>::T), (FixedFft<G, R2, R3>
     {
         const int half = N / 2;
         const int y = live ? row / P : 0, p = live ? row - y * P : 0;
-        const C *src = in + (size_t)y * N * sP + (p / nz) * nzp + p % nz;
+        const size_t at = (size_t)y * N * sP + (p / nz) * nzp + p % nz;
+        const C *src = in + at;
+        C *own = CLEAR ? clr + at : nullptr;
+        const bool pad = CLEAR && nzp > nz && p % nz == nz - 1;
+        const C zero = cmk<G>((G)0.0, (G)0.0);
 #pragma unroll
         for (int k = 0; k < (R * MB + T - 1) / T; ++k) {
             const int j = tid / R + k * (T / R);
@@ -104,12 +110,26 @@ __global__ void __launch_bounds__((FixedFft<G, R2, R3>::T), (FixedFft<G, R2, R3>
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
                 const int pos = j + q * MB;                                     // l - N/2
-                v[q] = live && pos < N - half ? src[(size_t)(pos + half) * sP] : cmk<G>((G)0.0, (G)0.0);
+                const bool in_row = live && pos < N - half;
+                const size_t l = (size_t)(pos + half) * sP;
+                v[q] = in_row ? (CLEAR ? own[l] : src[l]) : zero;
             }
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
                 const int l = j + (q - 4) * MB + half;
-                v[4 + q] = live && l >= 0 ? src[(size_t)l * sP] : cmk<G>((G)0.0, (G)0.0);
+                v[4 + q] = live && l >= 0 ? (CLEAR ? own[(size_t)l * sP] : src[(size_t)l * sP]) : zero;
+            }
+            if constexpr (CLEAR) {
+                if (live) {
+#pragma unroll
+                    for (int q = 0; q < 8; ++q) {
+                        const int l = j + (q < 4 ? q : q - 8) * MB + half;
+                        if (q < 4 ? l < N : l >= 0) {
+                            own[(size_t)l * sP] = zero;
+                            if (pad) own[(size_t)l * sP + 1] = zero;
+                        }
+                    }
+                }
             }
             dft16_half(v, o);
             C *d = mine + (j / R3) * S3 + j % R3;
@@ -165,7 +185,7 @@ __global__ void __launch_bounds__((FixedFft<G, R2, R3>::T), (FixedFft<G, R2, R3>
 
 template <class G, int R2, int R3>
 cudaError_t fft_fixed_go(const cpx<G> *in, cpx<G> *out, int rows, const DimGeom &dg, int P, int sP, int nz, int nzp,
-                         const cpx<G> *twB, cudaStream_t st)
+                         const cpx<G> *twB, cpx<G> *clr, cudaStream_t st)
 {
     using F = FixedFft<G, R2, R3>;
     static_assert(F::T % F::R == 0 && F::T <= 1024, "a thread keeps one row");
@@ -179,12 +199,23 @@ cudaError_t fft_fixed_go(const cpx<G> *in, cpx<G> *out, int rows, const DimGeom 
     if (e != cudaSuccess) return e;
     if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
     if (!attr_set[dev]) {
-        e = cudaFuncSetAttribute(k_fft_fixed<G, R2, R3>, cudaFuncAttributeMaxDynamicSharedMemorySize, F::smem);
+        e = cudaFuncSetAttribute(k_fft_fixed<G, R2, R3, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, F::smem);
+        if constexpr (!F::P)
+            if (e == cudaSuccess)
+                e = cudaFuncSetAttribute(k_fft_fixed<G, R2, R3, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, F::smem);
         if (e != cudaSuccess) return e;
         attr_set[dev] = true;
     }
-    k_fft_fixed<G, R2, R3><<<(rows + F::R - 1) / F::R, F::T, F::smem, st>>>(in, out, rows, dg.nf1, dg.H, dg.B, P, sP, nz,
-                                                                        nzp, twB, twB + 16 * R2);
+    const unsigned blocks = (unsigned)((rows + F::R - 1) / F::R);
+    if constexpr (!F::P) {
+        if (clr) {
+            k_fft_fixed<G, R2, R3, true><<<blocks, F::T, F::smem, st>>>(nullptr, clr, out, rows, dg.nf1, dg.H, dg.B, P, sP, nz,
+                                                                       nzp, twB, twB + 16 * R2);
+            return cudaGetLastError();
+        }
+    }
+    k_fft_fixed<G, R2, R3, false><<<blocks, F::T, F::smem, st>>>(in, nullptr, out, rows, dg.nf1, dg.H, dg.B, P, sP, nz, nzp,
+                                                                twB, twB + 16 * R2);
     return cudaGetLastError();
 }
 

@@ -5,21 +5,21 @@
 namespace fv {
 
 cudaError_t fft_fixed_a(const cpx<float> *in, cpx<float> *out, int rows, const DimGeom &dg, int P, int sP, int nz,
-                        int nzp, const cpx<float> *twB, cudaStream_t st)
+                        int nzp, const cpx<float> *twB, cpx<float> *clr, cudaStream_t st)
 {
     switch (dg.M) {
-    case 256: return fft_fixed_go<float, 4, 4>(in, out, rows, dg, P, sP, nz, nzp, twB, st);
-    case 320: return fft_fixed_go<float, 5, 4>(in, out, rows, dg, P, sP, nz, nzp, twB, st);
-    case 384: return fft_fixed_go<float, 6, 4>(in, out, rows, dg, P, sP, nz, nzp, twB, st);
-    case 400: return fft_fixed_go<float, 5, 5>(in, out, rows, dg, P, sP, nz, nzp, twB, st);
-    case 480: return fft_fixed_go<float, 6, 5>(in, out, rows, dg, P, sP, nz, nzp, twB, st);
-    case 512: return fft_fixed_go<float, 8, 4>(in, out, rows, dg, P, sP, nz, nzp, twB, st);
-    case 576: return fft_fixed_go<float, 6, 6>(in, out, rows, dg, P, sP, nz, nzp, twB, st);
-    case 640: return fft_fixed_go<float, 8, 5>(in, out, rows, dg, P, sP, nz, nzp, twB, st);
-    case 720: return fft_fixed_go<float, 9, 5>(in, out, rows, dg, P, sP, nz, nzp, twB, st);
-    case 768: return fft_fixed_go<float, 8, 6>(in, out, rows, dg, P, sP, nz, nzp, twB, st);
-    case 800: return fft_fixed_go<float, 10, 5>(in, out, rows, dg, P, sP, nz, nzp, twB, st);
-    case 864: return fft_fixed_go<float, 9, 6>(in, out, rows, dg, P, sP, nz, nzp, twB, st);
+    case 256: return fft_fixed_go<float, 4, 4>(in, out, rows, dg, P, sP, nz, nzp, twB, clr, st);
+    case 320: return fft_fixed_go<float, 5, 4>(in, out, rows, dg, P, sP, nz, nzp, twB, clr, st);
+    case 384: return fft_fixed_go<float, 6, 4>(in, out, rows, dg, P, sP, nz, nzp, twB, clr, st);
+    case 400: return fft_fixed_go<float, 5, 5>(in, out, rows, dg, P, sP, nz, nzp, twB, clr, st);
+    case 480: return fft_fixed_go<float, 6, 5>(in, out, rows, dg, P, sP, nz, nzp, twB, clr, st);
+    case 512: return fft_fixed_go<float, 8, 4>(in, out, rows, dg, P, sP, nz, nzp, twB, clr, st);
+    case 576: return fft_fixed_go<float, 6, 6>(in, out, rows, dg, P, sP, nz, nzp, twB, clr, st);
+    case 640: return fft_fixed_go<float, 8, 5>(in, out, rows, dg, P, sP, nz, nzp, twB, clr, st);
+    case 720: return fft_fixed_go<float, 9, 5>(in, out, rows, dg, P, sP, nz, nzp, twB, clr, st);
+    case 768: return fft_fixed_go<float, 8, 6>(in, out, rows, dg, P, sP, nz, nzp, twB, clr, st);
+    case 800: return fft_fixed_go<float, 10, 5>(in, out, rows, dg, P, sP, nz, nzp, twB, clr, st);
+    case 864: return fft_fixed_go<float, 9, 6>(in, out, rows, dg, P, sP, nz, nzp, twB, clr, st);
     default: return cudaErrorInvalidValue;
     }
 }

@@ -5,15 +5,15 @@
 namespace fv {
 
 cudaError_t fft_pairs_c(const cpx<Pf> *in, cpx<Pf> *out, int rows, const DimGeom &dg, int P, int sP, int nz,
-                        int nzp, const cpx<Pf> *twB, cudaStream_t st)
+                        int nzp, const cpx<Pf> *twB, cpx<Pf> *clr, cudaStream_t st)
 {
     switch (dg.M) {
-    case 1920: return fft_fixed_go<Pf, 12, 10>(in, out, rows, dg, P, sP, nz, nzp, twB, st);
-    case 2048: return fft_fixed_go<Pf, 16, 8>(in, out, rows, dg, P, sP, nz, nzp, twB, st);
-    case 2160: return fft_fixed_go<Pf, 15, 9>(in, out, rows, dg, P, sP, nz, nzp, twB, st);
-    case 2304: return fft_fixed_go<Pf, 12, 12>(in, out, rows, dg, P, sP, nz, nzp, twB, st);
-    case 2400: return fft_fixed_go<Pf, 15, 10>(in, out, rows, dg, P, sP, nz, nzp, twB, st);
-    case 2560: return fft_fixed_go<Pf, 16, 10>(in, out, rows, dg, P, sP, nz, nzp, twB, st);
+    case 1920: return fft_fixed_go<Pf, 12, 10>(in, out, rows, dg, P, sP, nz, nzp, twB, clr, st);
+    case 2048: return fft_fixed_go<Pf, 16, 8>(in, out, rows, dg, P, sP, nz, nzp, twB, clr, st);
+    case 2160: return fft_fixed_go<Pf, 15, 9>(in, out, rows, dg, P, sP, nz, nzp, twB, clr, st);
+    case 2304: return fft_fixed_go<Pf, 12, 12>(in, out, rows, dg, P, sP, nz, nzp, twB, clr, st);
+    case 2400: return fft_fixed_go<Pf, 15, 10>(in, out, rows, dg, P, sP, nz, nzp, twB, clr, st);
+    case 2560: return fft_fixed_go<Pf, 16, 10>(in, out, rows, dg, P, sP, nz, nzp, twB, clr, st);
     default: return cudaErrorInvalidValue;
     }
 }

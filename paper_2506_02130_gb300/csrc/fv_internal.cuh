@@ -528,10 +528,10 @@ cudaError_t launch_fft_pass(const cpx<G> *in, cpx<G> *out, long rows, const DimG
 // The same pass for FP32 rows of a compile-time length (dg.fixed; M >= 2 N, no prescale): row r = (y, p) with
 // P = rows per y, its value l at in[(y N + l) sP + (p / nz) nzp + p % nz] (P = sP = nz = nzp = 1: contiguous rows).
 // tw: the tables of launch_fixed_twiddles (fft_fixed_table complex values).
-// G: float, or Pf for grids of float pairs.
+// G: float, or Pf for grids of float pairs.  clr (float; nullptr or in): the rows, padding plane included, are left zero.
 template <class G>
 cudaError_t launch_fft_fixed(const cpx<G> *in, cpx<G> *out, long rows, const DimGeom &dg, int P, int sP, int nz, int nzp,
-                             const cpx<G> *tw, cudaStream_t st);
+                             const cpx<G> *tw, cudaStream_t st, cpx<G> *clr = nullptr);
 // The smallest compile-time length M >= target, or false (target above 4096).
 bool fft_choose_fixed(int target, int *radix, int &nstages, int &M);
 size_t fft_fixed_table(const DimGeom &dg);

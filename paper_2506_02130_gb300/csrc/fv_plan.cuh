@@ -127,6 +127,7 @@ struct fv_plan_s {
     // what one execution workspace must hold for this plan (set by prepare)
     struct WsNeed {
         size_t grid = 0, bufA = 0, bufB = 0, vu = 0;   // bytes
+        bool apart = false;                            // the second band beside the grid, not in its place
         long n_src = 0;
         int nb = 0;
         size_t frac_per_src = 0, cs_per_src = 0;       // bytes per source

@@ -158,8 +158,10 @@ size_t workspace_layout(const fv_plan_s::WsNeed &need, char *base, fv_plan_s::Wo
     };
     fv_plan_s::Workspace tmp;
     fv_plan_s::Workspace &o = w ? *w : tmp;
-    // the grid is dead once the first FFT pass has read it: the second band takes its place
-    o.grid = o.bufB = take(std::max(need.grid, need.bufB));
+    // the grid is dead once the first FFT pass has read it: the second band takes its place, unless the grid is to be
+    // left clear for the next slice
+    o.grid = o.bufB = take(need.apart ? need.grid : std::max(need.grid, need.bufB));
+    if (need.apart) o.bufB = take(need.bufB);
     o.bufA = take(need.bufA);
     o.Vu = (cpx<double> *)take(need.vu);
     if (need.tiled) {
@@ -191,6 +193,12 @@ size_t workspace_layout(const fv_plan_s::WsNeed &need, char *base, fv_plan_s::Wo
     }
     return off;
 }
+
+// Largest grid that the x pass leaves clear for the next slice.  It saves a memset launch per transform, which small
+// grids feel (61 antennas, six beam groups, 1.5 MB: 3.50 -> 2.92 ms for 384 transforms); its zeros pass through the SMs'
+// stores and the L2 beside the other streams' data, which large grids feel more (127 antennas, 26 MB: 28.0 -> 35.8 ms;
+// 350 antennas, 36 MB: 85 -> 108 ms).  4 MB: the grids and bands of eight streams stay in the L2.
+constexpr size_t kClearInPass = (size_t)4 << 20;
 
 // Bytes of a slice in the general form: the grid and both bands side by side at the general FFT lengths, coordinates and
 // strengths per source for the spreading on that grid.  The static scratch takes or refuses a plan by this size, so
@@ -795,7 +803,7 @@ static fv_status prepare(fv_plan_s *p)
         p->need.pairs = 256 + p->pair_chunk * per;
         p->need.vu = sizeof(cpx<double>);
     }
-    p->ws_bytes = (long long)(pre_total * gs + tw_total * es + p->n_streams * workspace_layout(p->need, nullptr, nullptr));
+    p->need.apart = false;
     // the general form: its spreading method, bins of 8 x 4 cells and records
     general.grid *= es;
     general.bufA *= es;
@@ -814,6 +822,13 @@ static fv_status prepare(fv_plan_s *p)
     general.ring_slots = g_ring ? (int)std::min<long>(kRingSlotsMax, 8 * std::max<long>(p->n_src, 1) / kRingPart + 1) : 0;
     general.ring_np = g_ring ? p->n_pol : 0;
     p->static_need = general_bytes(general);
+    if (p->strip) {
+        // beside a small grid, but where the static scratch takes the plan and would not hold it so
+        p->need.apart = p->need.grid <= kClearInPass;
+        if (p->static_need <= FV_STATIC_SCRATCH_BYTES && workspace_layout(p->need, nullptr, nullptr) > FV_STATIC_SCRATCH_BYTES)
+            p->need.apart = false;
+    }
+    p->ws_bytes = (long long)(pre_total * gs + tw_total * es + p->n_streams * workspace_layout(p->need, nullptr, nullptr));
     fv_status ls = prepare_lattice(p);
     if (ls != FV_OK) return ls;
     CK(cudaStreamSynchronize(p->stream));
@@ -848,12 +863,12 @@ static SliceGeom slice_geom_for(const fv_plan_s *p, int f, int t, const fv_plan_
 // table, the fixed ones behind it; rows as launch_fft_fixed), else the general kernel on contiguous rows.
 template <class G>
 static cudaError_t fft_pass(const cpx<G> *in, cpx<G> *out, long rows, const DimGeom &dg, const G *pre, const cpx<G> *tw,
-                            cudaStream_t st, int P = 1, int sP = 1, int nz = 1, int nzp = 1)
+                            cudaStream_t st, int P = 1, int sP = 1, int nz = 1, int nzp = 1, cpx<G> *clr = nullptr)
 {
     if constexpr (sizeof(G) == 4) {
-        if (dg.fixed && !pre) return launch_fft_fixed(in, out, rows, dg, P, sP, nz, nzp, tw + dg.M, st);
+        if (dg.fixed && !pre) return launch_fft_fixed(in, out, rows, dg, P, sP, nz, nzp, tw + dg.M, st, clr);
     }
-    if (sP != 1) return cudaErrorInvalidValue;
+    if (sP != 1 || clr) return cudaErrorInvalidValue;
     return launch_fft_pass<G>(in, out, rows, dg, pre, tw, st);
 }
 
@@ -987,6 +1002,17 @@ fv_status run_slices(fv_plan_s *p, fv_plan_s::Workspace &wk, cudaStream_t st, ch
     const G *pre = (const G *)p->d_pre;
     const cpx<G> *tw = (const cpx<G> *)p->d_tw;
     int t_binned = -1;
+    // strips: a small grid with a place of its own is cleared once, and left clear by the x passes
+    size_t held_max = 0;
+    for (long q = k_begin; p->strip && q < std::min(k_end, k_begin + nf); ++q) {
+        const DimGeom *D = p->gf[q % nf].dim;
+        held_max = std::max(held_max, (size_t)p->n_pol * D[0].nf1 * D[1].nf1 * strip_planes(D[2].nf1) * sizeof(cpx<G>));
+    }
+    const bool apart = wk.bufB != wk.grid && held_max <= kClearInPass;
+    bool clean = false;
+    const fv_plan_s::BeamGroup *last_group = nullptr;
+    for (const auto &gr : p->groups)
+        if (gr.u1 > gr.u0) last_group = &gr;
     TimeBin tb{};
     for (long k = k_begin; k < k_end; ++k) {
         const int t = (int)(k / nf), f = (int)(k % nf);
@@ -1031,11 +1057,21 @@ fv_status run_slices(fv_plan_s *p, fv_plan_s::Workspace &wk, cudaStream_t st, ch
             cpx<double> *Vug = wk.Vu + (size_t)gr.u0 * p->n_pol;
             const DimGeom *D = g.dim;
             const size_t gel = (size_t)p->n_pol * D[0].nf1 * D[1].nf1 * D[2].nf1;
+            bool last = true;                       // no transform follows in this call
             if (p->strip) {
-                CK(prof_begin(p, PC_MEMSET, st));
-                const size_t held = gel / D[2].nf1 * strip_planes(D[2].nf1);
-                CK(cudaMemsetAsync(grid, 0, held * sizeof(cpx<G>), st));
-                CK(prof_end(p, held * es));
+                last = k + 1 == k_end && &gr == last_group;
+                if (!clean) {
+                    // every grid of the call's channels where the x passes leave them clear, else this one
+                    CK(prof_begin(p, PC_MEMSET, st));
+                    size_t held = 0;
+                    for (long q = k; q < (apart ? std::min(k_end, k + nf) : k + 1); ++q) {
+                        const DimGeom *Dq = p->gf[q % nf].dim;
+                        held = std::max(held, (size_t)p->n_pol * Dq[0].nf1 * Dq[1].nf1 * strip_planes(Dq[2].nf1));
+                    }
+                    CK(cudaMemsetAsync(grid, 0, held * sizeof(cpx<G>), st));
+                    CK(prof_end(p, held * es));
+                    clean = apart;
+                }
                 g.pre_x = pre + p->pre_off[(size_t)f * 3];         // applied as rows are added to the grid
                 g.pre_y = pre + p->pre_off[(size_t)f * 3 + 1];
                 CK(prof_begin(p, PC_SPREAD, st));
@@ -1102,7 +1138,8 @@ fv_status run_slices(fv_plan_s *p, fv_plan_s::Workspace &wk, cudaStream_t st, ch
             const int np = p->n_pol, nz = D[2].nf1, nzp = strip_planes(nz);
             const long r1 = (long)np * nz * D[1].nf1;
             CK(prof_begin(p, PC_FFT_X, st));
-            if (p->strip) CK(fft_pass<G>(grid, A, r1, D[0], nullptr, tw + p->tw_off[o0], st, np * nz, np * nzp, nz, nzp));
+            if (p->strip) CK(fft_pass<G>(grid, A, r1, D[0], nullptr, tw + p->tw_off[o0], st, np * nz, np * nzp, nz, nzp,
+                                             clean && !last ? grid : nullptr));
             else if (p->pairs)
                 CK(launch_fft_fixed<Pf>((const cpx<Pf> *)grid, (cpx<Pf> *)A, r1, D[0], 1, 1, 1, 1,
                                         (const cpx<Pf> *)p->d_tw + p->tw_off[o0] + D[0].M, st));

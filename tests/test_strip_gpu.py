@@ -141,3 +141,20 @@ def test_sources_on_the_horizon_are_cut_as_in_fp64():
     p.set_sky(prob.sky.ra, prob.sky.dec, prob.sky.flux)
     assert rel_l2(mixed, p.run()) <= 2e-5
     p.close()
+
+
+@pytest.mark.parametrize("z_sigma,heights,polarised", [(0.0, "auto", True), (0.002, "terms", True), (0.05, "terms", False),
+                                                      (0.02, "grid", True)])
+def test_grid_left_clear_between_slices(z_sigma, heights, polarised):
+    """The x pass leaves the grid clear for the next slice: channels of growing and shrinking grids, odd planes and
+    their padding, one stream, against every channel in a plan of its own (the same sums in another order)."""
+    prob = _prob(1500, polarised, n_chan=6, z_sigma=z_sigma)
+    order = [3, 0, 5, 1, 4, 2]
+    prob.freqs_hz = prob.freqs_hz[order]
+    prob.sky.flux = np.ascontiguousarray(prob.sky.flux[:, :, order])
+    flux, freqs = prob.sky.flux, prob.freqs_hz
+    out, _ = _run(prob, 1e-6, heights=heights, n_streams=1)
+    for f in range(6):
+        prob.freqs_hz, prob.sky.flux = freqs[f:f + 1], np.ascontiguousarray(flux[:, :, f:f + 1])
+        one, _ = _run(prob, 1e-6, heights=heights, n_streams=1)
+        assert rel_l2(out[f], one[0]) <= 1e-5
