@@ -127,10 +127,12 @@ def peaks():
 
 
 # the source files that define each kernel class of the type-3 route (plus the shared device header)
-KERNEL_FILES = {"bin": ("fv_spread.cu", "fv_staged.cuh"), "prep": ("fv_spread.cu", "fv_staged.cuh"),
-                "spread": ("fv_spread.cu", "fv_spread_ring.cu", "fv_staged.cuh"), "fft_x": ("fv_fft.cu",),
-                "fft_y": ("fv_fft.cu",), "fft_z": ("fv_fft.cu",), "interp": ("fv_kernels.cu",),
-                "scatter": ("fv_kernels.cu",)}
+KERNEL_FILES = {"bin": ("fv_spread.cu", "fv_staged.cuh"), "prep": ("fv_spread.cu", "fv_staged.cuh", "fv_prep.cuh"),
+                "spread": ("fv_spread.cu", "fv_spread_strip.cu", "fv_spread_ring.cu", "fv_staged.cuh", "fv_prep.cuh",
+                           "fv_pairs.cu", "fv_pair.cuh"),
+                "fft_x": ("fv_fft.cu", "fv_fft_fixed.cuh", "fv_dft.cuh", "fv_pair.cuh"),
+                "fft_y": ("fv_fft.cu", "fv_fft_fixed.cuh", "fv_dft.cuh", "fv_pair.cuh"), "fft_z": ("fv_fft.cu",),
+                "interp": ("fv_kernels.cu", "fv_pairs.cu", "fv_pair.cuh"), "scatter": ("fv_kernels.cu",)}
 
 
 def kernel_source_hash(kernel_class):
@@ -816,8 +818,8 @@ def run_sim(args, rank, world, local, dist):
                                  "what": "useful FP32 flops of the spreading (n_pol w^2 complex x real "
                                          "multiply-adds per visible source)"}
             roof["note"] = ("neither bound is reached: the spreading is bound by instruction issue and "
-                            "shared-memory latency (a warp's lanes cover 8 x 8 cells, of which a source "
-                            "reaches about a quarter); ncu figures in profiles/")
+                            "shared-memory latency (a warp adds a source to 16 x 8 cells in registers, of "
+                            "which its footprint covers 49); ncu figures in profiles/")
     gpu_launches = int(sum(v["launches"] for k, v in prof.items() if k != "memset")) * args.steps
 
     # ---- end to end through the C ABI with host buffers (pinned): set_sky copies the step's inputs in,

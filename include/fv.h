@@ -50,7 +50,9 @@ typedef enum {
 } fv_status;
 
 typedef enum {
-    FV_FP64 = 0,    /* every step in FP64; output complex128 */
+    FV_FP64 = 0,    /* FP64 accuracy; output complex128.  Type-3 slices at sigma = 2 with kernels of at
+                       most 13 points and the mode sums of small lattices (eps >= 1e-12) hold grids and
+                       sums as pairs of floats (48 bits), everything else is FP64 */
     FV_MIXED = 1    /* spread, FFT and interpolation in FP32 with FP64 centring,
                        rescaling, phases and deconvolution; output complex64 */
 } fv_precision;
@@ -110,7 +112,8 @@ typedef struct {
                                  norms, resolves about 1e-8, so a smaller eps gets the largest
                                  basis); ignored by the other routes */
     int bin_size[2];          /* cells of the highest channel's grid per bin of the per-time source sort
-                                 in x and y; 0 = 8 x 4; 1 <= each <= 64 */
+                                 in x and y; 0 = 8 x 4, or (16 - w) x 1 where the sort is by strips
+                                 (FV_MIXED gather plans, w <= 7); 1 <= each <= 64 */
     int heights;              /* fv_heights: how the type-3 route evaluates the up axis of a
                                  non-coplanar array (one whose baselines have b_up != 0) */
 } fv_opts;
@@ -206,7 +209,9 @@ int fv_lattice_detect(int n_ant, const double *enu_m, double tol_m, double basis
 /* How the ES spreading step is run (all give the same result up to rounding). */
 typedef enum {
     FV_SPREAD_AUTO = 0,
-    FV_SPREAD_GATHER = 1,     /* per-tile, each thread sums the sources covering its cells; the tile's
+    FV_SPREAD_GATHER = 1,     /* FV_MIXED, w <= 7, FFT lengths up to 4,096: each warp adds a run of the
+                                 sources, sorted by strips, to a window of cells in registers.  Else
+                                 per-tile, each thread sums the sources covering its cells; the tile's
                                  sorted sources are staged in shared memory by bulk asynchronous copies
                                  (FV_MIXED two-dimensional grids: persistent CTAs, a producer warp
                                  streaming chunks into a shared-memory ring, 8 x 8 blocks per warp) */

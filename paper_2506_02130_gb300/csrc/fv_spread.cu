@@ -3,7 +3,7 @@
 // Per time (shared by every channel of that time):
 //   k_bin_count    rotate equatorial -> ENU (Section 2.3), cut the horizon, and
 //                  count the visible sources per tile of the top channel's grid;
-//   k_bin_scan     exclusive scan of the counts (one CTA);
+//   k_bin_sums, k_bin_scan   exclusive scan of the counts (a CTA per block of them);
 //   k_bin_scatter  counting-sort the visible directions by tile.
 // Per (time, channel) slice:
 //   k_prep         beam x flux strengths (Eq. 1-3), prephase e^{i D.(s-C)}

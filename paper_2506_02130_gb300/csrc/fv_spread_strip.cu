@@ -21,7 +21,7 @@
 // Bound by instruction issue (56 % busy, 16 warps an SM).  Measured per slice, one stream: 350-antenna workload
 // (443,000 sources above the horizon, four products, 1500 x 750 cells) 54 us and 8 us to clear the grid, against
 // 33 + 117 us for the preparation pass and the ring gather; 127-antenna workload (35,000 sources, 8 height terms)
-// 26 + 7 against 8 + 48 us with the register gather.
+// 28 + 7 against 8 + 48 us with the register gather.
 #include "fv_staged.cuh"
 #include "fv_prep.cuh"
 
