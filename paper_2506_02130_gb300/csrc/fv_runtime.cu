@@ -2154,13 +2154,6 @@ fv_status fv_set_sky(fv_plan_t p, long n_src, const double *ra_rad, const double
     if (n_stokes != (p->polarized ? 4 : 1) && !(n_stokes == 4 && !p->polarized))
         return p->fail(FV_ERR_ARG, p->polarized ? "polarised plan needs n_stokes = 4" : "n_stokes must be 1 or 4");
     if (n_src > 0 && (!ra_rad || !dec_rad || !flux)) return p->fail(FV_ERR_ARG, "NULL sky array");
-    for (long i = 0; i < n_src; ++i)
-        if (!std::isfinite(ra_rad[i]) || !std::isfinite(dec_rad[i]))
-            return p->fail(FV_ERR_ARG, "non-finite source coordinate");
-    p->have_sky = false;
-    // work still queued on the device may read the sky buffers this call rewrites (a plan's own streams,
-    // or a batch's lanes): wait for it, as freeing them would
-    CK(cudaDeviceSynchronize());
     // (re)allocate a buffer only when its size changes
     auto ensure = [&](void **ptr, size_t &cap, size_t bytes) -> cudaError_t {
         if (*ptr && cap == bytes) return cudaSuccess;
@@ -2171,21 +2164,42 @@ fv_status fv_set_sky(fv_plan_t p, long n_src, const double *ra_rad, const double
         if (e == cudaSuccess) cap = bytes;
         return e;
     };
+    // the coordinates go to a buffer that only this call uses, and are checked there (886,432 sources: 25 us; a loop
+    // on the host took 630), before anything of the sky that the plan holds is touched
+    const size_t ns = std::max<long>(n_src, 1);
+    CK(ensure((void **)&p->d_radec, p->radec_bytes, ns * 2 * sizeof(double) + sizeof(double)));
+    double *d_tmp = p->d_radec;
+    if (n_src) {
+        int *d_bad = (int *)(d_tmp + 2 * ns), bad = 0;
+        CK(cudaMemsetAsync(d_bad, 0, sizeof(int), p->stream));
+        CK(cudaMemcpyAsync(d_tmp, ra_rad, n_src * sizeof(double), cudaMemcpyHostToDevice, p->stream));
+        CK(cudaMemcpyAsync(d_tmp + ns, dec_rad, n_src * sizeof(double), cudaMemcpyHostToDevice, p->stream));
+        CK(launch_find_nonfinite(d_tmp, 2 * n_src, d_bad, p->stream));       // ns = n_src here
+        CK(cudaMemcpyAsync(&bad, d_bad, sizeof(int), cudaMemcpyDeviceToHost, p->stream));
+        CK(cudaStreamSynchronize(p->stream));
+        if (bad) return p->fail(FV_ERR_ARG, "non-finite source coordinate");
+    }
+    p->have_sky = false;
+    // work still queued on the device may read the sky buffers this call rewrites (a plan's own streams,
+    // or a batch's lanes): wait for it, as freeing them would
+    CK(cudaDeviceSynchronize());
     p->flux = nullptr;
     p->flux_borrowed = false;
     p->n_src = n_src;
     p->n_stokes = n_stokes;
     p->flux_fp64 = flux_is_fp64 ? 1 : 0;
-    const size_t ns = std::max<long>(n_src, 1);
     CK(ensure((void **)&p->d_e, p->e_bytes, ns * 3 * sizeof(double)));
-    CK(ensure((void **)&p->d_radec, p->radec_bytes, ns * 2 * sizeof(double)));
-    double *d_tmp = p->d_radec;
-    if (n_src) {
-        CK(cudaMemcpyAsync(d_tmp, ra_rad, n_src * sizeof(double), cudaMemcpyHostToDevice, p->stream));
-        CK(cudaMemcpyAsync(d_tmp + ns, dec_rad, n_src * sizeof(double), cudaMemcpyHostToDevice, p->stream));
-    }
     if (p->precision == FV_MIXED) CK(ensure((void **)&p->d_ep, p->ep_bytes, ns * 3 * sizeof(float2)));
     CK(launch_radec_to_unit(d_tmp, d_tmp + ns, n_src, p->d_e, p->d_ep, p->stream));
+    // the source extents and the fluxes are independent: extents on the plan's stream, fluxes on a second one (joined
+    // below), so that the copy from the host covers the FP64 work
+    const int nb = 304;
+    if (!p->d_Rt) CK(cudaMalloc(&p->d_Rt, std::max<size_t>(p->Rt.size(), 1) * sizeof(double)));
+    if (!p->d_ext) CK(cudaMalloc(&p->d_ext, (size_t)nb * 6 * sizeof(double)));
+    double *d_R = p->d_Rt, *d_ext = p->d_ext;
+    CK(cudaMemcpyAsync(d_R, p->Rt.data(), p->Rt.size() * sizeof(double), cudaMemcpyHostToDevice, p->stream));
+    CK(launch_source_extents(p->d_e, n_src, d_R, (int)p->lst.size(), d_ext, nb, p->stream));
+    cudaStream_t fs = p->sub.size() > 1 ? p->sub[1] : p->stream;
     const size_t fbytes = (size_t)n_stokes * n_src * p->freq.size() * (p->flux_fp64 ? 8 : 4);
     if (flux_on_device) {
         p->flux = flux;
@@ -2194,7 +2208,7 @@ fv_status fv_set_sky(fv_plan_t p, long n_src, const double *ra_rad, const double
         p->flux_owned_bytes = 0;
     } else if (n_src) {
         CK(ensure(&p->d_flux_owned, p->flux_owned_bytes, fbytes));
-        CK(cudaMemcpyAsync(p->d_flux_owned, flux, fbytes, cudaMemcpyHostToDevice, p->stream));
+        CK(cudaMemcpyAsync(p->d_flux_owned, flux, fbytes, cudaMemcpyHostToDevice, fs));
         p->flux = p->d_flux_owned;
     }
     if (flux_in_place(p)) {
@@ -2206,19 +2220,16 @@ fv_status fv_set_sky(fv_plan_t p, long n_src, const double *ra_rad, const double
         CK(ensure(&p->d_flux_t, p->flux_t_bytes, fbytes));
         if (!p->flux_borrowed)
             CK(launch_flux_transpose(p->flux, p->flux_fp64, n_src, n_stokes, (int)p->freq.size(), 0,
-                                     (int)p->freq.size(), p->d_flux_t, p->stream));
+                                     (int)p->freq.size(), p->d_flux_t, fs));
+    }
+    if (fs != p->stream) {
+        CK(cudaEventRecord(p->ev_join[1], fs));
+        CK(cudaStreamWaitEvent(p->stream, p->ev_join[1], 0));
     }
     // source extents over all times (visible directions only)
-    const int nb = 304;
-    if (!p->d_Rt) CK(cudaMalloc(&p->d_Rt, std::max<size_t>(p->Rt.size(), 1) * sizeof(double)));
-    if (!p->d_ext) CK(cudaMalloc(&p->d_ext, (size_t)nb * 6 * sizeof(double)));
-    double *d_R = p->d_Rt, *d_ext = p->d_ext;
-    CK(cudaMemcpyAsync(d_R, p->Rt.data(), p->Rt.size() * sizeof(double), cudaMemcpyHostToDevice, p->stream));
-    CK(launch_source_extents(p->d_e, n_src, d_R, (int)p->lst.size(), d_ext, nb, p->stream));
     std::vector<double> ext((size_t)nb * 6);
     CK(cudaMemcpyAsync(ext.data(), d_ext, ext.size() * sizeof(double), cudaMemcpyDeviceToHost, p->stream));
     CK(cudaStreamSynchronize(p->stream));
-    (void)d_tmp;
     double lo[3] = {INFINITY, INFINITY, INFINITY}, hi[3] = {-INFINITY, -INFINITY, -INFINITY};
     for (int b = 0; b < nb; ++b)
         for (int i = 0; i < 3; ++i) {
