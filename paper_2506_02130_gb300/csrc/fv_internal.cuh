@@ -424,7 +424,6 @@ cudaError_t launch_flux_transpose(const void *flux, int fp64, long n_src, int n_
 
 // e[3][n]: equatorial unit vectors from (ra, dec).
 // ep (nullable): the same as float pairs, [3][n].
-cudaError_t launch_find_nonfinite(const double *v, long n, int *bad, cudaStream_t st);
 cudaError_t launch_radec_to_unit(const double *ra, const double *dec, long n, double *e, float2 *ep, cudaStream_t st);
 
 // Per-block min/max of visible ENU directions over all times: out[nblocks][6].

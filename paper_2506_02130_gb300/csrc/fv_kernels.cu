@@ -128,22 +128,6 @@ cudaError_t launch_flux_transpose(const void *flux, int fp64, long n_src, int n_
     return cudaGetLastError();
 }
 
-// *bad |= 1 where a value is an infinity or NaN
-__global__ void __launch_bounds__(256) k_find_nonfinite(const double *__restrict__ v, long n, int *bad)
-{
-    bool any = false;
-    for (long i = blockIdx.x * 256L + threadIdx.x; i < n; i += gridDim.x * 256L) any = any || !isfinite(v[i]);
-    if (any) atomicOr(bad, 1);
-}
-
-cudaError_t launch_find_nonfinite(const double *v, long n, int *bad, cudaStream_t st)
-{
-    if (n <= 0) return cudaSuccess;
-    const unsigned blocks = (unsigned)std::min<long>((n + 255) / 256, 1216);
-    k_find_nonfinite<<<blocks, 256, 0, st>>>(v, n, bad);
-    return cudaGetLastError();
-}
-
 cudaError_t launch_radec_to_unit(const double *ra, const double *dec, long n, double *e, float2 *ep, cudaStream_t st)
 {
     if (n <= 0) return cudaSuccess;
