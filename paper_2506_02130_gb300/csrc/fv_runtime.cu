@@ -751,6 +751,7 @@ static fv_status prepare(fv_plan_s *p)
     }
     CK(cudaMalloc(&p->d_pre, std::max<size_t>(pre_total, 1) * gs));
     CK(cudaMalloc(&p->d_tw, std::max<size_t>(tw_total, 1) * es));
+    p->need = fv_plan_s::WsNeed{};      // another route may have set it (prepare_lattice)
     p->need.grid = std::max<size_t>(grid_e, 1) * es;
     p->need.bufA = std::max<size_t>(bufA_e, 1) * es;
     p->need.bufB = std::max<size_t>(bufB_e, 1) * es;
@@ -975,12 +976,28 @@ static fv_status run_slices_lattice(fv_plan_s *p, fv_plan_s::Workspace &wk, cuda
     return FV_OK;
 }
 
+// Whether a workspace has every per-source buffer that the plan's slices write: a layout made for another route must
+// not reach the kernels.
+static bool workspace_serves(const fv_plan_s *p, const fv_plan_s::Workspace &wk)
+{
+    const bool fp32 = p->precision == FV_MIXED;
+    if (p->use_lattice) {
+        const bool sorted = wk.counts && wk.offsets && wk.cursor && wk.sidx;
+        return sorted && (p->lat_dense ? (fp32 ? wk.rec != nullptr : wk.sdir != nullptr) : wk.sdir && wk.cell);
+    }
+    if (!p->tiled) return true;
+    if (!wk.bin_of || !wk.counts || !wk.offsets || !wk.cursor || !wk.sidx || (fp32 && !wk.tc)) return false;
+    if (p->strip) return wk.cell != nullptr;
+    return wk.sdir && (p->pairs ? wk.pairs != nullptr : wk.cell != nullptr);
+}
+
 template <class G>
 fv_status run_slices(fv_plan_s *p, fv_plan_s::Workspace &wk, cudaStream_t st, char *vis, size_t slice_bytes,
                      long k_begin, long k_end, OutMap om)
 {
     if (p->use_basis)
         return p->fail(FV_ERR_UNSUPPORTED, "the spectral-basis route runs whole times: use fv_execute");
+    if (!workspace_serves(p, wk)) return p->fail(FV_ERR_STATE, "the workspace lacks a buffer of the plan's route");
     if (p->use_lattice) return run_slices_lattice<G>(p, wk, st, vis, slice_bytes, k_begin, k_end, om);
     const int nf = (int)p->freq.size(), nt = (int)p->lst.size();
     cpx<G> *grid = (cpx<G> *)wk.grid;
