@@ -747,7 +747,7 @@ static fv_status prepare(fv_plan_s *p)
     if (reuse) {
         resolve_spread(p, (int)gs, w);
         p->geo_sig = sig;
-        return FV_OK;        // the lattice route's tables and decision depend on the array only: kept
+        return FV_OK;        // the lattice route's tables and decision depend on the array only (setup_array): kept
     }
     CK(cudaMalloc(&p->d_pre, std::max<size_t>(pre_total, 1) * gs));
     CK(cudaMalloc(&p->d_tw, std::max<size_t>(tw_total, 1) * es));
@@ -1904,6 +1904,7 @@ static fv_status setup_array(fv_plan_s *p)
     if (d == 2 && nonplanar) return p->fail(FV_ERR_ARG, "dims = 2 requested for a non-coplanar array");
     // lattice test (Section 2.2.1): baselines as integer combinations n of two lattice vectors
     std::vector<int> bln;
+    std::vector<double> bup;
     bool lat_ok = false;
     double lat_basis[4] = {0, 0, 0, 0};
     int lat_H[2] = {0, 0};
@@ -1911,8 +1912,8 @@ static fv_status setup_array(fv_plan_s *p)
         std::vector<int> kidx(2 * (size_t)n_ant);
         lat_ok = lattice_detect(n_ant, enu_m, p->lat_tol, lat_basis, kidx.data()) != 0;
         if (lat_ok) {
-            p->lat_bup.resize(n_bl);
-            for (int b = 0; b < n_bl; ++b) p->lat_bup[b] = enu_m[3 * pr[2 * b] + 2] - enu_m[3 * pr[2 * b + 1] + 2];
+            bup.resize(n_bl);
+            for (int b = 0; b < n_bl; ++b) bup[b] = enu_m[3 * pr[2 * b] + 2] - enu_m[3 * pr[2 * b + 1] + 2];
             bln.resize(2 * (size_t)n_bl);
             for (int b = 0; b < n_bl; ++b)
                 for (int k = 0; k < 2; ++k) {
@@ -1925,8 +1926,10 @@ static fv_status setup_array(fv_plan_s *p)
     if (p->transform_req == FV_TRANSFORM_LATTICE && !lat_ok)
         return p->fail(FV_ERR_UNSUPPORTED, "transform = FV_TRANSFORM_LATTICE, but the antennas' horizontal "
                                            "positions are not a lattice within lattice_tol_m");
-    if (!lat_ok) p->lat_bup.clear();
+    // the direct sums' mode tiles and the height weights are made from the baselines: other baselines, other tables
+    if (bln != p->lat_bln || bup != p->lat_bup) p->geo_sig.clear();
     p->lat_bln = bln;
+    p->lat_bup.swap(bup);
     p->lat_ok = lat_ok;        // reported whatever the route; the lattice route also needs transform != TYPE3
                                // and dims != 3
     std::memcpy(p->lat_basis, lat_basis, sizeof(lat_basis));

@@ -80,3 +80,61 @@ def test_an_array_that_is_no_lattice_replaces_one(height, precision, eps):
         assert p.info()["transform"] == info["transform"] == ("type3" if ant is moved else "lattice")
         _same(p.run(), ref, precision)
     p.close()
+
+
+def _halves():
+    """Two baseline lists of a hexagon of equal length: one baseline of every longest vector (along the lattice axes, east
+    and north), and half of the other vectors, in different corners of the mode plane."""
+    ant = W.hex_array(3)
+    pairs = W.cross_pairs(len(ant))
+    _, k, _ = fv.fv_lattice_detect(ant)
+    n = k[pairs[:, 0]] - k[pairs[:, 1]]
+    n[(n[:, 1] < 0) | ((n[:, 1] == 0) & (n[:, 0] < 0))] *= -1
+    vec, first = np.unique(n, axis=0, return_index=True)
+    enu = (ant[pairs[:, 0]] - ant[pairs[:, 1]])[first, :2]
+    edge = (np.abs(vec) == np.abs(vec).max(axis=0)).any(axis=1)
+    edge |= (np.isclose(enu, enu.max(axis=0)) | np.isclose(enu, enu.min(axis=0))).any(axis=1)
+    ends, rest = first[edge], first[~edge]
+    m = len(rest) // 2
+    return ant, pairs[np.concatenate([ends, rest[:m]])], pairs[np.concatenate([ends, rest[-m:]])]
+
+
+@pytest.mark.parametrize("precision,eps", [(fv.FV_MIXED, 1e-6), (fv.FV_FP64, 1e-9)])
+def test_other_baselines_of_the_same_lattice(precision, eps):
+    """Baseline lists of equal length and extent with other modes."""
+    prob = W.config_hex127(seed=7, n_chan=2, n_time=1, n_point=2000, nside=0, radius=3)
+    ant, a, b = _halves()
+    sky = (prob.sky.ra, prob.sky.dec, prob.sky.flux)
+    p = _plan(prob, precision, eps)
+    p.set_array(ant, a)
+    p.set_sky(*sky)
+    infos = []
+    for pairs in (a, b, a):
+        p.set_array(ant, pairs)
+        ref, info = _fresh(prob, precision, eps, ant, pairs, sky)
+        infos.append((info["n_bl"], info["n_unique"], info["lattice_modes"]))
+        assert info["transform"] == "lattice"
+        _same(p.run(), ref, precision)
+    assert infos[0] == infos[1]
+    p.close()
+
+
+@pytest.mark.parametrize("precision,eps", [(fv.FV_MIXED, 1e-6), (fv.FV_FP64, 1e-9), (fv.FV_FP64, 1e-13)])
+def test_other_heights_on_the_same_lattice(precision, eps):
+    """The same lattice and number of height terms with other heights (direct sums, and the grid at 1e-13)."""
+    prob = W.config_hex127(seed=8, n_chan=2, n_time=1, n_point=2000, nside=0, radius=3)
+    rng = np.random.default_rng(9)
+    one = W.hex_array(3)
+    one[:, 2] = rng.normal(0.0, 0.05, len(one))
+    two = one.copy()
+    two[:, 2] = -one[::-1, 2]                       # the same largest difference
+    sky = (prob.sky.ra, prob.sky.dec, prob.sky.flux)
+    p = _plan(prob, precision, eps)
+    p.set_array(one)
+    p.set_sky(*sky)
+    for ant in (one, two):
+        p.set_array(ant)
+        ref, info = _fresh(prob, precision, eps, ant, None, sky)
+        assert info["transform"] == "lattice" and info["lattice_terms"] > 1
+        _same(p.run(), ref, precision)
+    p.close()
