@@ -12,6 +12,7 @@
 #include "fv_internal.cuh"
 #include "fv_staged.cuh"
 #include "fv_plan.cuh"
+#include "fv_tables.cuh"
 
 #include <algorithm>
 #include <cmath>
@@ -615,7 +616,7 @@ static fv_status prepare(fv_plan_s *p)
     p->gf.assign(nf, SliceGeom{});
     p->pre_off.assign((size_t)nf * 3, 0);
     p->tw_off.assign((size_t)nf * 3, 0);
-    size_t pre_total = 0, tw_total = 0;
+    size_t pre_total = 0;
     for (int i = 0; i < 3; ++i) { p->nf1_max[i] = 1; p->M_max[i] = 1; }
     size_t grid_e = 0, bufA_e = 0, bufB_e = 0;
     fv_plan_s::WsNeed general;                // general_bytes, in elements here
@@ -625,7 +626,7 @@ static fv_status prepare(fv_plan_s *p)
         const int M = fft_choose_length((int)std::ceil(p->sigma * dg.nf1 - 1e-9), o.radix, o.nstages, p->fft_max_radix);
         return 2 * ((size_t)std::ceil(M / (2.0 * p->sigma) + 0.5 * w) + 1) + 1;
     };
-    std::map<int, size_t> tw_of;
+    TableMap tw_of;
     p->xy_fixed = true;
     for (int f = 0; f < nf; ++f) {
         SliceGeom &g = p->gf[f];
@@ -663,11 +664,7 @@ static fv_status prepare(fv_plan_s *p)
             p->M_max[i] = std::max(p->M_max[i], dg.M);
             p->pre_off[(size_t)f * 3 + i] = pre_total;
             pre_total += dg.nf1;
-            // twiddle tables by length: channels of one length share them (a compile-time length has its own
-            // tables behind the plain one)
-            const auto at = tw_of.emplace(dg.M, tw_total);
-            p->tw_off[(size_t)f * 3 + i] = at.first->second;
-            if (at.second) tw_total += dg.M + (dg.fixed ? fft_fixed_table(dg) : 0);
+            p->tw_off[(size_t)f * 3 + i] = tw_of.place(dg.M, dg.fixed, fft_fixed_table(dg));
         }
         for (int i = 0; i < 2; ++i) {
             const double a = g.kappa * g.dim[i].pscale;
@@ -741,6 +738,7 @@ static fv_status prepare(fv_plan_s *p)
         CK(cudaMemcpyAsync(p->d_tgt_bc, p->h_tgt_bc.data(), (size_t)p->n_u * sizeof(float4), cudaMemcpyHostToDevice,
                            p->stream));
     }
+    const size_t tw_total = tw_of.total();
     const bool reuse = p->d_pre != nullptr && sig == p->geo_sig;
     if (!reuse) free_geometry(p);
     p->geo_sig.clear();
@@ -760,7 +758,7 @@ static fv_status prepare(fv_plan_s *p)
         for (int i = 0; i < p->d; ++i) {
             const DimGeom &dg = p->gf[f].dim[i];
             const size_t to = p->tw_off[(size_t)f * 3 + i];
-            const bool first = tw_of.erase(dg.M) != 0;          // the first dimension of this length makes its tables
+            const bool first = tw_of.take(dg.M, dg.fixed);      // the first axis of this length makes its tables
             if (p->precision == FV_FP64) {
                 CK(launch_prescale_table<double>((double *)p->d_pre + p->pre_off[(size_t)f * 3 + i], dg.nf1, dg.M, w,
                                                  p->beta, p->d_glx, p->d_glw, p->nq, p->stream));
