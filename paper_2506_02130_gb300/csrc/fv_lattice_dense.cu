@@ -31,7 +31,7 @@ namespace fv {
 namespace {
 
 constexpr int kDenseThreads = 256;
-constexpr int kDenseChain = 256;          // sources an FP32 sum takes before it goes to the FP64 sums
+constexpr int kDenseChain = 256;          // sources a thread's sum takes before it goes to the FP64 sums
 
 // the arithmetic of one precision: values in shared memory and the thread's sums
 template <class G> struct Dense;
@@ -389,8 +389,9 @@ __global__ void __launch_bounds__(kDenseThreads, 2)
                 }
             }
             held += (n + groups - 1) / groups;
-            // at the end, and in FP32 before a sum grows long (its rounding grows with the number of its terms)
-            if (block + base + CS >= last || (sizeof(G) == 4 && held >= kDenseChain)) {
+            // at the end, and before a sum grows long: its rounding grows with the number of its terms (pairs: 7e-14 of
+            // the sum after 256, 1.2e-12 after 4,096, 4.6e-12 after 20,000)
+            if (block + base + CS >= last || held >= kDenseChain) {
                 held = 0;
                 flush();
             }
