@@ -61,6 +61,7 @@ namespace {
 
 constexpr int kPsTileX = 16, kPsTileY = 8, kPsPatchX = kPsTileX / 8;    // a warp: 8 x 4 cells
 constexpr int kPsPatches = kPsPatchX * (kPsTileY / 4), kPsThreads = 32 * kPsPatches, kPsChunk = 64;
+constexpr int kPsTidy = 64;                             // sources a warp's sums take between two pair2_tidy
 
 // Horner in pairs; value p (even + s odd) and its mirror (even - s odd)
 __device__ __forceinline__ void pair_kernel(const Pf *es, int p, Pf s, Pf s2, Pf &v, Pf &mirror)
@@ -112,6 +113,7 @@ __global__ void __launch_bounds__(kPsThreads, 512 / kPsThreads) k_spread_pairs(c
     for (int p = 0; p < NP; ++p)
 #pragma unroll
         for (int z = 0; z < NZ; ++z) acc[p][z] = Pair2{make_float2(0.0f, 0.0f), make_float2(0.0f, 0.0f)};
+    int held = 0;                               // sources since the warp's last pair2_tidy
     for (int k = threadIdx.x; k < kPairPoly; k += kPsThreads) s_es[k] = es.v[k];
     if (threadIdx.x < kPsPatches) s_cnt[threadIdx.x] = 0;
     if (threadIdx.x == 0) {
@@ -260,6 +262,14 @@ __global__ void __launch_bounds__(kPsThreads, 512 / kPsThreads) k_spread_pairs(c
                         }
                     }
                 }
+            }
+            held += cnt;
+            if (held >= kPsTidy) {
+                held = 0;
+#pragma unroll
+                for (int p = 0; p < NP; ++p)
+#pragma unroll
+                    for (int z = 0; z < NZ; ++z) pair2_tidy(acc[p][z]);
             }
             __syncthreads();
             if (threadIdx.x < kPsPatches) s_cnt[threadIdx.x] = 0;

@@ -2,7 +2,8 @@
 
 A pair sum whose low part is not kept below the high part's rounding loses accuracy in proportion to its length (4.6e-12
 of the sum after 20,000 terms).  The direct sums go to FP64 after 256 sources: 7e-14 a chain, which adds up as the sums
-do, and a few 2^-47 each for phases and strengths, so 4e-13 in all.
+do, and a few 2^-47 each for phases and strengths, so 4e-13 in all.  The type-3 spreading's cells are tidied as they
+grow: the pair path stays within 1.2 times the FP64 path's error plus 3e-13, as for small skies.
 """
 import dataclasses
 
@@ -24,6 +25,15 @@ def _run(prob, eps, **kw):
         p.close()
 
 
+def _small_array(seed, n_src, z_sigma):
+    prob = W.config_hex127(seed=seed, n_chan=1, n_time=1, n_point=n_src, nside=0, radius=1)
+    rng = np.random.default_rng(seed)
+    prob.ant_enu = W.hex_array(1)
+    prob.ant_enu[:, :2] += rng.normal(0.0, 0.4, (7, 2))
+    prob.ant_enu[:, 2] = rng.normal(0.0, z_sigma, 7) if z_sigma else 0.0
+    return prob
+
+
 @pytest.mark.parametrize("height", [0.0, 0.05])
 def test_direct_sums_of_many_sources(height):
     """Fluxes of both signs through a flat beam (sums that grow as a random walk), 64 channels a launch, so that a channel
@@ -38,3 +48,15 @@ def test_direct_sums_of_many_sources(height):
     e = rel_l2(out[:1], oracle_vis(OracleProblem.from_workload(one), "factored"))
     print(f"error {e:.3e}")
     assert e <= 4e-13
+
+
+@pytest.mark.parametrize("z_sigma", [0.0, 0.05])
+@pytest.mark.parametrize("seed", [1, 2])
+def test_type3_cells_of_many_sources(seed, z_sigma):
+    """1.5 million visible sources on a grid of about 9,000 cells: some 25,000 terms a cell."""
+    prob = _small_array(seed, 3000000, z_sigma)
+    exact = oracle_vis(OracleProblem.from_workload(prob), "factored")
+    e = rel_l2(_run(prob, 1e-11, transform="type3"), exact)
+    e0 = rel_l2(_run(prob, 1e-11, transform="type3", fft_max_radix=8), exact)
+    print(f"error {e:.3e} (FP64 path {e0:.3e})")
+    assert e <= 1.2 * e0 + 3e-13
