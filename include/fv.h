@@ -51,7 +51,7 @@ typedef enum {
 
 typedef enum {
     FV_FP64 = 0,    /* FP64 accuracy; output complex128.  Type-3 slices at sigma = 2 with kernels of at
-                       most 13 points and the mode sums of small lattices (eps >= 1e-12) hold grids and
+                       most 13 points (13: up to 1,000 sources a grid cell) and the mode sums of small lattices (eps >= 1e-12) hold grids and
                        sums as pairs of floats (48 bits), everything else is FP64 */
     FV_MIXED = 1    /* spread, FFT and interpolation in FP32 with FP64 centring,
                        rescaling, phases and deconvolution; output complex64 */

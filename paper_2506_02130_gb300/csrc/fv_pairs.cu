@@ -2,9 +2,11 @@
 //
 // GB300 has 64 FP32 multiply-adds for one of FP64, so an FP64 slice was bound by the FP64 pipe in every step: on the
 // 127-antenna workload (35,000 sources, 10 height terms, 12-point kernel) 1,050 us of spreading, 515 + 420 us of FFT
-// passes and 400 us of interpolation (now 210, 90 + 74 and 62 us).  A pair of floats carries 48 bits, and a multiply-add of pairs takes about 13
-// operations.  FP64 plans take this path at sigma = 2 and kernels of at most 13 points, whose own error (1.7e-12 at
-// w = 13) stays well above the pairs' (about 1e-14 an operation); wider kernels and other sigma keep FP64 throughout.
+// passes and 400 us of interpolation (now 210, 90 + 74 and 62 us).  A pair of floats carries 48 bits, and a multiply-add
+// of pairs takes about 13 operations.  FP64 plans take this path at sigma = 2 and kernels of at most 13 points (at 13
+// points, own error 1.7e-12, only up to kPairTermsMax terms a cell), where the transform's own error stays above the
+// pairs' (about 1e-14 an operation, and growing with the length of the cells' sums); wider kernels and other sigma keep
+// FP64 throughout.
 // FP64 remains in the per-time directions, the strengths, coordinates and phases (k_prep), the per-target set-up and
 // the tables.
 #include "fv_pairs.cuh"

@@ -579,6 +579,13 @@ static fv_status choose_heights(fv_plan_s *p)
     return FV_OK;
 }
 
+// Terms a cell may take on average in pairs with a 13-point kernel.  That kernel's own error (1.7e-12) is near what the
+// pairs' rounding adds up to in long sums: against the FP64 path the error was 1.00 to 1.03 times at 850 and 2,200 terms a
+// cell, 0.95 to 1.11 at 2,900 and 1.23 to 1.66 at 14,000, and the time 0.2 to 0.4 times (300,000 sources, 37 antennas:
+// 0.79 against 2.91 ms; 7 antennas, 2,900 terms: 3.4 against 10.1).  Kernels of 12 points and fewer (1.5e-11) were
+// within 1.02 times at 14,000 terms.
+constexpr double kPairTermsMax = 1000.0;
+
 // FP64 slices in pairs of floats (fv_pairs.cu): sigma = 2, gather spreading (AUTO or asked for), products and planes
 // that its kernels hold, and x and y FFT lengths with a compile-time form in every channel (so in the top one).
 static fv_status choose_pairs(fv_plan_s *p)
@@ -587,16 +594,26 @@ static fv_status choose_pairs(fv_plan_s *p)
     if (p->precision != FV_FP64 || p->use_basis || std::fabs(p->sigma - 2.0) > 1e-12 || p->fft_max_radix != 16 ||
         (p->spread_req != FV_SPREAD_AUTO && p->spread_req != FV_SPREAD_GATHER) || p->n_u <= 0 || !p->d_u_off)
         return FV_OK;
-    const double nu_top = *std::max_element(p->freq.begin(), p->freq.end());
     DimGeom d[3]{};
     p->pairs = true;
-    for (int i = 0; i < p->d; ++i) {
-        if (dim_geometry(p, 2.0 * M_PI * nu_top / FV_C_LIGHT * p->bhalf[i], p->S[i], d[i], i < 2) != FV_OK) {
-            p->err.clear();
+    auto geometry = [&](double nu) {
+        for (int i = 0; i < p->d; ++i)
+            if (dim_geometry(p, 2.0 * M_PI * nu / FV_C_LIGHT * p->bhalf[i], p->S[i], d[i], i < 2) != FV_OK) {
+                p->err.clear();
+                return p->pairs = false;       // prepare reports it
+            }
+        return true;
+    };
+    if (p->w == kPairW) {
+        // the lowest channel's grid has the fewest cells, so the most terms a cell (half of the sources are up)
+        if (!geometry(*std::min_element(p->freq.begin(), p->freq.end()))) return FV_OK;
+        const double terms = 0.5 * p->n_src * p->w * p->w / ((double)d[0].nf1 * d[1].nf1);
+        if (terms > kPairTermsMax) {
             p->pairs = false;
-            return FV_OK;              // prepare reports it
+            return FV_OK;
         }
     }
+    if (!geometry(*std::max_element(p->freq.begin(), p->freq.end()))) return FV_OK;
     const int nz = p->d == 3 ? d[2].nf1 : std::max(p->hK, 1);
     p->pairs = d[0].fixed && d[1].fixed && pairs_fit(p->w, p->n_pol, nz);
     if (p->pairs) p->pair_poly = pair_polynomials(p->w, p->beta);

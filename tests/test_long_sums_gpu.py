@@ -60,3 +60,15 @@ def test_type3_cells_of_many_sources(seed, z_sigma):
     e0 = rel_l2(_run(prob, 1e-11, transform="type3", fft_max_radix=8), exact)
     print(f"error {e:.3e} (FP64 path {e0:.3e})")
     assert e <= 1.2 * e0 + 3e-13
+
+
+@pytest.mark.parametrize("z_sigma", [0.0, 0.05])
+@pytest.mark.parametrize("seed,n_src", [(1, 300000), (1, 1500000), (2, 1500000)])
+def test_long_sums_with_the_widest_pair_kernel_stay_in_fp64(seed, n_src, z_sigma):
+    """At eps 1e-12 the kernel's own error leaves no room for the pairs' rounding in sums of thousands of terms."""
+    prob = _small_array(seed, n_src, z_sigma)
+    exact = oracle_vis(OracleProblem.from_workload(prob), "factored")
+    e = rel_l2(_run(prob, 1e-12, transform="type3"), exact)
+    e0 = rel_l2(_run(prob, 1e-12, transform="type3", fft_max_radix=8), exact)
+    print(f"error {e:.3e} (FP64 path {e0:.3e})")
+    assert e <= 1.02 * e0
