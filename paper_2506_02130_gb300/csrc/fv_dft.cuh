@@ -77,6 +77,9 @@ template <int R> struct Fac {
 
 template <class G, int R> struct Dft;
 
+template <class G> struct Dft<G, 1> {
+    static __device__ __forceinline__ void run(cpx<G> *) {}
+};
 template <class G> struct Dft<G, 2> {
     static __device__ __forceinline__ void run(cpx<G> *v)
     {

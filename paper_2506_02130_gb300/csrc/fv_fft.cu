@@ -313,8 +313,13 @@ cudaError_t fft_pairs_c(FV_FIXED_ARGS(Pf));
 cudaError_t fft_pairs_d(FV_FIXED_ARGS(Pf));
 
 struct FixedLength { short M, R2, R3; };
-// every product 16 R2 R3 up to 4096 of the radices 4, 5, 6, 8, 9, 10, 12, 15, 16, at most 17 % apart above 480
+// every product 16 R2 R3 from 256 to 4096 of the radices 4, 5, 6, 8, 9, 10, 12, 15, 16, at most 17 % apart above 480, and
+// 16 R2 below (two stages), for the short axis of a thin array: with nothing below 256 an axis that needs 20 points had
+// a band of 139 values in place of 27.  East-west line of 60 antennas, 760 m, 0.4 m of scatter across: four products x 7
+// height terms 76 -> 25 MB a stream and 124 -> 103 us a slice, FP64 with 16 up planes 91 -> 36 MB and 463 -> 400 us
+// (general lengths and the spreading that goes with them: 260 and 1,123 us).
 static const FixedLength kFixed[] = {
+    {32, 2, 1}, {48, 3, 1}, {64, 4, 1}, {80, 5, 1}, {96, 6, 1}, {128, 8, 1}, {160, 10, 1}, {192, 12, 1},
     {256, 4, 4}, {320, 5, 4}, {384, 6, 4}, {400, 5, 5}, {480, 6, 5}, {512, 8, 4},
     {576, 6, 6}, {640, 8, 5}, {720, 9, 5}, {768, 8, 6}, {800, 10, 5}, {864, 9, 6},
     {960, 10, 6}, {1024, 8, 8}, {1152, 9, 8}, {1200, 15, 5}, {1280, 10, 8}, {1296, 9, 9},
@@ -330,7 +335,7 @@ bool fft_choose_fixed(int target, int *radix, int &nstages, int &M)
             radix[0] = 16;
             radix[1] = l.R2;
             radix[2] = l.R3;
-            nstages = 3;
+            nstages = l.R3 > 1 ? 3 : 2;
             return true;
         }
     return false;

@@ -1,5 +1,5 @@
 // FFT passes of FP32 grids, and of grids of float pairs (G = Pf: FP64 plans), with compile-time lengths
-// M = 16 R2 R3 (M >= 2 N, no prescale): the same transform as k_fft_rows (zero-padded rows of N values at l - N/2 mod M, sign +, band of outputs m in [-H, B-1-H], written
+// M = 16 R2 R3 (R3 = 1 below 256: the third stage only stores; M >= 2 N, no prescale): the same transform as k_fft_rows (zero-padded rows of N values at l - N/2 mod M, sign +, band of outputs m in [-H, B-1-H], written
 // transposed as out[b][row]).
 //
 // With n = n1 R2 R3 + n2 R3 + n3 and m = m1 + 16 m2 + 16 R2 m3 the transform is three stages of register DFTs,

@@ -1,4 +1,4 @@
-// Instances of the compile-time-length FFT pass, lengths 256 to 864 (one translation unit of several, so
+// Instances of the compile-time-length FFT pass, lengths 32 to 864 (one translation unit of several, so
 // that they compile side by side).
 #include "fv_fft_fixed.cuh"
 
@@ -8,6 +8,14 @@ cudaError_t fft_fixed_a(const cpx<float> *in, cpx<float> *out, int rows, const D
                         int nzp, const cpx<float> *twB, cpx<float> *clr, cudaStream_t st)
 {
     switch (dg.M) {
+    case 32: return fft_fixed_go<float, 2, 1>(in, out, rows, dg, P, sP, nz, nzp, twB, clr, st);
+    case 48: return fft_fixed_go<float, 3, 1>(in, out, rows, dg, P, sP, nz, nzp, twB, clr, st);
+    case 64: return fft_fixed_go<float, 4, 1>(in, out, rows, dg, P, sP, nz, nzp, twB, clr, st);
+    case 80: return fft_fixed_go<float, 5, 1>(in, out, rows, dg, P, sP, nz, nzp, twB, clr, st);
+    case 96: return fft_fixed_go<float, 6, 1>(in, out, rows, dg, P, sP, nz, nzp, twB, clr, st);
+    case 128: return fft_fixed_go<float, 8, 1>(in, out, rows, dg, P, sP, nz, nzp, twB, clr, st);
+    case 160: return fft_fixed_go<float, 10, 1>(in, out, rows, dg, P, sP, nz, nzp, twB, clr, st);
+    case 192: return fft_fixed_go<float, 12, 1>(in, out, rows, dg, P, sP, nz, nzp, twB, clr, st);
     case 256: return fft_fixed_go<float, 4, 4>(in, out, rows, dg, P, sP, nz, nzp, twB, clr, st);
     case 320: return fft_fixed_go<float, 5, 4>(in, out, rows, dg, P, sP, nz, nzp, twB, clr, st);
     case 384: return fft_fixed_go<float, 6, 4>(in, out, rows, dg, P, sP, nz, nzp, twB, clr, st);

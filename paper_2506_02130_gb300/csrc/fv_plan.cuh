@@ -154,6 +154,7 @@ struct fv_plan_s {
     bool pairs = false;         // FP64 slices in pairs of floats (fv_pairs.cu)
     fv::PairPoly pair_poly{};   //   their kernel values as polynomials
     int pair_chunk = 0;         //   targets one interpolation launch takes
+    bool plain = false;         // general FFT lengths only (and with them neither strips nor pairs)
     bool xy_fixed = false;      // every channel's x and y FFT lengths are compile-time lengths (launch_fft_fixed)
     bool strip = false;         // FP32 gather plans, w <= 7: preparation and spreading in one pass (fv_spread_strip.cu)
     fv::EsPoly es_poly{};       //   its kernel values as polynomials

@@ -496,7 +496,7 @@ static fv_status dim_geometry(fv_plan_s *p, double X, double S, DimGeom &dg, boo
     dg.nf1 = next235even(nf1);
     // FP32 grids at sigma >= 2 and FP64 in pairs: a compile-time length where there is one (up to 4,096 points)
     const int target = (int)std::ceil(p->sigma * dg.nf1 - 1e-9);
-    dg.fixed = xy && (p->precision == FV_MIXED ? p->sigma >= 2.0 : p->pairs) && p->fft_max_radix == 16 &&
+    dg.fixed = xy && !p->plain && (p->precision == FV_MIXED ? p->sigma >= 2.0 : p->pairs) && p->fft_max_radix == 16 &&
                fft_choose_fixed(target, dg.radix, dg.nstages, dg.M);
     if (!dg.fixed) dg.M = fft_choose_length(target, dg.radix, dg.nstages, p->fft_max_radix);
     if (dg.M < 0 || dg.M > maxM)
@@ -591,7 +591,7 @@ constexpr double kPairTermsMax = 1000.0;
 static fv_status choose_pairs(fv_plan_s *p)
 {
     p->pairs = false;
-    if (p->precision != FV_FP64 || p->use_basis || std::fabs(p->sigma - 2.0) > 1e-12 || p->fft_max_radix != 16 ||
+    if (p->plain || p->precision != FV_FP64 || p->use_basis || std::fabs(p->sigma - 2.0) > 1e-12 || p->fft_max_radix != 16 ||
         (p->spread_req != FV_SPREAD_AUTO && p->spread_req != FV_SPREAD_GATHER) || p->n_u <= 0 || !p->d_u_off)
         return FV_OK;
     DimGeom d[3]{};
@@ -620,30 +620,29 @@ static fv_status choose_pairs(fv_plan_s *p)
     return FV_OK;
 }
 
-static fv_status prepare(fv_plan_s *p)
+// Sizes of the type-3 slices of a plan: table and buffer elements, and the general form's needs (elements).
+struct SliceSizes {
+    size_t pre_total = 0, grid = 0, bufA = 0, bufB = 0;
+    fv_plan_s::WsNeed general;
+    TableMap tables;
+};
+
+// Grid and FFT geometry of every channel (p->gf and what follows from it).
+static fv_status slice_geometry(fv_plan_s *p, SliceSizes &z)
 {
-    p->pairs = false;
-    const fv_status hs = choose_heights(p);
-    if (hs != FV_OK) return hs;
-    if (p->use_basis) return prepare_basis(p);
-    const fv_status cps = choose_pairs(p);
-    if (cps != FV_OK) return cps;
     const int nf = (int)p->freq.size();
     const int w = p->w;
     p->gf.assign(nf, SliceGeom{});
     p->pre_off.assign((size_t)nf * 3, 0);
     p->tw_off.assign((size_t)nf * 3, 0);
-    size_t pre_total = 0;
+    z = SliceSizes{};
     for (int i = 0; i < 3; ++i) { p->nf1_max[i] = 1; p->M_max[i] = 1; }
-    size_t grid_e = 0, bufA_e = 0, bufB_e = 0;
-    fv_plan_s::WsNeed general;                // general_bytes, in elements here
     const auto general_B = [&](const DimGeom &dg) {
         if (!dg.fixed) return (size_t)dg.B;
         DimGeom o{};
         const int M = fft_choose_length((int)std::ceil(p->sigma * dg.nf1 - 1e-9), o.radix, o.nstages, p->fft_max_radix);
         return 2 * ((size_t)std::ceil(M / (2.0 * p->sigma) + 0.5 * w) + 1) + 1;
     };
-    TableMap tw_of;
     p->xy_fixed = true;
     for (int f = 0; f < nf; ++f) {
         SliceGeom &g = p->gf[f];
@@ -679,9 +678,9 @@ static fv_status prepare(fv_plan_s *p)
             dg.C = p->C[i];
             p->nf1_max[i] = std::max(p->nf1_max[i], dg.nf1);
             p->M_max[i] = std::max(p->M_max[i], dg.M);
-            p->pre_off[(size_t)f * 3 + i] = pre_total;
-            pre_total += dg.nf1;
-            p->tw_off[(size_t)f * 3 + i] = tw_of.place(dg.M, dg.fixed, fft_fixed_table(dg));
+            p->pre_off[(size_t)f * 3 + i] = z.pre_total;
+            z.pre_total += dg.nf1;
+            p->tw_off[(size_t)f * 3 + i] = z.tables.place(dg.M, dg.fixed, fft_fixed_table(dg));
         }
         for (int i = 0; i < 2; ++i) {
             const double a = g.kappa * g.dim[i].pscale;
@@ -698,20 +697,114 @@ static fv_status prepare(fv_plan_s *p)
         size_t pass2 = (size_t)D[1].B * D[0].B * p->n_pol * D[2].nf1;
         size_t pass3 = p->d == 3 && D[2].nf1 > FV_ZDIRECT_MAX ? (size_t)D[2].B * D[1].B * D[0].B * p->n_pol : 0;
         const size_t gb[3] = {general_B(D[0]), general_B(D[1]), general_B(D[2])}, npl = (size_t)p->n_pol * D[2].nf1;
-        general.grid = std::max(general.grid, npl * D[0].nf1 * D[1].nf1);
-        general.bufA = std::max({general.bufA, gb[0] * npl * D[1].nf1, p->d == 3 ? gb[2] * gb[1] * gb[0] * p->n_pol : 0});
-        general.bufB = std::max(general.bufB, gb[1] * gb[0] * npl);
-        grid_e = std::max(grid_e, grid_c);
-        bufA_e = std::max(bufA_e, std::max(pass1, pass3));
-        bufB_e = std::max(bufB_e, pass2);
+        z.general.grid = std::max(z.general.grid, npl * D[0].nf1 * D[1].nf1);
+        z.general.bufA = std::max({z.general.bufA, gb[0] * npl * D[1].nf1, p->d == 3 ? gb[2] * gb[1] * gb[0] * p->n_pol : 0});
+        z.general.bufB = std::max(z.general.bufB, gb[1] * gb[0] * npl);
+        z.grid = std::max(z.grid, grid_c);
+        z.bufA = std::max(z.bufA, std::max(pass1, pass3));
+        z.bufB = std::max(z.bufB, pass2);
     }
+    return FV_OK;
+}
+
+// What a workspace holds for the plan's slices (after resolve_spread); static_need: the general form's bytes.
+static fv_plan_s::WsNeed slice_need(fv_plan_s *p, const SliceSizes &z, size_t &static_need)
+{
     const size_t es = p->elem();
     const size_t gs = p->precision == FV_FP64 ? sizeof(double) : sizeof(float);
+    fv_plan_s::WsNeed need;
+    need.grid = std::max<size_t>(z.grid, 1) * es;
+    need.bufA = std::max<size_t>(z.bufA, 1) * es;
+    need.bufB = std::max<size_t>(z.bufB, 1) * es;
+    need.vu = std::max<size_t>((size_t)p->n_u * p->n_pol, 1) * sizeof(cpx<double>);
+    need.tiled = p->tiled;
+    need.n_src = std::max<long>(p->n_src, 1);
+    need.nb = p->nbx * p->nby;
+    // the gather spreading reads staged records: 16 (FP32) or 32 (FP64) bytes per source where the split
+    // coordinates take 12 or 24, and strengths padded to 16 bytes
+    const bool staged = p->spread_method == FV_SPREAD_GATHER || p->spread_method == FV_SPREAD_TENSOR;
+    need.frac_per_src = p->strip ? 0 : (p->ring ? sizeof(RingRec) : (staged ? 4 * gs : 3 * gs));
+    // ring gather: a work list over the tiles of the largest grid, and slots for the parts of split tiles
+    // (a tile's candidates come to at most 4 n_src, split tiles have more than kRingPart candidates each,
+    // so there are at most 8 n_src / kRingPart parts; beyond kRingSlotsMax tiles run whole)
+    need.ring_tiles = p->ring ? ring_tiles(p->nf1_max[0], p->nf1_max[1]) : 0;
+    need.ring_slots = p->ring ? (int)std::min<long>(kRingSlotsMax, 8 * std::max<long>(p->n_src, 1) / kRingPart + 1) : 0;
+    need.ring_np = p->ring ? p->n_pol : 0;
+    need.cs_per_src =
+        p->strip ? 0 : (staged ? (size_t)staged_cs_stride((int)gs, p->n_pol) * es : (size_t)p->n_pol * es);
+    // FP32 grids take each slice's coordinates and prephase from per-time records (no FP64 per slice)
+    need.tc = p->precision == FV_MIXED && p->tiled;
+    // pairs: about 2 MB of targets a launch; no visibilities per target (the output is written directly) and no cells
+    need.cells = !p->pairs;
+    need.pairs = 0;
+    if (p->pairs) {
+        const size_t per = sizeof(PairTarget) + sizeof(cpx<Pf>) * p->nf1_max[2] * (p->d == 3 ? 1 : 0) +
+                           sizeof(cpx<Pf>) * std::max(p->hK, 1);
+        p->pair_chunk = (int)std::min<size_t>(p->n_u, ((size_t)2 << 20) / per);
+        need.pairs = 256 + p->pair_chunk * per;
+        need.vu = sizeof(cpx<double>);
+    }
+    need.apart = false;
+    // the general form: its spreading method, bins of 8 x 4 cells and records
+    fv_plan_s::WsNeed general = z.general;
+    general.grid *= es;
+    general.bufA *= es;
+    general.bufB *= es;
+    general.vu = std::max<size_t>((size_t)p->n_u * p->n_pol, 1) * sizeof(cpx<double>);
+    const bool g_staged = p->general_method == FV_SPREAD_GATHER || p->general_method == FV_SPREAD_TENSOR;
+    const bool g_ring = p->ring_ok && g_staged;
+    const int gT[2] = {p->bin_req[0] > 0 ? p->bin_req[0] : 8, p->bin_req[1] > 0 ? p->bin_req[1] : 4};
+    general.tiled = p->general_method != FV_SPREAD_ATOMIC;
+    general.n_src = std::max<long>(p->n_src, 1);
+    general.nb = ((p->nf1_top[0] + gT[0] - 1) / gT[0]) * ((p->nf1_top[1] + gT[1] - 1) / gT[1]);
+    general.frac_per_src = g_ring ? sizeof(RingRec) : (g_staged ? 4 * gs : 3 * gs);
+    general.cs_per_src = g_staged ? (size_t)staged_cs_stride((int)gs, p->n_pol) * es : (size_t)p->n_pol * es;
+    general.tc = p->precision == FV_MIXED && general.tiled;
+    general.ring_tiles = g_ring ? ring_tiles(p->nf1_max[0], p->nf1_max[1]) : 0;
+    general.ring_slots = g_ring ? (int)std::min<long>(kRingSlotsMax, 8 * std::max<long>(p->n_src, 1) / kRingPart + 1) : 0;
+    general.ring_np = g_ring ? p->n_pol : 0;
+    static_need = general_bytes(general);
+    if (p->strip) {
+        // beside a small grid, but where the static scratch takes the plan and would not hold it so
+        need.apart = need.grid <= kClearInPass;
+        if (static_need <= FV_STATIC_SCRATCH_BYTES && workspace_layout(need, nullptr, nullptr) > FV_STATIC_SCRATCH_BYTES)
+            need.apart = false;
+    }
+    return need;
+}
+
+static fv_status prepare(fv_plan_s *p)
+{
+    p->pairs = p->plain = false;
+    const fv_status hs = choose_heights(p);
+    if (hs != FV_OK) return hs;
+    if (p->use_basis) return prepare_basis(p);
+    const int nf = (int)p->freq.size();
+    const int w = p->w;
+    const size_t es = p->elem();
+    const size_t gs = p->precision == FV_FP64 ? sizeof(double) : sizeof(float);
+    SliceSizes z;
+    fv_plan_s::WsNeed need;
+    size_t static_need = 0;
+    for (;; p->plain = true) {
+        const fv_status cps = choose_pairs(p);
+        if (cps != FV_OK) return cps;
+        const fv_status ss = slice_geometry(p, z);
+        if (ss != FV_OK) return ss;
+        resolve_spread(p, (int)gs, w);
+        need = slice_need(p, z, static_need);
+        // a compile-time length can be longer than the general one, its band with it, and pairs hold targets: where the
+        // static scratch takes the general form and not this one, the plan has the general form (rarely: the form in
+        // use shares the grid's place with the second band and mostly needs less)
+        if (p->plain || static_need > FV_STATIC_SCRATCH_BYTES ||
+            workspace_layout(need, nullptr, nullptr) <= FV_STATIC_SCRATCH_BYTES)
+            break;
+    }
     // a new sky with the same grid sizes (the usual case: same array, same channels) keeps the
     // tables and workspaces of the previous one
     std::vector<long> sig = {(long)p->n_src, (long)p->n_pol, (long)p->n_streams, (long)p->spread_req, (long)p->d,
-                             (long)p->hK, (long)p->pairs,
-                             (long)grid_e, (long)bufA_e, (long)bufB_e, (long)p->lat_ok, (long)p->lat_H[0],
+                             (long)p->hK, (long)p->pairs, (long)p->plain,
+                             (long)z.grid, (long)z.bufA, (long)z.bufB, (long)p->lat_ok, (long)p->lat_H[0],
                              (long)p->lat_H[1], (long)p->n_u, (long)p->n_bl};
     for (int k = 0; k < 4; ++k) {
         long long bits;
@@ -755,27 +848,23 @@ static fv_status prepare(fv_plan_s *p)
         CK(cudaMemcpyAsync(p->d_tgt_bc, p->h_tgt_bc.data(), (size_t)p->n_u * sizeof(float4), cudaMemcpyHostToDevice,
                            p->stream));
     }
-    const size_t tw_total = tw_of.total();
+    const size_t tw_total = z.tables.total();
     const bool reuse = p->d_pre != nullptr && sig == p->geo_sig;
     if (!reuse) free_geometry(p);
     p->geo_sig.clear();
     if (reuse) {
-        resolve_spread(p, (int)gs, w);
         p->geo_sig = sig;
         return FV_OK;        // the lattice route's tables and decision depend on the array only (setup_array): kept
     }
-    CK(cudaMalloc(&p->d_pre, std::max<size_t>(pre_total, 1) * gs));
+    CK(cudaMalloc(&p->d_pre, std::max<size_t>(z.pre_total, 1) * gs));
     CK(cudaMalloc(&p->d_tw, std::max<size_t>(tw_total, 1) * es));
-    p->need = fv_plan_s::WsNeed{};      // another route may have set it (prepare_lattice)
-    p->need.grid = std::max<size_t>(grid_e, 1) * es;
-    p->need.bufA = std::max<size_t>(bufA_e, 1) * es;
-    p->need.bufB = std::max<size_t>(bufB_e, 1) * es;
-    p->need.vu = std::max<size_t>((size_t)p->n_u * p->n_pol, 1) * sizeof(cpx<double>);
+    p->need = need;
+    p->static_need = static_need;
     for (int f = 0; f < nf; ++f) {
         for (int i = 0; i < p->d; ++i) {
             const DimGeom &dg = p->gf[f].dim[i];
             const size_t to = p->tw_off[(size_t)f * 3 + i];
-            const bool first = tw_of.take(dg.M, dg.fixed);      // the first axis of this length makes its tables
+            const bool first = z.tables.take(dg.M, dg.fixed);      // the first axis of this length makes its tables
             if (p->precision == FV_FP64) {
                 CK(launch_prescale_table<double>((double *)p->d_pre + p->pre_off[(size_t)f * 3 + i], dg.nf1, dg.M, w,
                                                  p->beta, p->d_glx, p->d_glw, p->nq, p->stream));
@@ -791,60 +880,7 @@ static fv_status prepare(fv_plan_s *p)
             }
         }
     }
-    resolve_spread(p, (int)gs, w);
-    p->need.tiled = p->tiled;
-    p->need.n_src = std::max<long>(p->n_src, 1);
-    p->need.nb = p->nbx * p->nby;
-    // the gather spreading reads staged records: 16 (FP32) or 32 (FP64) bytes per source where the split
-    // coordinates take 12 or 24, and strengths padded to 16 bytes
-    const bool staged = p->spread_method == FV_SPREAD_GATHER || p->spread_method == FV_SPREAD_TENSOR;
-    p->need.frac_per_src = p->strip ? 0 : (p->ring ? sizeof(RingRec) : (staged ? 4 * gs : 3 * gs));
-    // ring gather: a work list over the tiles of the largest grid, and slots for the parts of split tiles
-    // (a tile's candidates come to at most 4 n_src, split tiles have more than kRingPart candidates each,
-    // so there are at most 8 n_src / kRingPart parts; beyond kRingSlotsMax tiles run whole)
-    p->need.ring_tiles = p->ring ? ring_tiles(p->nf1_max[0], p->nf1_max[1]) : 0;
-    p->need.ring_slots = p->ring ? (int)std::min<long>(kRingSlotsMax, 8 * std::max<long>(p->n_src, 1) / kRingPart + 1) : 0;
-    p->need.ring_np = p->ring ? p->n_pol : 0;
-    p->need.cs_per_src =
-        p->strip ? 0 : (staged ? (size_t)staged_cs_stride((int)gs, p->n_pol) * es : (size_t)p->n_pol * es);
-    // FP32 grids take each slice's coordinates and prephase from per-time records (no FP64 per slice)
-    p->need.tc = p->precision == FV_MIXED && p->tiled;
-    // pairs: about 2 MB of targets a launch; no visibilities per target (the output is written directly) and no cells
-    p->need.cells = !p->pairs;
-    p->need.pairs = 0;
-    if (p->pairs) {
-        const size_t per = sizeof(PairTarget) + sizeof(cpx<Pf>) * p->nf1_max[2] * (p->d == 3 ? 1 : 0) +
-                           sizeof(cpx<Pf>) * std::max(p->hK, 1);
-        p->pair_chunk = (int)std::min<size_t>(p->n_u, ((size_t)2 << 20) / per);
-        p->need.pairs = 256 + p->pair_chunk * per;
-        p->need.vu = sizeof(cpx<double>);
-    }
-    p->need.apart = false;
-    // the general form: its spreading method, bins of 8 x 4 cells and records
-    general.grid *= es;
-    general.bufA *= es;
-    general.bufB *= es;
-    general.vu = std::max<size_t>((size_t)p->n_u * p->n_pol, 1) * sizeof(cpx<double>);
-    const bool g_staged = p->general_method == FV_SPREAD_GATHER || p->general_method == FV_SPREAD_TENSOR;
-    const bool g_ring = p->ring_ok && g_staged;
-    const int gT[2] = {p->bin_req[0] > 0 ? p->bin_req[0] : 8, p->bin_req[1] > 0 ? p->bin_req[1] : 4};
-    general.tiled = p->general_method != FV_SPREAD_ATOMIC;
-    general.n_src = std::max<long>(p->n_src, 1);
-    general.nb = ((p->nf1_top[0] + gT[0] - 1) / gT[0]) * ((p->nf1_top[1] + gT[1] - 1) / gT[1]);
-    general.frac_per_src = g_ring ? sizeof(RingRec) : (g_staged ? 4 * gs : 3 * gs);
-    general.cs_per_src = g_staged ? (size_t)staged_cs_stride((int)gs, p->n_pol) * es : (size_t)p->n_pol * es;
-    general.tc = p->precision == FV_MIXED && general.tiled;
-    general.ring_tiles = g_ring ? ring_tiles(p->nf1_max[0], p->nf1_max[1]) : 0;
-    general.ring_slots = g_ring ? (int)std::min<long>(kRingSlotsMax, 8 * std::max<long>(p->n_src, 1) / kRingPart + 1) : 0;
-    general.ring_np = g_ring ? p->n_pol : 0;
-    p->static_need = general_bytes(general);
-    if (p->strip) {
-        // beside a small grid, but where the static scratch takes the plan and would not hold it so
-        p->need.apart = p->need.grid <= kClearInPass;
-        if (p->static_need <= FV_STATIC_SCRATCH_BYTES && workspace_layout(p->need, nullptr, nullptr) > FV_STATIC_SCRATCH_BYTES)
-            p->need.apart = false;
-    }
-    p->ws_bytes = (long long)(pre_total * gs + tw_total * es + p->n_streams * workspace_layout(p->need, nullptr, nullptr));
+    p->ws_bytes = (long long)(z.pre_total * gs + tw_total * es + p->n_streams * workspace_layout(p->need, nullptr, nullptr));
     fv_status ls = prepare_lattice(p);
     if (ls != FV_OK) return ls;
     CK(cudaStreamSynchronize(p->stream));
