@@ -1145,8 +1145,9 @@ fv_status run_slices(fv_plan_s *p, fv_plan_s::Workspace &wk, cudaStream_t st, ch
                 CK(prof_begin(p, PC_SPREAD, st));
                 CK(launch_spread_strip(wk.tc, wk.sidx, wk.offsets + nb, p->n_src, p->flux, p->flux_fp64, nf, f, g,
                                        p->es_poly, (cpx<float> *)grid, st));
-                // the visible sources' records, indexes and fluxes read once, the grid written once
-                CK(prof_end(p, nvis * (48.0 + 4.0 + p->n_stokes * (p->flux_fp64 ? 8.0 : 4.0)) + gel * es));
+                // the visible sources' fluxes read once and the grid written once, as for the other methods (the records and
+                // indexes are the sort's output, counted there)
+                CK(prof_end(p, nvis * p->n_stokes * (p->flux_fp64 ? 8.0 : 4.0) + gel * es));
             } else if (p->tiled) {
                 G *frac = (G *)wk.frac;
                 cpx<G> *cs = (cpx<G> *)wk.cs;
