@@ -426,6 +426,9 @@ cudaError_t launch_flux_transpose(const void *flux, int fp64, long n_src, int n_
 // ep (nullable): the same as float pairs, [3][n].
 cudaError_t launch_radec_to_unit(const double *ra, const double *dec, long n, double *e, float2 *ep, cudaStream_t st);
 
+// *bad |= 1 if one of v[0..n) is an infinity or NaN.
+cudaError_t launch_find_nonfinite(const double *v, long n, int *bad, cudaStream_t st);
+
 // Per-block min/max of visible ENU directions over all times: out[nblocks][6].
 cudaError_t launch_source_extents(const double *e, long n, const double *R_all, int n_time,
                                   double *out, int nblocks, cudaStream_t st);

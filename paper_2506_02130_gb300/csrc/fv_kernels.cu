@@ -65,6 +65,21 @@ __global__ void k_radec_to_unit(const double *ra, const double *dec, long n, dou
     }
 }
 
+// *bad |= 1 where a value is an infinity or NaN
+__global__ void __launch_bounds__(256) k_find_nonfinite(const double *__restrict__ v, long n, int *bad)
+{
+    bool any = false;
+    for (long i = blockIdx.x * 256L + threadIdx.x; i < n; i += gridDim.x * 256L) any = any || !isfinite(v[i]);
+    if (any) atomicOr(bad, 1);
+}
+
+cudaError_t launch_find_nonfinite(const double *v, long n, int *bad, cudaStream_t st)
+{
+    if (n <= 0) return cudaSuccess;
+    k_find_nonfinite<<<(unsigned)std::min<long>((n + 255) / 256, 1216), 256, 0, st>>>(v, n, bad);
+    return cudaGetLastError();
+}
+
 // out[f][n][k] = in[k][n][f], f0 <= f < f1, through a shared tile of S sources x C channels (C at most 32, S C about
 // 1,024) of every Stokes parameter: reads run along the channels of a source (all of them at once where the tile
 // holds them all), writes along (source, Stokes), a source's values in one store.  The rows of a tile are C | 1

@@ -1680,21 +1680,6 @@ static fv_status execute_slices(fv_plan_s *p, char *vis, size_t slice_bytes, cha
     return FV_OK;
 }
 
-// *bad |= 1 where a value is an infinity or NaN
-static __global__ void __launch_bounds__(256) k_find_nonfinite(const double *__restrict__ v, long n, int *bad)
-{
-    bool any = false;
-    for (long i = blockIdx.x * 256L + threadIdx.x; i < n; i += gridDim.x * 256L) any = any || !isfinite(v[i]);
-    if (any) atomicOr(bad, 1);
-}
-
-static cudaError_t launch_find_nonfinite(const double *v, long n, int *bad, cudaStream_t st)
-{
-    if (n <= 0) return cudaSuccess;
-    k_find_nonfinite<<<(unsigned)std::min<long>((n + 255) / 256, 1216), 256, 0, st>>>(v, n, bad);
-    return cudaGetLastError();
-}
-
 extern "C" {
 
 void fv_opts_default(fv_opts *o)
