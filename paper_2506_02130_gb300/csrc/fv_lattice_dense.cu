@@ -468,7 +468,23 @@ static size_t dense_smem(const DenseGeom &dg, int elem)
            (size_t)kDenseThreads * ((elem == 4 ? 4 : 8) * 4 + (size_t)JB * elem);
 }
 
-bool dense_plan(int elem, double eps, int K, int n_pol, int H1, int H2, int n_bl, const int *bln, DenseGeom &dg,
+// Modes up to which J sums a mode are faster than the type-1 transform of a w-point kernel, for skies of more than
+// kDenseFew sources.  FP32: a source costs the direct sums modes (2 + J) multiply-adds and the grid about J (1,000 + 33 w^2)
+// of them.  FP64 (pairs): the sums of 4 terms go together, so the cost goes by the terms rounded up to fours (one term
+// alone: two of them), against J (70 + 1.85 w^2) and the FP64 preparation.  Measured per slice (200,000 sources, 16
+// channels), direct sums against the grid: FP32, one term: 325 modes 36.5 / 37.3 us (w = 4), 861 modes 53.5 / 39.9 (w = 4)
+// and 53.7 / 49.2 (w = 7: kept, its error is a quarter of the grid's), 1,431 modes 69.5 / 41.9 (w = 4), 69.6 / 51.1 (w = 7);
+// 5 terms, w = 4: 861 modes 112 / 111, 1,431 modes 157 / 119.  FP64, one term: 861 modes 274 / 187 (w = 4), 274 / 264 (w = 7),
+// 1,431 modes 440 / 269 (w = 7), 440 / 399 (w = 11); 5 terms, w = 4: 325 modes 408 / 453, 861 modes 1,013 / 633; 7 terms,
+// w = 7: 1,431 modes 1,383 / 1,235.
+static double dense_modes_max(int elem, int w, int J)
+{
+    if (elem == 4) return J * (1000.0 + 33.0 * w * w) / (J + 2.0);
+    const int slots = J == 1 ? 2 : (J + 3) / 4 * 4;
+    return (95.0 + J * (70.0 + 1.85 * w * w)) / (0.14 * slots);
+}
+
+bool dense_plan(int elem, double eps, int w, long n_src, int K, int n_pol, int H1, int H2, int n_bl, const int *bln, DenseGeom &dg,
                 std::vector<int> &tiles)
 {
     if (elem == 8 && eps < 1e-12) return false;
@@ -483,7 +499,9 @@ bool dense_plan(int elem, double eps, int K, int n_pol, int H1, int H2, int n_bl
     // sources a chunk: as many as two CTAs an SM hold tables for, 64 at most (fewer barriers)
     dg.CS = 64;
     while (dg.CS > 8 && dense_smem(dg, elem) > 100 * 1024) dg.CS /= 2;
-    if ((long)(2 * H1 + 1) * (H2 + 1) > kDenseModes || dense_smem(dg, elem) > 100 * 1024) return false;
+    const long modes = (long)(2 * H1 + 1) * (H2 + 1);
+    if (modes > kDenseModes || dense_smem(dg, elem) > 100 * 1024) return false;
+    if (n_src > kDenseFew && (double)modes > dense_modes_max(elem, w, dg.J)) return false;
     // the tiles that hold a mode of some baseline
     const int ta = dg.NA / TA, tb = dg.NB / TB;
     std::vector<char> need((size_t)ta * tb, 0);

@@ -6,10 +6,11 @@
 
 namespace fv {
 
-// Largest (2 H_1 + 1)(H_2 + 1) evaluated directly.  A mode of a source costs about a thirtieth of a footprint cell of
-// the spreading's shared-memory atomics (w^2 of those a source), so the direct sum stays ahead to well over a
-// thousand modes; larger lattices keep the grid.
+// Largest (2 H_1 + 1)(H_2 + 1) evaluated directly, for skies of up to kDenseFew sources: the grid's clearing, FFT passes
+// and launches cost twice a small sky's direct sums (2,000 sources, 1,431 modes, one term, 16 channels: 6.6 against
+// 16.6 us a slice in FP32, 12.6 against 32.7 in FP64).  Larger skies: dense_modes_max.
 constexpr int kDenseModes = 1600;
+constexpr long kDenseFew = 50000;
 
 struct DenseGeom {
     double a[2][2];          // lattice vectors (east, north), m
@@ -23,7 +24,7 @@ struct DenseGeom {
 inline size_t dense_modes(const DenseGeom &dg) { return (size_t)dg.J * (2 * dg.H1 + 1) * (dg.H2 + 1); }
 
 // Host: the geometry (without a and tiles) and its tile list, or false where the grid has to do it.
-bool dense_plan(int elem, double eps, int K, int n_pol, int H1, int H2, int n_bl, const int *bln, DenseGeom &dg,
+bool dense_plan(int elem, double eps, int w, long n_src, int K, int n_pol, int H1, int H2, int n_bl, const int *bln, DenseGeom &dg,
                 std::vector<int> &tiles);
 
 // Mode sums (FP64) [nch][J][H_2 + 1][2 H_1 + 1] of channels f0 .. f0 + nch of one time from its sources above the horizon

@@ -403,7 +403,7 @@ static fv_status prepare_lattice(fv_plan_s *p)
     dfree_t(p->d_lat_dec);
     // the mode sums directly where the lattice is small enough (fv_lattice_dense.cu), else the type-1 transform
     std::vector<int> tiles;
-    p->lat_dense = dense_plan((int)gs, p->eps, K, p->n_pol, lg.H[0], lg.H[1], p->n_bl, p->lat_bln.data(), p->dense, tiles);
+    p->lat_dense = dense_plan((int)gs, p->eps, w, p->n_src, K, p->n_pol, lg.H[0], lg.H[1], p->n_bl, p->lat_bln.data(), p->dense, tiles);
     dfree_t(p->d_lat_tiles);
     dfree_t(p->d_lat_freq);
     if (p->lat_dense) {
