@@ -52,9 +52,9 @@ def parse():
     ap.add_argument("--fft-radix", type=int, default=0, choices=[0, 8, 16],
                     help="largest FFT stage radix of the timed plan (0: the library default)")
     ap.add_argument("--fp64-eps", type=float, default=1e-6,
-                    help="tolerance of the plain FP64 comparison leg (its error is reported beside the mixed path's)")
+                    help="tolerance of the FP64 comparison leg (its error is reported beside the mixed path's)")
     ap.add_argument("--no-fp64-compare", action="store_true",
-                    help="skip timing the plain FP64 path (one slice after another) beside the mixed path")
+                    help="skip timing FP64 plans (one slice after another) beside the mixed path")
     ap.add_argument("--workload", default="hex350", choices=["hex350", "hex127", "batch", "serve"],
                     help="hex350: the 350-antenna polarised simulation, 256 channels x 4 times, 886,432 sources "
                          "(default); hex127: the 127-antenna, 64-channel, 10-time simulation; batch: 2,048 ragged "
@@ -376,7 +376,8 @@ def run_batch(args, rank, world, local, dist):
                           "(lanes overlap, so per-class times add concurrent launches)"}
     gpu_launches = int(sum(v["launches"] for k, v in prof.items() if k != "memset")) * args.steps
 
-    # the plain FP64 path, one slice per fv_execute, each slice alone (device time of that call)
+    # FP64 plans (pairs of floats where the library takes them), one slice per fv_execute, each slice alone (device time
+    # of that call)
     plain = None
     if not args.no_fp64_compare:
         tot = 0.0
@@ -522,7 +523,7 @@ def run_serve(args, rank, world, local, dist):
     for p in plans.values():
         launches += sum(v["launches"] for k, v in fv.fv_profile_read(p.handle).items() if k != "memset")
 
-    # the plain FP64 path: one slice per fv_execute on an FP64 plan of each array (device time per slice)
+    # FP64 plans: one slice per fv_execute on an FP64 plan of each array (device time per slice)
     plain = None
     if not args.no_fp64_compare:
         per = {}
@@ -923,8 +924,8 @@ def run_sim(args, rank, world, local, dist):
                                   "function of the band (Appendix A), expanded to the channels in the "
                                   "interpolation"})
 
-    # ---- the plain FP64 path at equal accuracy: one slice after another on one stream (no batching, no
-    # concurrent slices), at the tolerance whose error matches the mixed path's; on the 350-antenna
+    # ---- an FP64 plan at equal accuracy (grids and sums in pairs of floats): one slice after another on one stream (no
+    # batching, no concurrent slices), at the tolerance whose error matches the mixed path's; on the 350-antenna
     # workload a seeded subset of channels (all times) keeps the leg short
     fp64 = None
     extra_slices = []
@@ -954,7 +955,7 @@ def run_sim(args, rank, world, local, dist):
         fp64 = {"value": world * n64 * 3 / (ms64 / 1e3), "unit": "visibilities/s", "ms_per_step": ms64 / 3,
                 "eps": args.fp64_eps, "steps": 3, "warmup": 1, "streams": 1, "channels": len(ch),
                 "visibilities_per_step": n64, "kernel_width": p64.info()["kernel_width"],
-                "what": "plain FP64 type-3 path, one slice after another on one stream, at the tolerance whose "
+                "what": "FP64 type-3 plan (pairs of floats), one slice after another on one stream, at the tolerance whose "
                         "error against the direct sum matches the mixed path's (error in "
                         "rel_l2_vs_oracle_sample.fp64_plain)"
                         + (f"; channels {ch[0]}, {ch[1]}, ... (every 16th) of the {nf}, all times"

@@ -51,10 +51,16 @@ typedef enum {
 
 typedef enum {
     FV_FP64 = 0,    /* FP64 accuracy; output complex128.  Type-3 slices at sigma = 2 with kernels of at
-                       most 13 points (13: up to 1,000 sources a grid cell) and the mode sums of small lattices (eps >= 1e-12) hold grids and
-                       sums as pairs of floats (48 bits), everything else is FP64 */
-    FV_MIXED = 1    /* spread, FFT and interpolation in FP32 with FP64 centring,
-                       rescaling, phases and deconvolution; output complex64 */
+                       most 13 points (13: up to 1,000 sources a grid cell on average) and the mode
+                       sums of small lattices (eps >= 1e-12) hold grids, kernel values and sums as
+                       pairs of floats (48 bits) with FP64 directions, strengths, coordinates and
+                       phases; everything else is FP64.  spread_method = FV_SPREAD_SCATTER or
+                       FV_SPREAD_ATOMIC with transform = FV_TRANSFORM_TYPE3 keeps every step in FP64 */
+    FV_MIXED = 1    /* beam, spreading, FFT and interpolation in FP32; source directions, centring, grid
+                       geometry and tables in FP64; the coordinates and phase arguments of sources and
+                       of the targets of FP32 interpolations as pairs of floats (48 bits), their sines,
+                       the height weights and the deconvolution factors applied in FP32; output
+                       complex64 */
 } fv_precision;
 
 typedef enum {

@@ -6,11 +6,11 @@
 // the real strengths I + Q', I - Q', U', V), so W_j(-n) = conj W_j(n) and half of the modes do.  A source costs one
 // complex product per mode, shared by all terms, and one packed multiply-add per mode and term, all in registers:
 // a thread holds a tile of modes x terms and walks the sources, whose phase factors e^{-i n x} and real strengths
-// the CTA has put in shared memory 32 (16 in FP64) at a time.  Groups of threads and CTAs take different sources and
+// the CTA has put in shared memory up to 64 at a time.  Groups of threads and CTAs take different sources and
 // add their sums with global reductions.  There is no spreading kernel, grid, FFT or deconvolution, and every
 // channel of a time goes into one launch.
 //
-// Why: the type-1 transform of such an array spread each source over w^2 cells of every term's grid with
+// Why (skies of up to 50,000 sources, or few enough modes: dense_modes_max): the type-1 transform of such an array spread each source over w^2 cells of every term's grid with
 // shared-memory float atomics (each a compare-and-swap loop): 74 us of a 127-antenna slice (35,000 sources, 7 terms)
 // beside 35 us for strengths, clearing, FFT passes and lookup.  The direct sum has more multiply-adds (about 290
 // modes x 9 packed operations a source) but they run on the FMA pipe, about 40 % of whose rate it reaches: 17.7 us

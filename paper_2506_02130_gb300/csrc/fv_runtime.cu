@@ -384,11 +384,13 @@ static fv_status prepare_lattice(fv_plan_s *p)
         return FV_OK;
     }
     if (p->transform_req == FV_TRANSFORM_AUTO && cells * K > t3) return FV_OK;
-    // four products: the lattice spreading adds every product of every source with global atomics into one
-    // small grid, which contends; measured per slice on the 350-antenna workload (886k sources, K = 1) the
-    // lattice route took 0.52 ms against the type-3 route's 0.20 ms (about 6 N K units against N + t3 for
-    // the type-3 spreading and FFT passes), so auto keeps polarised plans on the type-3 route unless
-    // 6 N K < N + t3
+    // Four products: type-3 unless 6 N K < N + t3.  This line and the one above compare the grids of the two transforms;
+    // they were drawn with the type-1 spreading's global atomics (350 antennas, 886,000 sources, four products: 0.52 ms a
+    // slice by the lattice, 0.20 by type-3) and are kept although small lattices take direct sums now, so that a plan
+    // keeps its route.  With today's kernels (16 channels, microseconds a slice, lattice / type-3): 331 antennas flat, four
+    // products, 20,000 sources 22 / 53, 200,000 87 / 68, 900,000 358 / 108; one product 15 / 21, 53 / 29, 221 / 56; 5 cm
+    // heights, one product 31 / 138, 117 / 154, 486 / 199: the sums win for small skies and height terms, type-3 for
+    // large flat ones.
     if (p->transform_req == FV_TRANSFORM_AUTO && p->n_pol == 4 &&
         6.0 * (double)p->n_src * K >= (double)p->n_src + (double)t3)
         return FV_OK;
