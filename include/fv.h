@@ -161,14 +161,15 @@ typedef enum {
  *   exp(-i a u_s') = exp(-i a/2) sum_q eps_q (-i)^q J_q(a/2) T_q(u)
  * (eps_0 = 1, else 2), truncated at the K terms whose tail bound
  * 2 sum_{q>=K} (|a|/4)^q / q! is below eps / 10, so a slice is K type-1
- * transforms with strengths c_s T_q(u_s) combined per baseline.  Each runs
- * on a periodic grid of about 2 sigma (2 max|n_d| + 1) points per axis with no
- * interpolation step.  FV_TRANSFORM_AUTO takes this route when the array is a
- * lattice, K <= 24 and K times its grid is no larger than the type-3 grid of
- * the top channel (t3 cells), and, for four products, 6 n_src K < n_src + t3
- * (the lattice spreading adds every product with global atomics into one small
- * grid, which contends for many sources); FV_TRANSFORM_TYPE3 never takes it;
- * FV_TRANSFORM_LATTICE
+ * transforms with strengths c_s T_q(u_s) combined per baseline.  Lattices of
+ * at most 1,600 modes (fewer for skies of more than 50,000 sources at loose
+ * tolerances, where the grid is faster) are summed mode by mode; else each
+ * transform runs on a periodic grid of about 2 sigma (2 max|n_d| + 1) points
+ * per axis with no interpolation step.  FV_TRANSFORM_AUTO takes this route when
+ * the array is a lattice, K <= 24 and K times its grid is no larger than the
+ * type-3 grid of the top channel (t3 cells), and, for four products,
+ * 6 n_src K < n_src + t3 (many polarised sources are faster by the type-3
+ * route); FV_TRANSFORM_TYPE3 never takes it; FV_TRANSFORM_LATTICE
  * always does, and fv_set_array fails with FV_ERR_UNSUPPORTED if the array is
  * not a lattice or needs more than 24 terms.
  *
