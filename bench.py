@@ -877,8 +877,8 @@ def run_sim(args, rank, world, local, dist):
         lat_route, li = route_leg("lattice_route", transform="lattice")
         lat_route.update({"lattice_terms": li["lattice_terms"], "lattice_modes": li["lattice_modes"],
                           "lattice_grid": li["lattice_grid"],
-                          "what": "same workload, plan with transform=lattice (type-1 transforms on the "
-                                  "horizontal lattice, heights by Chebyshev terms)"})
+                          "what": "same workload, plan with transform=lattice (mode sums of the horizontal "
+                                  "lattice, directly or by type-1 transforms, heights by Chebyshev terms)"})
 
     # ---- the up axis of a non-coplanar array on the type-3 route: Chebyshev height terms on a 2-D grid
     # against the third grid dimension (Section 2.2.2), same workload, both timed like the headline
