@@ -585,7 +585,7 @@ static fv_status choose_heights(fv_plan_s *p)
 // pairs' rounding adds up to in long sums: against the FP64 path the error was 1.00 to 1.03 times at 850 and 2,200 terms a
 // cell, 0.95 to 1.11 at 2,900 and 1.23 to 1.66 at 14,000, and the time 0.2 to 0.4 times (300,000 sources, 37 antennas:
 // 0.79 against 2.91 ms; 7 antennas, 2,900 terms: 3.4 against 10.1).  Kernels of 12 points and fewer (1.5e-11) were
-// within 1.02 times at 14,000 terms.
+// within 1.03 times at 14,000 terms.
 constexpr double kPairTermsMax = 1000.0;
 
 // FP64 slices in pairs of floats (fv_pairs.cu): sigma = 2, gather spreading (AUTO or asked for), products and planes
